@@ -856,51 +856,117 @@ __device__ __forceinline__ void node_ijk_i32(const LevelDims& d, int n, int& i, 
   i = r - j * d.nnx;
 }
 
-// Full-weighting restriction b_c = P^T r over the fine nodes of the mask.
+// Interpolation between a level and its coarsening, computed instead of read
+// from the tables of struct Axis (same rule and weights; the weights 1/2 and
+// 1 are exact, so the sums round identically): a table entry is a dependent
+// load in front of every transferred value, and the transfers are bound by
+// that latency.  Coarse node I of a coarsened axis sits on fine node 2 I;
+// with an odd element count the last fine node keeps its own coarse node.
+struct Axis1 {
+  int nf, nc, c;   // fine nodes, coarse nodes, coarsened
+};
+struct Xfer1 {
+  Axis1 a[3];
+};
+
+// Entry t of the support of coarse node I: fine node (-1: none) and weight.
+template <typename T>
+__device__ __forceinline__ int sup_of(const Axis1& a, int I, int t, T& w) {
+  w = (T)1;
+  if (!a.c) return t == 0 ? I : -1;
+  const int f = 2 * I - 1 + t;
+  if (f < 0 || f >= a.nf) return -1;
+  if (f == a.nf - 1 && !(a.nf & 1)) return I == a.nc - 1 ? f : -1;   // the last fine node of an odd element count
+  if (t != 1) w = (T)0.5;
+  return f;
+}
+
+// Parent q (0, 1) of fine node i: coarse node (-1: none) and weight.
+template <typename T>
+__device__ __forceinline__ int par_of(const Axis1& a, int i, int q, T& w) {
+  w = (T)1;
+  if (!a.c) return q == 0 ? i : -1;
+  if (i == a.nf - 1 && !(a.nf & 1)) return q == 0 ? a.nc - 1 : -1;
+  if (!(i & 1)) return q == 0 ? i >> 1 : -1;
+  w = (T)0.5;
+  return (i >> 1) + q;
+}
+
+// Full-weighting restriction (P^T r)_C over the fine nodes of the mask.
 // The phi_e / c_e masks are all ones (no mask load); elsewhere a masked-out
 // residual is selected away (never multiplied: it may hold stale values).
 template <typename T>
-__global__ void k_restrict(LevelDims fd, LevelDims cd, Xfer X, Ptr4<const T> fr, Ptr4<const uint8_t> fm, Ptr4<T> cb,
+__device__ __forceinline__ T restrict_row(const LevelDims& fd, const LevelDims& cd, const Xfer1& X, const T* r,
+                                          const uint8_t* __restrict__ m, bool all_on, int C) {
+  int I, J, K;
+  node_ijk_i32(cd, C, I, J, K);
+  T acc = 0;
+#pragma unroll
+  for (int tz = 0; tz < 3; ++tz) {
+    T wz;
+    const int fk = sup_of<T>(X.a[2], K, tz, wz);
+    if (fk < 0) continue;
+#pragma unroll
+    for (int ty = 0; ty < 3; ++ty) {
+      T wy;
+      const int fj = sup_of<T>(X.a[1], J, ty, wy);
+      if (fj < 0) continue;
+#pragma unroll
+      for (int tx = 0; tx < 3; ++tx) {
+        T wx;
+        const int fi = sup_of<T>(X.a[0], I, tx, wx);
+        if (fi < 0) continue;
+        const int f = fi + fd.nnx * (fj + fd.nny * fk);
+        const T v = r[f];
+        const bool on = all_on || m[f];
+        acc += on ? wx * wy * wz * v : (T)0;
+      }
+    }
+  }
+  return acc;
+}
+
+template <typename T>
+__global__ void k_restrict(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> fr, Ptr4<const uint8_t> fm, Ptr4<T> cb,
                            HList hl, BRange br) {
   const int h = pk(hl.h, blockIdx.y);
   if ((int)blockIdx.x >= pk(br.cnt, h)) return;   // coarse blocks without rows of the coarse mask
   const int C = (pk(br.lo, h) + (int)blockIdx.x) * blockDim.x + threadIdx.x;
   if (C >= (int)cd.n) return;
-  int I, J, K;
-  node_ijk_i32(cd, C, I, J, K);
   const T* __restrict__ r = pk(fr.p, h);
-  const uint8_t* __restrict__ m = pk(fm.p, h);
-  const bool all_on = h >= 2;
-  const T* swx = supw_t<T>(X.a[0]);
-  const T* swy = supw_t<T>(X.a[1]);
-  const T* swz = supw_t<T>(X.a[2]);
+  pk(cb.p, h)[C] = restrict_row<T>(fd, cd, X, r, pk(fm.p, h), h >= 2, C);
+}
+
+// (P x_c)_f: trilinear interpolation of the coarse correction at fine node f.
+template <typename T>
+__device__ __forceinline__ T prolong_row(const LevelDims& fd, const LevelDims& cd, const Xfer1& X, const T* cx, int f) {
+  int i, j, k;
+  node_ijk_i32(fd, f, i, j, k);
   T acc = 0;
 #pragma unroll
-  for (int tz = 0; tz < 3; ++tz) {
-    const int fk = X.a[2].sup[K * 3 + tz];
-    if (fk < 0) continue;
-    const T wz = swz[K * 3 + tz];
+  for (int c3 = 0; c3 < 2; ++c3) {
+    T wz;
+    const int pz = par_of<T>(X.a[2], k, c3, wz);
+    if (pz < 0) continue;
 #pragma unroll
-    for (int ty = 0; ty < 3; ++ty) {
-      const int fj = X.a[1].sup[J * 3 + ty];
-      if (fj < 0) continue;
-      const T wy = swy[J * 3 + ty];
+    for (int c2 = 0; c2 < 2; ++c2) {
+      T wy;
+      const int py = par_of<T>(X.a[1], j, c2, wy);
+      if (py < 0) continue;
 #pragma unroll
-      for (int tx = 0; tx < 3; ++tx) {
-        const int fi = X.a[0].sup[I * 3 + tx];
-        if (fi < 0) continue;
-        const int f = fi + fd.nnx * (fj + fd.nny * fk);
-        const T v = r[f];
-        const bool on = all_on || m[f];
-        acc += on ? swx[I * 3 + tx] * wy * wz * v : (T)0;
+      for (int c1 = 0; c1 < 2; ++c1) {
+        T wx;
+        const int px = par_of<T>(X.a[0], i, c1, wx);
+        if (px < 0) continue;
+        acc += wx * wy * wz * cx[px + cd.nnx * (py + cd.nny * pz)];
       }
     }
   }
-  pk(cb.p, h)[C] = acc;
+  return acc;
 }
 
 template <typename T>
-__global__ void k_prolong(LevelDims fd, LevelDims cd, Xfer X, Ptr4<const T> cx_, Ptr4<const uint8_t> fm, Ptr4<T> fx,
+__global__ void k_prolong(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> cx_, Ptr4<const uint8_t> fm, Ptr4<T> fx,
                           HList hl, BRange br) {
   const int h = pk(hl.h, blockIdx.y);
   if ((int)blockIdx.x >= pk(br.cnt, h)) return;   // fine blocks without rows of the mask
@@ -910,37 +976,21 @@ __global__ void k_prolong(LevelDims fd, LevelDims cd, Xfer X, Ptr4<const T> cx_,
   // (phi_e / c_e masks are all ones)
   const bool on = h >= 2 || pk(fm.p, h)[f];
   const T xf = pk(fx.p, h)[f];
-  int i, j, k;
-  node_ijk_i32(fd, f, i, j, k);
   const T* __restrict__ cx = pk(cx_.p, h);
-  const T* pwx = parw_t<T>(X.a[0]);
-  const T* pwy = parw_t<T>(X.a[1]);
-  const T* pwz = parw_t<T>(X.a[2]);
-  T acc = 0;
-#pragma unroll
-  for (int c3 = 0; c3 < 2; ++c3) {
-    const int pz = X.a[2].par[k * 2 + c3];
-    if (pz < 0) continue;
-    const T wz = pwz[k * 2 + c3];
-#pragma unroll
-    for (int c2 = 0; c2 < 2; ++c2) {
-      const int py = X.a[1].par[j * 2 + c2];
-      if (py < 0) continue;
-      const T wy = pwy[j * 2 + c2];
-#pragma unroll
-      for (int c1 = 0; c1 < 2; ++c1) {
-        const int px = X.a[0].par[i * 2 + c1];
-        if (px < 0) continue;
-        acc += pwx[i * 2 + c1] * wy * wz * cx[px + cd.nnx * (py + cd.nny * pz)];
-      }
-    }
-  }
+  const T acc = prolong_row<T>(fd, cd, X, cx, f);
   if (on) pk(fx.p, h)[f] = xf + acc;
 }
 
 // x = A^-1 b at the coarsest level (dense FP64 inverse): one warp per row,
 // lanes over the columns, a fixed-order warp reduction.
 constexpr int kCoarseWarps = 8;
+template <typename T>
+__device__ __forceinline__ double coarse_row(int n, const double* __restrict__ A, const T* b, int lane) {
+  double acc = 0.0;
+  for (int cidx = lane; cidx < n; cidx += 32) acc += A[cidx] * (double)b[cidx];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
 template <typename T>
 __global__ void __launch_bounds__(32 * kCoarseWarps) k_coarse_solve(int n, const double* __restrict__ inv,
                                                                     Ptr4<const T> b, Ptr4<const uint8_t> mask,
@@ -949,12 +999,356 @@ __global__ void __launch_bounds__(32 * kCoarseWarps) k_coarse_solve(int n, const
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * kCoarseWarps + (threadIdx.x >> 5);
   if (r >= n) return;   // per warp
-  const double* A = inv + (size_t)h * n * n + (size_t)r * n;
-  const T* bb = pk(b.p, h);
-  double acc = 0.0;
-  for (int cidx = lane; cidx < n; cidx += 32) acc += A[cidx] * (double)bb[cidx];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  const double acc = coarse_row<T>(n, inv + (size_t)h * n * n + (size_t)r * n, pk(b.p, h), lane);
   if (lane == 0 && pk(mask.p, h)[r]) pk(x.p, h)[r] = (T)acc;   // masked-out rows are never read (and may be shared)
+}
+
+// ---------------------------------------------------------------- coarse tail
+// The V-cycle from level l0 down to the coarsest level and back up to l0 in
+// one launch, one thread-block cluster per hierarchy.  Launched level by
+// level, the small levels are bound by latency: 7 dependent launches per
+// level, each waiting on several rounds of L2 loads.  Here every vector of
+// the tail lives in shared memory: rows are owned by thread (at most one per
+// thread and level; contiguous chunks of rows per block), a thread keeps its
+// row's 27 coefficients, b, 1/diag, d and x in registers over the level's
+// steps and stores x into the shared memory of every block that owns a
+// neighbour row (the residual: of the blocks that own a parent row; the
+// final x: a child row), with one cluster barrier per step.  A level of at
+// most kTailThreads rows runs on the first block alone (block barriers); the
+// coarsest dense solve, FP64 and bound by the FP64 rate of an SM, is spread
+// over the cluster.  Only the x of level l0 goes back to global memory.  Per
+// row the arithmetic and its order are those of k_cheb, k_resid, k_restrict,
+// k_prolong and k_coarse_solve.
+constexpr int kTailThreads = 512;
+constexpr int kTailMaxCluster = 16;
+// Rows per block before a level takes another block of the cluster: one per
+// thread in FP32; in FP64 the stencil is bound by the FP64 rate of the SM
+// (27 clocks per row and step).
+template <typename T>
+constexpr int kTailRows = kTailThreads;
+template <>
+constexpr int kTailRows<double> = 128;
+constexpr size_t kTailMaxSmem = 216 * 1024;   // dynamic; the static part is under 8 KB
+
+struct TailLevel {
+  LevelDims d;
+  Xfer1 X;                     // towards the next level
+  int oA, oB, ob;              // shared offsets (elements): x buffers (at node 0, inside their guards), own b
+  int lo[kNH], hi[kNH];        // row range of each hierarchy's mask
+  const void* st[kNH];
+  const void* dinv[kNH];
+  const uint8_t* mask[kNH];
+};
+
+struct TailArgs {
+  int nl;                      // levels of the tail
+  int l0;                      // multigrid level of lev[0] (Chebyshev table row)
+  int deg, cs;                 // Chebyshev degree, blocks per cluster
+  int len;                     // shared elements
+  int h[kNH];                  // hierarchy of each cluster
+  const void* ctab;
+  const double* inv;           // coarsest inverses [kNH][n][n]
+  const void* b[kNH];          // right-hand side and result of lev[0]
+  void* x[kNH];
+  TailLevel lev[kMaxLevels];
+};
+
+// A level as its cluster uses it (copied to shared memory once: the kernel
+// parameters of a level are cold in the constant cache at its first use).
+struct TailLv {
+  const void* st;
+  const void* dinv;
+  const uint8_t* mask;
+  LevelDims d;
+  Xfer1 X;
+  int lo, rows, chunk, nr;     // first row, rows, rows per block, blocks that own rows
+  int oA, oB, ob;
+  float rch, rsx, rsxy;        // 1 / chunk, 1 / nnx, 1 / (nnx nny)
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+  // not .aligned: the rows' branches may leave a warp's lanes unconverged
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+
+// a / b for 0 <= a < 2^14 and 1 <= b < 2^14, rb = 1.0f / b: a + 1/2 is at
+// least 1/(2 b) of the quotient away from an integer, far above the rounding
+// of the FP32 product (an integer division is a chain of ~100 clocks).
+__device__ __forceinline__ int small_div(int a, float rb) { return (int)(((float)a + 0.5f) * rb); }
+
+// Block that owns row n of level L (n clamped to the level's rows).
+__device__ __forceinline__ int tail_owner(const TailLv& L, int n) {
+  if (L.nr == 1) return 0;
+  const int i = n - L.lo;
+  return small_div(i < 0 ? 0 : (i >= L.rows ? L.rows - 1 : i), L.rch);
+}
+
+__device__ __forceinline__ void tail_ijk(const TailLv& L, int n, int (&id)[3]) {
+  id[2] = small_div(n, L.rsxy);
+  const int r = n - id[2] * (L.d.nnx * L.d.nny);
+  id[1] = small_div(r, L.rsx);
+  id[0] = r - id[1] * L.d.nnx;
+}
+
+// restrict_row and prolong_row with the axes' entries formed once and absent
+// entries as weight 0 on an index inside the level (acc + 0 r = acc): 27 and
+// 8 independent loads.
+template <typename T>
+__device__ __forceinline__ T tail_restrict(const TailLv& F, const TailLv& C, const T* r, int c) {
+  int id[3];
+  tail_ijk(C, c, id);
+  int f[3][3];
+  T w[3][3];
+  const int str[3] = {1, F.d.nnx, F.d.nnx * F.d.nny};
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    const Axis1 A = F.X.a[ax];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const int s = sup_of<T>(A, id[ax], t, w[ax][t]);
+      if (s < 0) w[ax][t] = (T)0;
+      f[ax][t] = (s < 0 ? 0 : s) * str[ax];
+    }
+  }
+  T acc = 0;
+#pragma unroll
+  for (int tz = 0; tz < 3; ++tz)
+#pragma unroll
+    for (int ty = 0; ty < 3; ++ty) {
+      const T wyz = w[1][ty] * w[2][tz];
+      const int o = f[1][ty] + f[2][tz];
+#pragma unroll
+      for (int tx = 0; tx < 3; ++tx) acc += w[0][tx] * wyz * r[o + f[0][tx]];
+    }
+  return acc;
+}
+
+template <typename T>
+__device__ __forceinline__ T tail_prolong(const TailLv& F, const TailLv& C, const T* x, const int (&id)[3]) {
+  int p[3][2];
+  T w[3][2];
+  const int str[3] = {1, C.d.nnx, C.d.nnx * C.d.nny};
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    const Axis1 A = F.X.a[ax];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int s = par_of<T>(A, id[ax], t, w[ax][t]);
+      if (s < 0) w[ax][t] = (T)0;
+      p[ax][t] = (s < 0 ? 0 : s) * str[ax];
+    }
+  }
+  T acc = 0;
+#pragma unroll
+  for (int c3 = 0; c3 < 2; ++c3)
+#pragma unroll
+    for (int c2 = 0; c2 < 2; ++c2) {
+      const T wyz = w[1][c2] * w[2][c3];
+      const int o = p[1][c2] + p[2][c3];
+#pragma unroll
+      for (int c1 = 0; c1 < 2; ++c1) acc += w[0][c1] * wyz * x[o + p[0][c1]];
+    }
+  return acc;
+}
+
+// v into entry `off` of the shared memory of blocks r0 .. r1 of the cluster.
+template <typename T>
+__device__ __forceinline__ void tail_put(T* sm, int off, int r0, int r1, T v) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(sm + off);
+  for (int r = r0; r <= r1; ++r) {
+    unsigned ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(r));
+    if constexpr (sizeof(T) == 4)
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(ra), "f"(v) : "memory");
+    else
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+  }
+}
+
+// The 27 coefficients of row n, and (A x)_n in difference form summed in
+// offset order (as stencil_rows), x in shared memory.
+template <typename TS, typename T>
+__device__ __forceinline__ void row_coef(const void* st, int N, int n, T (&c)[27]) {
+  const TS* p = static_cast<const TS*>(st);
+#pragma unroll
+  for (int o = 0; o < 27; ++o) c[o] = (T)tof(__ldg(p + o * N + n));
+}
+template <typename T>
+__device__ __forceinline__ T row_apply(const T (&c)[27], const T* x, int sy, int sz, int n, T xn) {
+  T ax = c[13] * xn;
+#pragma unroll
+  for (int o = 0; o < 27; ++o)
+    if (o != 13) ax += c[o] * (x[n + (o % 3 - 1) + ((o / 3) % 3 - 1) * sy + (o / 9 - 1) * sz] - xn);
+  return ax;
+}
+
+// TS0: storage of lev[0] (multigrid level 0 keeps FP32 stencils under the
+// BF16 option), TS: of the levels below.  One loop visits the levels down
+// and up, so that every piece of code appears once: instruction fetch of
+// code that a launch executes once costs more than its arithmetic.  Measured
+// (clocks of one launch at 2,025 rows, 3 levels, 4 blocks per cluster): 40 k
+// = 20 us, of which a step (27 shared loads, 8 k clocks in all) plus its
+// barrier (0.2 k in one block, 0.9-1.9 k in a cluster of 4-16) take half,
+// the first loads of each level most of the rest; with the vectors in global
+// memory and global loads of the transfer tables 33 us, launched level by
+// level (17 launches) 70 us.  FP64 is bound by the FP64 rate of the SMs.
+template <typename TS0, typename TS, typename T>
+__global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant__ TailArgs a) {
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  __shared__ TailLv lv[kMaxLevels];
+  __shared__ T ch[kMaxLevels * kMaxDeg * 3];
+  T* sm = reinterpret_cast<T*>(tail_smem);
+  const int h = a.h[blockIdx.x / a.cs];
+  const int rank = blockIdx.x % a.cs;
+  const int tid = threadIdx.x;
+  const bool all_on = h >= 2;
+  for (int i = tid; i < a.len; i += kTailThreads) sm[i] = (T)0;
+  if (tid < a.nl) {
+    const TailLevel& L = a.lev[tid];
+    TailLv v;
+    v.st = L.st[h];
+    v.dinv = L.dinv[h];
+    v.mask = L.mask[h];
+    v.d = L.d;
+    v.X = L.X;
+    v.lo = L.lo[h];
+    v.rows = L.hi[h] - L.lo[h];
+    v.nr = max(1, min(a.cs, (v.rows + kTailRows<T> - 1) / kTailRows<T>));
+    v.chunk = (v.rows + v.nr - 1) / v.nr;
+    v.oA = L.oA;
+    v.oB = L.oB;
+    v.ob = L.ob;
+    v.rch = 1.0f / (float)max(1, v.chunk);
+    v.rsx = 1.0f / (float)v.d.nnx;
+    v.rsxy = 1.0f / (float)(v.d.nnx * v.d.nny);
+    lv[tid] = v;
+  }
+  const T* __restrict__ ctab = static_cast<const T*>(a.ctab);
+  for (int i = tid; i < a.nl * a.deg * 3; i += kTailThreads)
+    ch[i] = cheb_at(ctab, a.l0 + i / (3 * a.deg), i / 3 % a.deg, i % 3, h);
+  __syncthreads();
+  if (a.cs > 1) cluster_barrier();   // no store into a block that has not started and cleared its vectors
+  const int nd = a.nl - 1;           // smoothed levels
+#pragma unroll 1
+  for (int v = 0; v < 2 * nd; ++v) {
+    const bool up = v >= nd;
+    const int q = up ? 2 * nd - 1 - v : v;
+    const TailLv& L = lv[q];
+    const TailLv& B = lv[q + 1];
+    if (v == nd) {
+      // the coarsest level's dense solve, rows over the warps of the cluster
+      const int n = (int)B.d.n, lane = tid & 31;
+      const double* inv = a.inv + (size_t)h * n * n;
+      if (a.cs > 1) cluster_barrier();
+      else __syncthreads();
+#pragma unroll 1
+      for (int r = rank * (kTailThreads / 32) + (tid >> 5); r < n; r += a.cs * (kTailThreads / 32)) {
+        const bool on = all_on || __ldg(B.mask + r);
+        const double acc = coarse_row<T>(n, inv + (size_t)r * n, sm + B.ob, lane);
+        if (lane < L.nr && on) tail_put(sm, B.oA + r, lane, lane, (T)acc);
+      }
+      if (a.cs > 1) cluster_barrier();
+      else __syncthreads();
+    }
+    const bool multi = L.nr > 1;
+    if (!multi && rank > 0) continue;
+    const int sy = L.d.nnx, sz = L.d.nnx * L.d.nny;
+    const int n = L.lo + rank * L.chunk + tid;
+    const bool in = tid < L.chunk && n < L.lo + L.rows;
+    const bool on = in && (all_on || __ldg(L.mask + n));
+    // x is in the first buffer after an even number of steps
+    int x = (up && (a.deg & 1)) ? L.oB : L.oA, xo = (up && (a.deg & 1)) ? L.oA : L.oB;
+    T c[27];
+    T bq = (T)0, iq = (T)0, dq = (T)0, xq = (T)0;
+    int id[3] = {0, 0, 0};
+    int r0 = 0, r1 = 0, g0 = 0, g1 = 0;   // blocks of the neighbour rows; of the parent (down) or child (up) rows
+    if (in) {   // on the way up these loads are in flight over the barrier
+      if (!std::is_same<TS0, TS>::value && q == 0) row_coef<TS0, T>(L.st, (int)L.d.n, n, c);
+      else row_coef<TS, T>(L.st, (int)L.d.n, n, c);
+      bq = q == 0 ? static_cast<const T*>(a.b[h])[n] : sm[L.ob + tid];
+      iq = __ldg(static_cast<const T*>(L.dinv) + n);
+      if (up) xq = sm[x + n];
+      r0 = tail_owner(L, n - sz - sy - 1);
+      r1 = tail_owner(L, n + sz + sy + 1);
+      tail_ijk(L, n, id);
+      const TailLv& U = lv[up && q > 0 ? q - 1 : q];   // the finer level of the transfer
+      const TailLv& G = up ? U : B;                    // the level whose owners get the last vector
+      if (G.nr > 1) {
+        int c0 = 0, c1 = 0, st = 1;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          const Axis1 A = U.X.a[ax];
+          T w;
+          int e0, e1;
+          if (up) {
+            const int s0 = sup_of<T>(A, id[ax], 0, w), s1 = sup_of<T>(A, id[ax], 1, w), s2 = sup_of<T>(A, id[ax], 2, w);
+            e0 = s0 >= 0 ? s0 : s1;
+            e1 = s2 >= 0 ? s2 : (s1 >= 0 ? s1 : s0);
+          } else {
+            e0 = par_of<T>(A, id[ax], 0, w);
+            e1 = par_of<T>(A, id[ax], 1, w);
+            if (e1 < 0) e1 = e0;
+          }
+          c0 += st * e0;
+          c1 += st * e1;
+          st *= up ? A.nf : A.nc;
+        }
+        g0 = tail_owner(G, c0);
+        g1 = tail_owner(G, c1);
+      }
+    }
+    if (up) {
+      if (v > nd) {   // (the coarsest solve ended with a barrier)
+        if (multi) cluster_barrier();
+        else __syncthreads();
+      }
+      if (in) {
+        xq += tail_prolong<T>(L, B, sm + B.oA, id);
+        if (on) tail_put(sm, x + n, r0, r1, xq);
+      }
+      if (multi) cluster_barrier();
+      else __syncthreads();
+    }
+    // down: deg steps from x = 0, then the residual (s == deg); up: deg steps
+    const int ns = up ? a.deg : a.deg + 1;
+#pragma unroll 1
+    for (int s = 0; s < ns; ++s) {
+      if (in) {
+        T res = bq;
+        if (up || s > 0) res -= row_apply<T>(c, sm + x, sy, sz, n, xq);
+        T val = res;
+        if (s < a.deg) {
+          const T z = iq * res;
+          const T* cf = ch + (q * a.deg + s) * 3;
+          dq = s == 0 ? cf[0] * z : cf[1] * dq + cf[2] * z;
+          xq += dq;
+          val = xq;
+        }
+        if (on) {
+          const bool last = s == ns - 1;   // the residual, to the parents' blocks; the final x, to the children's
+          if (last && up && q == 0) static_cast<T*>(a.x[h])[n] = val;
+          else tail_put(sm, xo + n, last ? g0 : r0, last ? g1 : r1, val);
+        }
+      }
+      if (s < a.deg) {
+        const int t = x;
+        x = xo;
+        xo = t;
+      }
+      if (up && s == ns - 1) break;   // the level above starts with the barrier
+      if (multi) cluster_barrier();
+      else __syncthreads();
+    }
+    if (!up && rank < B.nr) {
+      const int C = B.lo + rank * B.chunk + tid;
+      if (tid < B.chunk && C < B.lo + B.rows) {
+        // rows outside the mask hold exact zeros in the shared vectors
+        const T val = tail_restrict<T>(L, B, sm + xo, C);
+        if (q + 1 < nd) sm[B.ob + tid] = val;
+        else tail_put(sm, B.ob + C, 0, a.cs - 1, val);   // every block solves rows of the coarsest level
+      }
+    }
+  }
 }
 
 size_t tsize(int precision, int level) {
@@ -968,6 +1362,10 @@ HList make_hl(const int* hs, int nhs) {
   HList l{};
   for (int i = 0; i < kNH; ++i) l.h[i] = i < nhs ? hs[i] : hs[0];
   return l;
+}
+
+Xfer1 xfer1(const MGLevel& A, const MGLevel& B) {
+  return Xfer1{{{A.nnx, B.nnx, A.cx}, {A.nny, B.nny, A.cy}, {A.nnz, B.nnz, A.cz}}};
 }
 
 LevelDims dims(const MGLevel& L) { return LevelDims{L.nnx, L.nny, L.nnz, L.n}; }
@@ -1055,12 +1453,94 @@ p4d_status level0_stencil_step(p4d_ctx* c, MGLevel& A, const int* hs, int nhs, c
   return P4D_OK;
 }
 
+// Shared-memory layout of the tail from level l0 (elements; offsets into
+// `lev` when given): per level two x buffers with guards and the block's own
+// b, at the coarsest b and x.
+int tail_layout(const p4d_ctx* c, int l0, TailLevel* lev) {
+  int o = 0;
+  for (int l = l0; l < c->nlev; ++l) {
+    const MGLevel& A = c->lev[l];
+    const int n = (int)A.n, G = A.nnx * A.nny + A.nnx + 1;
+    const bool last = l == c->nlev - 1;
+    int oA, oB, ob;
+    if (last) {
+      oA = o;
+      oB = o;
+      ob = o + n;
+      o += 2 * n;
+    } else {
+      oA = o + G;
+      oB = o + n + 3 * G;
+      ob = o + 2 * n + 4 * G;
+      o += 2 * n + 4 * G + kTailThreads;
+    }
+    if (lev) {
+      lev[l - l0].oA = oA;
+      lev[l - l0].oB = oB;
+      lev[l - l0].ob = ob;
+    }
+  }
+  return o;
+}
+
+cudaLaunchConfig_t tail_config(int cs, int nhs, size_t smem, cudaStream_t stream, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(cs * nhs));
+  cfg.blockDim = dim3(kTailThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// The levels l0 .. L - 1 in one launch (see k_tail).
+template <typename TS0, typename TS, typename T>
+p4d_status tail_launch(p4d_ctx* c, const int* hs, int nhs, int l0) {
+  const int L = c->nlev;
+  TailArgs a;
+  a.nl = L - l0;
+  a.l0 = l0;
+  a.deg = c->prm.cheb_degree;
+  a.cs = c->tail_cs;
+  a.ctab = cheb_tab<T>(c);
+  a.inv = c->lev[L - 1].inv;
+  a.len = tail_layout(c, l0, a.lev);
+  for (int t = 0; t < kNH; ++t) a.h[t] = t < nhs ? hs[t] : hs[0];
+  for (int h = 0; h < kNH; ++h) {
+    a.b[h] = c->lev[l0].b[h];
+    a.x[h] = c->lev[l0].x[h];
+  }
+  for (int q = 0; q < a.nl; ++q) {
+    const MGLevel& A = c->lev[l0 + q];
+    TailLevel& B = a.lev[q];
+    B.d = dims(A);
+    if (q + 1 < a.nl) B.X = xfer1(A, c->lev[l0 + q + 1]);
+    for (int h = 0; h < kNH; ++h) {
+      B.lo[h] = A.blo[h] * kBlock;
+      B.hi[h] = (int)std::min<int64_t>(A.n, (int64_t)(A.blo[h] + A.bcnt[h]) * kBlock);
+      B.st[h] = A.st[h];
+      B.dinv[h] = A.dinv[h];
+      B.mask[h] = A.mask[h];
+    }
+  }
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = tail_config(a.cs, nhs, sizeof(T) * a.len, c->stream, at);
+  ::p4d::count_launch();
+  P4D_TRY(cudaLaunchKernelEx(&cfg, l0 == 0 ? k_tail<TS0, TS, T> : k_tail<TS, TS, T>, a));
+  return P4D_OK;
+}
+
 template <typename TS0, typename TS, typename T>
 p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
-  const int L = c->nlev;
+  const int LT = c->tail_l0 >= 0 ? c->tail_l0 : c->nlev - 1;   // levels above: one launch per operation
   const int deg = c->prm.cheb_degree;
   HList hl = make_hl<T>(hs, nhs);
-  for (int l = 0; l < L - 1; ++l) {
+  for (int l = 0; l < LT; ++l) {
     MGLevel& A = c->lev[l];
     MGLevel& B = c->lev[l + 1];
     unsigned gx = 1;
@@ -1082,17 +1562,19 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
     for (int h = 0; h < kNH; ++h) { fr.p[h] = (const T*)A.r[h]; fm.p[h] = A.mask[h]; cb.p[h] = (T*)B.b[h]; }
     unsigned gxc = 1;
     const BRange brc = brange(B, hs, nhs, &gxc);
-    ::p4d::count_launch(), k_restrict<T><<<dim3(gxc, nhs), kBlock, 0, c->stream>>>(dims(A), dims(B), A.X, fr, fm, cb, hl, brc);
+    ::p4d::count_launch(), k_restrict<T><<<dim3(gxc, nhs), kBlock, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fr, fm, cb, hl, brc);
   }
-  {
-    MGLevel& C = c->lev[L - 1];
+  if (c->tail_l0 >= 0) {
+    P4D_TRYS((tail_launch<TS0, TS, T>(c, hs, nhs, LT)));
+  } else {
+    MGLevel& C = c->lev[LT];
     Ptr4<const T> b;
     Ptr4<const uint8_t> m;
     Ptr4<T> x;
     for (int h = 0; h < kNH; ++h) { b.p[h] = (const T*)C.b[h]; m.p[h] = C.mask[h]; x.p[h] = (T*)C.x[h]; }
     ::p4d::count_launch(), k_coarse_solve<T><<<dim3((unsigned)((C.n + kCoarseWarps - 1) / kCoarseWarps), nhs), 32 * kCoarseWarps, 0, c->stream>>>((int)C.n, C.inv, b, m, x, hl);
   }
-  for (int l = L - 2; l >= 0; --l) {
+  for (int l = LT - 1; l >= 0; --l) {
     MGLevel& A = c->lev[l];
     MGLevel& B = c->lev[l + 1];
     Ptr4<const T> cxp;
@@ -1102,7 +1584,7 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
     unsigned gx = 1;
     const BRange br = brange(A, hs, nhs, &gx);
     const dim3 grid(gx, nhs);
-    ::p4d::count_launch(), k_prolong<T><<<grid, kBlock, 0, c->stream>>>(dims(A), dims(B), A.X, cxp, fm, fx, hl, br);
+    ::p4d::count_launch(), k_prolong<T><<<grid, kBlock, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), cxp, fm, fx, hl, br);
     for (int s = 0; s < deg; ++s) {
       if (l == 0) prof_mark(c, 3);
       if (l == 0) P4D_TRYS((level0_stencil_step<TS0, T>(c, A, hs, nhs, hl, br, grid, 0, s)));
@@ -1128,6 +1610,47 @@ p4d_status alloc_x(p4d_ctx* c, void** p, size_t ts, const MGLevel& lv) {
   P4D_TRYS(dalloc(c, &base, bytes));
   P4D_TRY(cudaMemset(base, 0, bytes));
   *p = static_cast<char*>(base) + ts * G;
+  return P4D_OK;
+}
+
+// First level of the single-launch tail and its cluster size (-1: no tail).
+// The finest level is taken that has at most one row per thread of the
+// largest cluster (FP64: two blocks' worth of rows per block, see kTailRows)
+// and whose shared vectors fit: one more level in the tail replaces seven
+// launches.  Measured per FGMRES solve (level by level / tail from 2,000
+// rows / from this rule's level): 9 x 9 x 25 nodes 2.35 / - / 1.74 ms,
+// 65 x 65 x 49 5.46 / 5.00 / 4.80 ms, FP64 41 x 37 x 37 8.28 / 7.97 / 7.57
+// ms, 129 x 129 x 97 18.5 / 18.0 / 17.7 ms.
+p4d_status tail_plan(p4d_ctx* c) {
+  c->tail_l0 = -1;
+  const int L = c->nlev;
+  const bool fp64 = c->prm.precision == 0;
+  const size_t tv = fp64 ? sizeof(double) : sizeof(float);
+  const int rpb = fp64 ? kTailRows<double> : kTailRows<float>;
+  const int64_t most = (int64_t)kTailMaxCluster * (fp64 ? 2 * rpb : rpb);
+  if (c->lev[L - 1].n > kTailThreads) return P4D_OK;
+  for (int l = 0; l < L - 1 && c->tail_l0 < 0; ++l)
+    if (c->lev[l].n <= most && tv * tail_layout(c, l, nullptr) <= kTailMaxSmem) c->tail_l0 = l;
+  if (c->tail_l0 < 0) return P4D_OK;
+  int cs = 1;
+  while (cs < kTailMaxCluster && (int64_t)cs * rpb < c->lev[c->tail_l0].n) cs *= 2;
+  c->tail_cs = cs;
+  const bool z = c->tail_l0 == 0;
+  const void* k = fp64 ? (const void*)k_tail<double, double, double>
+                  : c->prm.precision == 1 ? (const void*)k_tail<float, float, float>
+                  : z ? (const void*)k_tail<float, __nv_bfloat16, float>
+                      : (const void*)k_tail<__nv_bfloat16, __nv_bfloat16, float>;
+  // process-wide attributes shared by every handle: always the largest values
+  P4D_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  P4D_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailMaxSmem));
+  // a device (partition) that cannot hold such a cluster keeps the launches per level
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = tail_config(cs, 1, tv * tail_layout(c, c->tail_l0, nullptr), nullptr, at);
+  int fit = 0;
+  if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) != cudaSuccess || fit < 1) {
+    cudaGetLastError();
+    c->tail_l0 = -1;
+  }
   return P4D_OK;
 }
 
@@ -1206,6 +1729,7 @@ p4d_status mg_plan(p4d_ctx* c) {
   }
   c->nlev = L;
   if (c->lev[L - 1].n > 4096) return P4D_ERR_INVALID_ARG;   // coarsest level too large for a dense inverse
+  P4D_TRYS(tail_plan(c));
   for (int l = 0; l < L; ++l) {
     MGLevel& lv = c->lev[l];
     const int64_t n = lv.n;
@@ -1232,6 +1756,13 @@ p4d_status mg_plan(p4d_ctx* c) {
       for (int h = 0; h < kNH; ++h) {
         lv.st[h] = st[fh[h]]; lv.dinv[h] = di[fh[h]]; lv.x[h] = x[fh[h]]; lv.x2[h] = x2[fh[h]];
         lv.b[h] = b[fh[h]]; lv.r[h] = r[fh[h]]; lv.d[h] = d[fh[h]];
+      }
+      if (c->tail_l0 == 0) {
+        // the tail's clusters run the two phi_s hierarchies unsynchronized,
+        // and a row next to the other electrode loads its neighbour there
+        // (times an exact zero): iterates of their own
+        P4D_TRYS(alloc_x(c, &lv.x[1], tv, lv));
+        P4D_TRYS(alloc_x(c, &lv.x2[1], tv, lv));
       }
       ::p4d::count_launch(), k_mask0<<<nblocks(n), kBlock, 0, c->stream>>>(n, c->label, lv.mask[0], lv.mask[1], lv.mask[2], lv.mask[3]);
     } else {

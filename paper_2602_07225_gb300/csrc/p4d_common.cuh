@@ -203,6 +203,8 @@ struct p4d_ctx {
   p4d::MGLevel lev[p4d::kMaxLevels];
   double lam_h[p4d::kMaxLevels][p4d::kNH] = {};   // Gershgorin bounds (host copy, per Newton update)
   double* lam_pin = nullptr;           // pinned staging for lam
+  int tail_l0 = -1;                    // first level of the single-launch V-cycle tail (-1: none)
+  int tail_cs = 1;                     // its blocks per cluster
   void* yc = nullptr;                  // [NE][nc] particle solve work (compute precision)
 
   // concentration-dependent transport (transport.cu, transport_model 1)

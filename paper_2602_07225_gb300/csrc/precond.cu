@@ -197,9 +197,10 @@ __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref
   }
 }
 
+// x0c: phi_s of the cathode (x0, or the cathode hierarchy's own iterate).
 template <typename T>
 __global__ void k_store(Grid g, const uint8_t* __restrict__ label, int fmask, const T* __restrict__ x0,
-                        const T* __restrict__ x1, const T* __restrict__ x2, VRef zref_) {
+                        const T* __restrict__ x0c, const T* __restrict__ x1, const T* __restrict__ x2, VRef zref_) {
   double* __restrict__ zm = zref_.get();
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t nn = g.nn;
@@ -207,7 +208,11 @@ __global__ void k_store(Grid g, const uint8_t* __restrict__ label, int fmask, co
   const T* xs[3] = {x0, x1, x2};
   for (int f = 0; f < 3; ++f) {
     if (!(fmask & (1 << f))) continue;
-    if (f == 0 && !(label[n] & kLabActive)) continue;
+    if (f == 0) {
+      const uint8_t l = label[n];
+      if (l & kLabActive) zm[n] = (double)((l & kLabCathode) ? x0c : x0)[n];
+      continue;
+    }
     zm[f * nn + n] = (double)xs[f][n];
   }
 }
@@ -296,7 +301,7 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
     ::p4d::count_launch(), k_load<T, TRANS, FULL><<<nblocks(nn), kBlock, 0, c->stream>>>(a, r, yc, z, 7, 0, scaled, b[0], b[1], b[2]);
     const int hs[4] = {0, 1, 2, 3};
     P4D_TRYS(mg_vcycle(c, hs, 4));
-    ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 7, (const T*)l0.x[0], (const T*)l0.x[2],
+    ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 7, (const T*)l0.x[0], (const T*)l0.x[1], (const T*)l0.x[2],
                                                       (const T*)l0.x[3], z);
   } else {
     int done = 0;
@@ -309,7 +314,7 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
       for (int q = 0; q < 2; ++q)
         if (kHOfField[f][q] >= 0) hs[nh++] = kHOfField[f][q];
       P4D_TRYS(mg_vcycle(c, hs, nh));
-      ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 1 << f, (const T*)l0.x[0], (const T*)l0.x[2],
+      ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 1 << f, (const T*)l0.x[0], (const T*)l0.x[1], (const T*)l0.x[2],
                                                         (const T*)l0.x[3], z);
       done |= 1 << f;
     }
