@@ -7,9 +7,11 @@
 // first cancelled more than half of the vector ("twice is enough" with the
 // Daniel-Gragg-Kaufman-Stewart test, decided on the device).  Each pass is a
 // register-blocked multi-dot over the basis with a fixed-shape two-stage
-// reduction (deterministic order).  The Hessenberg
-// column, Givens rotations and residual estimate are updated on the device by
-// one thread; the host reads one scalar per iteration.
+// reduction (deterministic order).  The second stage, the reorthogonalisation
+// test, the Hessenberg column, the Givens rotations and the residual estimate
+// run in the last block of the kernel that produced their inputs (each is a
+// few microseconds of latency as a launch of its own): an Arnoldi step
+// without refinement is multi-dot, update and scaling, three launches.
 #include <cmath>
 #include <cstring>
 #include "p4d_common.cuh"
@@ -63,14 +65,45 @@ __device__ __forceinline__ void warp_transpose_reduce(double (&a)[P], int lane) 
   for (int o = 16 >> Log2<P>::v; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
 }
 
+// True in every thread of the block that finishes its kernel last, with the
+// other blocks' writes visible; it resets the counter for the next launch.
+__device__ __forceinline__ bool last_block(unsigned* cnt) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+    if (last) *cnt = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Sum of p[0..n) by one warp (fixed order: lanes stride, then a butterfly).
+__device__ __forceinline__ double warp_sum(const double* p, int n, int lane) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = lane; b < n; b += 32) s += __ldcg(p + b);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// out[g0 + i] = V_{g0+i} . w (i < NG), out[kp1] = w . w (WW), summed over the
+// blocks by the last one.  flag (optional): skipped when *flag == 0, out
+// then zeroed (zero_if_skipped) or left as it is.
 template <int NG, bool WW>
 __global__ void __launch_bounds__(kRedThreads) k_mdot(const double* __restrict__ V, int64_t ldv, int g0, int kp1,
                                                       const double* __restrict__ w, int64_t len,
-                                                      double* __restrict__ partial, int pstride,
-                                                      const double* __restrict__ flag) {
-  if (flag && *flag == 0.0) return;   // conditional pass not needed
+                                                      double* __restrict__ partial, double* __restrict__ out,
+                                                      unsigned* cnt, const double* __restrict__ flag,
+                                                      int zero_if_skipped) {
   constexpr int NA = NG + (WW ? 1 : 0);
   constexpr int P = Pow2Up<NA>::v;
+  if (flag && *flag == 0.0) {   // conditional pass not needed
+    if (zero_if_skipped && blockIdx.x == 0 && threadIdx.x < NG) out[g0 + threadIdx.x] = 0.0;
+    return;
+  }
   __shared__ double red[kRedThreads / 32][P];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -114,148 +147,14 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot(const double* __restrict__
     double sum = 0.0;
 #pragma unroll
     for (int wv = 0; wv < kRedThreads / 32; ++wv) sum += red[wv][i];
-    partial[(int64_t)blockIdx.x * pstride + (i < NG ? g0 + i : kp1)] = sum;
+    partial[(int64_t)i * kRedBlocks + blockIdx.x] = sum;
+  }
+  if (!last_block(cnt)) return;
+  for (int i = warp; i < NA; i += kRedThreads / 32) {
+    const double sum = warp_sum(partial + (int64_t)i * kRedBlocks, gridDim.x, lane);
+    if (lane == 0) out[i < NG ? g0 + i : kp1] = sum;
   }
 }
-
-// out[i] = sum over blocks of partial[b][i]: one block per dot, strided
-// per-thread sums and a shared-memory tree (fixed order: deterministic).
-__global__ void k_reduce_partials(const double* __restrict__ partial, int nblk, int pstride, int nd,
-                                  double* __restrict__ out, const double* __restrict__ flag, int zero_if_skipped) {
-  __shared__ double red[256];
-  const int i = blockIdx.x;
-  if (i >= nd) return;
-  if (flag && *flag == 0.0) {
-    if (zero_if_skipped && threadIdx.x == 0) out[i] = 0.0;
-    return;
-  }
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += partial[(int64_t)b * pstride + i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[i] = red[0];
-}
-
-// w[n] -= sum_i h[i] V[i][n]   (h on the device).  With `partial`, each
-// block also writes the sum of the updated w[n]^2 over its elements.
-__global__ void __launch_bounds__(kBlock) k_maxpy(const double* __restrict__ V, int64_t ldv, int kp1,
-                                                  const double* __restrict__ h, double* __restrict__ w,
-                                                  int64_t len, double sign, const double* __restrict__ flag,
-                                                  double* __restrict__ partial) {
-  if (flag && *flag == 0.0) return;
-  __shared__ double hs[130];
-  __shared__ double red[kBlock / 32];
-  for (int i = threadIdx.x; i < kp1; i += blockDim.x) hs[i] = sign * h[i];
-  __syncthreads();
-  double ss = 0.0;
-  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x) {
-    double acc = w[n];
-    for (int i = 0; i < kp1; ++i) acc -= hs[i] * V[(int64_t)i * ldv + n];
-    w[n] = acc;
-    if (partial) ss = fma(acc, acc, ss);
-  }
-  if (!partial) return;
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < kBlock / 32; ++i) t += red[i];
-    partial[blockIdx.x] = t;
-  }
-}
-
-// y = x * f(*sp): mode 0 f = s, mode 1 f = 1/s, mode 2 f = 1/sqrt(s) (0 if
-// s == 0); x and y may be the same vector (no __restrict__ on them).
-__global__ void k_scale(const double* x, double* y, int64_t len, const double* __restrict__ sp, int mode) {
-  // the factor once per block (an FP64 divide and square root per thread
-  // cost more than the scaling itself on this GPU)
-  __shared__ double sfac;
-  if (threadIdx.x == 0) {
-    const double v = *sp;
-    sfac = mode == 0 ? v : (v != 0.0 ? (mode == 1 ? 1.0 / v : 1.0 / sqrt(v)) : 0.0);
-  }
-  __syncthreads();
-  const double s = sfac;
-  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x)
-    y[n] = x[n] * s;
-}
-
-// Per-field squared norms of (b / sqrt(d)) over the 4 fields (c_s optional),
-// one contiguous range per field.
-__global__ void k_field_norms(const double* __restrict__ b, const double* __restrict__ rsqd, int64_t nn, int64_t len,
-                              double* __restrict__ partial) {
-  double acc[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const int64_t lo = f * nn, hi = f < 3 ? (f + 1) * nn : len;
-    acc[f] = hi > lo ? sumsq_share<true>(b + lo, rsqd + lo, hi - lo) : 0.0;
-  }
-  block_sum4(acc, partial);
-}
-
-// Field weights of the Krylov norm: w_f = 1 / max(||b~_f||, floor_f), b~ = b/sqrt(d).
-// Forward solves: floor_f = (1e-14/rtol) ||(sqrt(d) u)_f|| with u the
-// linearization state -- a field's right-hand side is balanced against the
-// others unless it lies below the rounding level of the field's own terms
-// (then FGMRES could never reduce its residual by rtol).  Adjoint solves:
-// floor_f = 1e-2 ||b~|| (the adjoint variable has no state scale).
-__device__ void weights_of(const double* s4, const double* __restrict__ unorm2, double floor_rel, int adjoint,
-                           double* __restrict__ wf, double* __restrict__ iwf, double* bn2) {
-  double all = 0.0;
-  for (int f = 0; f < 4; ++f) all += s4[f];
-  double tot = 0.0;
-  for (int f = 0; f < 4; ++f) {
-    const double fl = adjoint ? 1e-4 * all : floor_rel * floor_rel * unorm2[f];
-    const double s = fmax(s4[f], fl);
-    wf[f] = s > 0.0 ? 1.0 / sqrt(s) : 1.0;
-    iwf[f] = s > 0.0 ? sqrt(s) : 1.0;
-    bn2[f] = s;
-    tot += s > 0.0 ? s4[f] / s : 0.0;
-  }
-  bn2[4] = tot;
-}
-
-__global__ void k_weights(const double* __restrict__ partial, int nblk, const double* __restrict__ unorm2,
-                          double floor_rel, int adjoint, double* __restrict__ wf, double* __restrict__ iwf,
-                          double* bn2) {
-  __shared__ double s4[4];
-  sum4_warps(partial, nblk, s4);
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  weights_of(s4, unorm2, floor_rel, adjoint, wf, iwf, bn2);
-}
-
-// The same from the four field sums already in sums[0..3] (bn2 may alias sums).
-__global__ void k_weights_sums(const double* sums, const double* __restrict__ unorm2, double floor_rel,
-                               double* __restrict__ wf, double* __restrict__ iwf, double* bn2) {
-  if (threadIdx.x != 0) return;
-  double s4[4];
-  for (int f = 0; f < 4; ++f) s4[f] = sums[f];
-  weights_of(s4, unorm2, floor_rel, 0, wf, iwf, bn2);
-}
-
-// dst = src when the second Gram-Schmidt pass ran (flag), else unchanged.
-__global__ void k_take_if(double* dst, const double* __restrict__ src, const double* __restrict__ flag) {
-  if (threadIdx.x == 0 && *flag != 0.0) *dst = *src;
-}
-
-// Per-field squared norms of an already scaled vector.
-__global__ void k_field_norms_plain(const double* __restrict__ r, int64_t nn, int64_t len, double* __restrict__ partial) {
-  double acc[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const int64_t lo = f * nn, hi = f < 3 ? (f + 1) * nn : len;
-    acc[f] = hi > lo ? sumsq_share<false>(r + lo, nullptr, hi - lo) : 0.0;
-  }
-  block_sum4(acc, partial);
-}
-
-__global__ void k_sum4(const double* __restrict__ partial, int nblk, double* out) { sum4_warps(partial, nblk, out); }
 
 // Hessenberg layout in hs: H[(m+1) x m] column-major, cs[m], sn[m], g[m+1], y[m], misc
 struct HLay {
@@ -281,55 +180,54 @@ HLay hlay(int m) {
 //   misc+2m+4              : status (0 ok, 1 breakdown, 2 nonfinite)
 //   misc+2m+5              : beta (initial residual norm)
 
-__global__ void k_init_cycle(double* hs, HLay L, int* kdev) {
-  if (threadIdx.x != 0) return;
-  *kdev = 0;   // Krylov column of the next preconditioner application
-  const double* nrm2 = hs + L.misc + 2 * L.m + 2;
-  const double beta = sqrt(*nrm2);
-  for (int i = 0; i <= L.m; ++i) hs[L.g + i] = 0.0;
-  hs[L.g] = beta;
-  hs[L.misc + 2 * L.m + 5] = beta;
-  hs[L.misc + 2 * L.m + 3] = beta;
-}
-
 // Column k: h = h1 + h2, h_{k+1,k} = ||w||, previous rotations, new rotation.
-// refine = 0: no second Gram-Schmidt pass ran, h2 is not read.
-__global__ void k_givens(double* hs, HLay L, int k, int* kdev, int refine) {
-  if (threadIdx.x != 0) return;
-  *kdev = k + 1;
+// refine = 0: no second Gram-Schmidt pass ran, h2 is not read.  All threads
+// of one block: the loads side by side, the rotations (a dependent chain) by
+// thread 0 in shared memory.
+__device__ void givens_block(double* hs, const HLay& L, int k, int* kdev, int refine) {
+  __shared__ double col[130], c_[130], s_[130];
   const int m = L.m;
-  double* H = hs + L.H;
-  double* cs = hs + L.cs;
-  double* sn = hs + L.sn;
-  double* g = hs + L.g;
   const double* h1 = hs + L.misc;
   const double* h2 = hs + L.misc + m + 1;
-  const double nw = sqrt(hs[L.misc + 2 * m + 2]);
-  double* col = H + (int64_t)k * (m + 1);
-  for (int i = 0; i <= k; ++i) col[i] = refine ? h1[i] + h2[i] : h1[i];
-  col[k + 1] = nw;
-  for (int i = 0; i < k; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
+  for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+    col[i] = refine ? __ldcg(h1 + i) + __ldcg(h2 + i) : __ldcg(h1 + i);
+    c_[i] = i < k ? hs[L.cs + i] : 0.0;
+    s_[i] = i < k ? hs[L.sn + i] : 0.0;
   }
-  const double den = hypot(col[k], col[k + 1]);
-  double status = 0.0;
-  if (!(den > 0.0) || !isfinite(den)) {
-    cs[k] = 1.0; sn[k] = 0.0;
-    status = isfinite(den) ? 1.0 : 2.0;
-  } else {
-    cs[k] = col[k] / den;
-    sn[k] = col[k + 1] / den;
-    col[k] = den;
-    col[k + 1] = 0.0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *kdev = k + 1;
+    double* g = hs + L.g;
+    const double gk = g[k];
+    const double nw = sqrt(__ldcg(hs + L.misc + 2 * m + 2));
+    for (int i = 0; i < k; ++i) {
+      const double t = c_[i] * col[i] + s_[i] * col[i + 1];
+      col[i + 1] = -s_[i] * col[i] + c_[i] * col[i + 1];
+      col[i] = t;
+    }
+    const double den = hypot(col[k], nw);
+    double status = 0.0, ck = 1.0, sk = 0.0, last = nw;
+    if (!(den > 0.0) || !isfinite(den)) {
+      status = isfinite(den) ? 1.0 : 2.0;
+    } else {
+      ck = col[k] / den;
+      sk = nw / den;
+      col[k] = den;
+      last = 0.0;
+    }
+    hs[L.cs + k] = ck;
+    hs[L.sn + k] = sk;
+    hs[L.H + (int64_t)k * (m + 1) + k + 1] = last;
+    const double gn = -sk * gk;
+    g[k + 1] = gn;
+    g[k] = ck * gk;
+    hs[L.misc + 2 * m + 3] = fabs(gn);
+    if (nw == 0.0 && status == 0.0) status = 1.0;   // happy breakdown: exact solution in the space
+    if (!isfinite(gn)) status = 2.0;
+    hs[L.misc + 2 * m + 4] = status;
   }
-  g[k + 1] = -sn[k] * g[k];
-  g[k] = cs[k] * g[k];
-  hs[L.misc + 2 * m + 3] = fabs(g[k + 1]);
-  if (nw == 0.0 && status == 0.0) status = 1.0;   // happy breakdown: exact solution in the space
-  if (!isfinite(g[k + 1])) status = 2.0;
-  hs[L.misc + 2 * m + 4] = status;
+  __syncthreads();
+  for (int i = threadIdx.x; i <= k; i += blockDim.x) hs[L.H + (int64_t)k * (m + 1) + i] = col[i];
 }
 
 // Reorthogonalise only when the first Gram-Schmidt pass cancelled more than
@@ -337,8 +235,7 @@ __global__ void k_givens(double* hs, HLay L, int k, int* kdev, int refine) {
 // Stewart); count the passes in misc+2m+7.
 // eta2 = 0.49: a second pass when ||w|| fell below 0.7 ||w_0||; eta2 = 2:
 // always (||w|| never grows in a pass).
-__global__ void k_reorth_flag(double* hs, HLay L, int k, double eta2) {
-  if (threadIdx.x != 0) return;
+__device__ void reorth_test(double* hs, const HLay& L, int k, double eta2) {
   double* misc = hs + L.misc;
   const double before = misc[k + 1];
   const double after = misc[2 * L.m + 2];
@@ -347,17 +244,348 @@ __global__ void k_reorth_flag(double* hs, HLay L, int k, double eta2) {
   misc[2 * L.m + 7] += f;
 }
 
-__global__ void k_backsolve(double* hs, HLay L, int kk) {
+// What the last block of an update does with ||w||^2.
+enum : int {
+  kFinNone = 0,     // no norm
+  kFinNorm = 1,     // write it
+  kFinReorth = 2,   // and decide on the second pass
+  kFinGivens = 3,   // and update the Hessenberg column
+};
+struct Fin {
+  int mode = kFinNone;
+  double* norm = nullptr;    // ||w||^2
+  int zero_if_skipped = 0;   // norm = 0 when the pass is skipped
+  double* hs = nullptr;      // kFinReorth, kFinGivens
+  HLay L{};
+  int k = 0;
+  double eta2 = 0.0;
+  int* kdev = nullptr;
+  int refine = 0;
+};
+
+// w[n] -= sum_i h[i] V[i][n] (h on the device), the products subtracted in
+// order of i; the loads of eight basis vectors are in flight at a time (R:
+// kp1 mod 8).  With fin.mode, each block also sums the updated w[n]^2 and
+// the last block finishes as fin says.  One element per thread and a grid of
+// up to 16 blocks per SM: 14 us at 614 k elements and 7 vectors against 20
+// us with one load per product in flight.
+template <int R>
+__global__ void __launch_bounds__(kBlock) k_maxpy(const double* __restrict__ V, int64_t ldv, int kp1,
+                                                  const double* __restrict__ h, double* __restrict__ w,
+                                                  int64_t len, double sign, const double* __restrict__ flag,
+                                                  double* __restrict__ partial, unsigned* cnt, Fin fin) {
+  if (flag && *flag == 0.0) {
+    if (blockIdx.x == 0) {
+      if (fin.mode == kFinGivens) givens_block(fin.hs, fin.L, fin.k, fin.kdev, fin.refine);
+      else if (fin.zero_if_skipped && threadIdx.x == 0) *fin.norm = 0.0;
+    }
+    return;
+  }
+  __shared__ double hs[130];
+  __shared__ double red[kBlock / 32];
+  for (int i = threadIdx.x; i < kp1; i += blockDim.x) hs[i] = sign * h[i];
+  __syncthreads();
+  double ss = 0.0;
+  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x) {
+    double acc = w[n];
+    const double* v = V + n;
+    int i = 0;
+    for (; i + 8 <= kp1; i += 8) {
+      double a[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) a[q] = v[(int64_t)(i + q) * ldv];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc -= hs[i + q] * a[q];
+    }
+    if (R > 0) {
+      double a[R > 0 ? R : 1];
+#pragma unroll
+      for (int q = 0; q < R; ++q) a[q] = v[(int64_t)(i + q) * ldv];
+#pragma unroll
+      for (int q = 0; q < R; ++q) acc -= hs[i + q] * a[q];
+    }
+    w[n] = acc;
+    if (fin.mode) ss = fma(acc, acc, ss);
+  }
+  if (!fin.mode) return;
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < kBlock / 32; ++i) t += red[i];
+    partial[blockIdx.x] = t;
+  }
+  if (!last_block(cnt)) return;
+  // each warp sums every eighth run of 32 partials; then the warps in order
+  double t = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) t += __ldcg(partial + b);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    t = 0.0;
+    for (int i = 0; i < kBlock / 32; ++i) t += red[i];
+    *fin.norm = t;
+    if (fin.mode == kFinReorth) reorth_test(fin.hs, fin.L, fin.k, fin.eta2);
+  }
+  if (fin.mode != kFinGivens) return;
+  __threadfence_block();
+  __syncthreads();
+  givens_block(fin.hs, fin.L, fin.k, fin.kdev, fin.refine);
+}
+
+// What block 0 of a scaling leaves behind.
+struct Tail {
+  int mode = 0;               // 1: start of a cycle (g, beta, kdev); 2: end of an Arnoldi step
+  double* hs = nullptr;
+  HLay L{};
+  int* kdev = nullptr;
+  double* stat = nullptr;     // mode 2: residual estimate and status of the step
+  double* gate = nullptr;     // mode 2: gate of the cycle's graph (see kGateOff) ...
+  int k = 0;                  // ... after step k
+  int next = 0;               // ... with a step k + 1 in the same graph, run when `handle` is set
+  cudaGraphConditionalHandle handle = 0;
+  int nf = 0;                 // mode 1 with gate: fields of the Krylov vector, ...
+  double limit = 0.0, rtol = 0.0;   // ... step limit and tolerance of the cycle
+};
+
+__device__ void init_cycle(const Tail& t) {
+  double* hs = t.hs;
+  const HLay& L = t.L;
+  *t.kdev = 0;   // Krylov column of the next preconditioner application
+  const double beta = sqrt(hs[L.misc + 2 * L.m + 2]);
+  for (int i = 0; i <= L.m; ++i) hs[L.g + i] = 0.0;
+  hs[L.g] = beta;
+  hs[L.misc + 2 * L.m + 5] = beta;
+  hs[L.misc + 2 * L.m + 3] = beta;
+  if (!t.gate) return;
+  // ||s.b_k|| and the tests the host makes before the first step
+  const double* bn2 = hs + L.misc + 2 * L.m + 8;
+  const double* bk2 = hs + L.misc + 2 * L.m + 16;
+  double bn = 0.0;
+  for (int f = 0; f < t.nf; ++f) {
+    const double wf = bn2[f] > 0 ? 1.0 / sqrt(bn2[f]) : 1.0;
+    bn += wf * wf * bk2[f];
+  }
+  bn = sqrt(bn);
+  t.gate[0] = (bn > 0.0 && isfinite(beta) && beta > t.rtol * bn) ? 0.0 : 1.0;
+  t.gate[1] = t.gate[2] = t.gate[3] = 0.0;
+  t.gate[4] = t.limit;
+  t.gate[5] = bn;
+  t.gate[6] = t.rtol;
+}
+
+// Condition of the first step of a segment of a cycle.
+__global__ void k_gate(cudaGraphConditionalHandle h, const double* __restrict__ gate, int k) {
+  if (threadIdx.x == 0) cudaGraphSetConditional(h, (gate[0] == 0.0 && (double)k < gate[4]) ? 1u : 0u);
+}
+
+// After Arnoldi step k: the cycle stops on a breakdown, a non-finite scalar
+// or a converged estimate, the same tests the host applies to a step's
+// status; otherwise the graph's next step runs (its conditional node's
+// handle is 0 unless set here).
+__device__ void step_done(const Tail& t) {
+  const double est = t.hs[t.L.misc + 2 * t.L.m + 3], st = t.hs[t.L.misc + 2 * t.L.m + 4];
+  if (t.stat) {
+    t.stat[0] = est;
+    t.stat[1] = st;
+  }
+  if (!t.gate) return;
+  double* gate = t.gate;
+  gate[1] = t.k + 1;
+  gate[2] = est;
+  gate[3] = st;
+  const bool stop = st != 0.0 || est / gate[5] <= gate[6];
+  if (stop) gate[0] = 1.0;
+  if (t.next) cudaGraphSetConditional(t.handle, (!stop && (double)(t.k + 1) < gate[4]) ? 1u : 0u);
+}
+
+// y = x / sqrt(*sp) (0 if *sp == 0); x and y may be the same vector (no
+// __restrict__ on them).
+__global__ void k_scale(const double* x, double* y, int64_t len, const double* __restrict__ sp, Tail t) {
+  // the factor once per block (an FP64 divide and square root per thread
+  // cost more than the scaling itself on this GPU)
+  __shared__ double sfac;
+  if (threadIdx.x == 0) {
+    const double v = *sp;
+    sfac = v != 0.0 ? 1.0 / sqrt(v) : 0.0;
+  }
+  __syncthreads();
+  const double s = sfac;
+  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x)
+    y[n] = x[n] * s;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (t.mode == 1) init_cycle(t);
+    else if (t.mode == 2) step_done(t);
+  }
+}
+
+// Field weights of the Krylov norm: w_f = 1 / max(||b~_f||, floor_f), b~ = b/sqrt(d).
+// Forward solves: floor_f = (1e-14/rtol) ||(sqrt(d) u)_f|| with u the
+// linearization state -- a field's right-hand side is balanced against the
+// others unless it lies below the rounding level of the field's own terms
+// (then FGMRES could never reduce its residual by rtol).  Adjoint solves:
+// floor_f = 1e-2 ||b~|| (the adjoint variable has no state scale).
+__device__ void weights_of(const double* s4, const double* __restrict__ unorm2, double floor_rel, int adjoint,
+                           double* __restrict__ wf, double* __restrict__ iwf, double* bn2) {
+  double all = 0.0;
+  for (int f = 0; f < 4; ++f) all += s4[f];
+  double tot = 0.0;
+  for (int f = 0; f < 4; ++f) {
+    const double fl = adjoint ? 1e-4 * all : floor_rel * floor_rel * unorm2[f];
+    const double s = fmax(s4[f], fl);
+    wf[f] = s > 0.0 ? 1.0 / sqrt(s) : 1.0;
+    iwf[f] = s > 0.0 ? sqrt(s) : 1.0;
+    bn2[f] = s;
+    tot += s > 0.0 ? s4[f] / s : 0.0;
+  }
+  bn2[4] = tot;
+}
+
+// Block sums of NV per-thread values into partial[v][block] (fixed order).
+template <int NV>
+__device__ __forceinline__ void sum_partials(const double (&acc)[NV], double* partial) {
+  __shared__ double red[NV][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int f = 0; f < NV; ++f) {
+    double a = acc[f];
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    if (lane == 0) red[f][warp] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += red[threadIdx.x][w];
+    partial[(int64_t)threadIdx.x * kRedBlocks + blockIdx.x] = t;
+  }
+}
+
+// Per-field squared norms of (b / sqrt(d)) over the 4 fields (c_s optional),
+// one contiguous range per field: sums[0..3], or with wf the Krylov weights
+// (see weights_of; bn2 is then sums[0..4]).
+__global__ void __launch_bounds__(kRedThreads) k_field_norms(const double* __restrict__ b,
+                                                             const double* __restrict__ rsqd, int64_t nn, int64_t len,
+                                                             double* __restrict__ partial, unsigned* cnt,
+                                                             const double* __restrict__ unorm2, double floor_rel,
+                                                             int adjoint, double* __restrict__ wf,
+                                                             double* __restrict__ iwf, double* __restrict__ sums) {
+  double acc[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const int64_t lo = f * nn, hi = f < 3 ? (f + 1) * nn : len;
+    acc[f] = hi > lo ? sumsq_share<true>(b + lo, rsqd + lo, hi - lo) : 0.0;
+  }
+  sum_partials<4>(acc, partial);
+  if (!last_block(cnt)) return;
+  __shared__ double s4[4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < 4) {
+    const double t = warp_sum(partial + (int64_t)warp * kRedBlocks, gridDim.x, lane);
+    if (lane == 0) s4[warp] = t;
+  }
+  __syncthreads();
+  if (wf) {
+    if (threadIdx.x == 0) weights_of(s4, unorm2, floor_rel, adjoint, wf, iwf, sums);
+  } else if (threadIdx.x < 4) {
+    sums[threadIdx.x] = s4[threadIdx.x];
+  }
+}
+
+// The three sets of field norms of a finished solve in one pass over its
+// vectors: out[0..3] = ||r_f||^2, out[8..11] = ||(sqd r)_f||^2, out[12..15] =
+// ||b_f||^2.
+__global__ void __launch_bounds__(kRedThreads) k_final_norms(const double* __restrict__ r,
+                                                             const double* __restrict__ sqd,
+                                                             const double* __restrict__ b, int64_t nn, int64_t len,
+                                                             double* __restrict__ partial, unsigned* cnt,
+                                                             double* __restrict__ out) {
+  double acc[12];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const int64_t lo = f * nn, hi = f < 3 ? (f + 1) * nn : len, stride = (int64_t)gridDim.x * blockDim.x;
+    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0, c0 = 0.0, c1 = 0.0;
+    int64_t i = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (; i + stride < hi; i += 2 * stride) {   // two elements in flight
+      const double r0 = r[i], r1 = r[i + stride], q0 = sqd[i], q1 = sqd[i + stride], v0 = b[i], v1 = b[i + stride];
+      const double u0 = r0 * q0, u1 = r1 * q1;
+      a0 = fma(r0, r0, a0);
+      a1 = fma(r1, r1, a1);
+      b0 = fma(u0, u0, b0);
+      b1 = fma(u1, u1, b1);
+      c0 = fma(v0, v0, c0);
+      c1 = fma(v1, v1, c1);
+    }
+    if (i < hi) {
+      const double r0 = r[i], u0 = r0 * sqd[i], v0 = b[i];
+      a0 = fma(r0, r0, a0);
+      b0 = fma(u0, u0, b0);
+      c0 = fma(v0, v0, c0);
+    }
+    acc[f] = a0 + a1;
+    acc[4 + f] = b0 + b1;
+    acc[8 + f] = c0 + c1;
+  }
+  sum_partials<12>(acc, partial);
+  if (!last_block(cnt)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int v = warp; v < 12; v += kRedThreads / 32) {
+    const double t = warp_sum(partial + (int64_t)v * kRedBlocks, gridDim.x, lane);
+    if (lane == 0) out[v < 4 ? v : v + 4] = t;
+  }
+}
+
+// The same from the four field sums already in sums[0..3] (bn2 may alias sums).
+__global__ void k_weights_sums(const double* sums, const double* __restrict__ unorm2, double floor_rel,
+                               double* __restrict__ wf, double* __restrict__ iwf, double* bn2) {
   if (threadIdx.x != 0) return;
-  const int m = L.m;
+  double s4[4];
+  for (int f = 0; f < 4; ++f) s4[f] = sums[f];
+  weights_of(s4, unorm2, floor_rel, 0, wf, iwf, bn2);
+}
+
+// dst = src when the second Gram-Schmidt pass ran (flag), else unchanged.
+__global__ void k_take_if(double* dst, const double* __restrict__ src, const double* __restrict__ flag) {
+  if (threadIdx.x == 0 && *flag != 0.0) *dst = *src;
+}
+
+// Launches of the above for the slab decomposition, whose sums pass through
+// an allreduce between a kernel and its decision.
+__global__ void k_givens(double* hs, HLay L, int k, int* kdev, int refine) { givens_block(hs, L, k, kdev, refine); }
+__global__ void k_reorth_flag(double* hs, HLay L, int k, double eta2) {
+  if (threadIdx.x == 0) reorth_test(hs, L, k, eta2);
+}
+
+// H y = g by one warp, column by column from the last: lane j keeps rows
+// j, j + 32, ... of g; the diagonal's reciprocals are formed side by side
+// (a serial row-wise substitution took 24 us at 13 columns).
+__global__ void __launch_bounds__(32) k_backsolve(double* hs, HLay L, int kk) {
+  const int lane = threadIdx.x, ld = L.m + 1;
   const double* H = hs + L.H;
-  const double* g = hs + L.g;
-  double* y = hs + L.y;
+  double g[4], rd[4], nx[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = lane + 32 * q;
+    g[q] = i < kk ? hs[L.g + i] : 0.0;
+    const double d = i < kk ? H[(int64_t)i * ld + i] : 0.0;
+    rd[q] = d != 0.0 ? 1.0 / d : 0.0;
+    nx[q] = i < kk - 1 ? H[(int64_t)(kk - 1) * ld + i] : 0.0;
+  }
   for (int i = kk - 1; i >= 0; --i) {
-    double s = g[i];
-    for (int j = i + 1; j < kk; ++j) s -= H[(int64_t)j * (m + 1) + i] * y[j];
-    const double d = H[(int64_t)i * (m + 1) + i];
-    y[i] = d != 0.0 ? s / d : 0.0;
+    double c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      c[q] = nx[q];
+      const int j = lane + 32 * q;
+      nx[q] = j < i - 1 ? H[(int64_t)(i - 1) * ld + j] : 0.0;   // the next column's load is in flight
+    }
+    const int iq = i >> 5;
+    const double mine = iq == 0 ? g[0] * rd[0] : (iq == 1 ? g[1] * rd[1] : (iq == 2 ? g[2] * rd[2] : g[3] * rd[3]));
+    const double y = __shfl_sync(0xffffffffu, mine, i & 31);
+    if (lane == 0) hs[L.y + i] = y;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) g[q] -= c[q] * y;   // rows j >= i: c = 0
   }
 }
 
@@ -414,8 +642,11 @@ __global__ void k_surface_coupling(int64_t NE, double tau, const int32_t* __rest
 
 struct Reducer {
   p4d_ctx* c;
+  // one element per thread and trip on small vectors (a block per 512
+  // elements: eight per thread left 3 blocks at 6,075 elements and 14 us),
+  // kRedBlocks blocks on large ones
   int nblk(int64_t len) const {
-    const int64_t want = (len + (int64_t)kRedThreads * 8 - 1) / ((int64_t)kRedThreads * 8);
+    const int64_t want = (len + (int64_t)kRedThreads * 2 - 1) / ((int64_t)kRedThreads * 2);
     return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, want));
   }
   // out[0..kp1) = V^T w, out[kp1] = w.w (optional)
@@ -424,24 +655,21 @@ struct Reducer {
   void mdot(const double* V, int64_t ldv, int kp1, const double* w, int64_t len, bool ww, double* out,
             const double* flag = nullptr, int zero_if_skipped = 0) {
     const int nb = nblk(len);
-    const int ps = 132;
-    if (kp1 == 0) launch_group<0>(ww, V, ldv, 0, kp1, w, len, nb, ps, flag);
+    if (kp1 == 0) launch_group<0>(ww, V, ldv, 0, kp1, w, len, nb, out, flag, zero_if_skipped);
     for (int g0 = 0; g0 < kp1; g0 += kDotGroup)
-      dispatch(std::min(kDotGroup, kp1 - g0), ww && g0 == 0, V, ldv, g0, kp1, w, len, nb, ps, flag);
-    ::p4d::count_launch(), k_reduce_partials<<<kp1 + (ww ? 1 : 0), 256, 0, c->stream>>>(c->part, nb, ps, kp1 + (ww ? 1 : 0), out, flag,
-                                                                  zero_if_skipped);
+      dispatch(std::min(kDotGroup, kp1 - g0), ww && g0 == 0, V, ldv, g0, kp1, w, len, nb, out, flag, zero_if_skipped);
   }
   template <int NG>
   void launch_group(bool ww, const double* V, int64_t ldv, int g0, int kp1, const double* w, int64_t len, int nb,
-                    int ps, const double* flag) {
-    if (ww) ::p4d::count_launch(), k_mdot<NG, true><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, g0, kp1, w, len, c->part, ps, flag);
-    else ::p4d::count_launch(), k_mdot<NG, false><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, g0, kp1, w, len, c->part, ps, flag);
+                    double* out, const double* flag, int z) {
+    if (ww) ::p4d::count_launch(), k_mdot<NG, true><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, g0, kp1, w, len, c->part, out, c->red_cnt, flag, z);
+    else ::p4d::count_launch(), k_mdot<NG, false><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, g0, kp1, w, len, c->part, out, c->red_cnt, flag, z);
   }
   void dispatch(int ng, bool ww, const double* V, int64_t ldv, int g0, int kp1, const double* w, int64_t len, int nb,
-                int ps, const double* flag) {
+                double* out, const double* flag, int z) {
     switch (ng) {
 #define P4D_MDOT_CASE(K) \
-  case K: launch_group<K>(ww, V, ldv, g0, kp1, w, len, nb, ps, flag); break;
+  case K: launch_group<K>(ww, V, ldv, g0, kp1, w, len, nb, out, flag, z); break;
       P4D_MDOT_CASE(1) P4D_MDOT_CASE(2) P4D_MDOT_CASE(3) P4D_MDOT_CASE(4) P4D_MDOT_CASE(5) P4D_MDOT_CASE(6)
       P4D_MDOT_CASE(7) P4D_MDOT_CASE(8) P4D_MDOT_CASE(9) P4D_MDOT_CASE(10) P4D_MDOT_CASE(11) P4D_MDOT_CASE(12)
       P4D_MDOT_CASE(13) P4D_MDOT_CASE(14) P4D_MDOT_CASE(15) P4D_MDOT_CASE(16)
@@ -449,16 +677,30 @@ struct Reducer {
       default: break;
     }
   }
-  // w -= V h over kp1 vectors; with norm_out, also norm_out = ||w_new||^2
+  // w -= V h over kp1 vectors, finished as fin says
   void maxpy(const double* V, int64_t ldv, int kp1, const double* h, double* w, int64_t len, double sign,
-             const double* flag, double* norm_out, unsigned gb) {
-    ::p4d::count_launch(), k_maxpy<<<gb, kBlock, 0, c->stream>>>(V, ldv, kp1, h, w, len, sign, flag,
-                                                               norm_out ? c->part : nullptr);
-    if (norm_out)
-      ::p4d::count_launch(), k_reduce_partials<<<1, 256, 0, c->stream>>>(c->part, (int)gb, 1, 1, norm_out, flag, 0);
+             const double* flag, const Fin& fin, unsigned gb) {
+    switch (kp1 & 7) {
+#define P4D_MAXPY_CASE(R) \
+  case R: ::p4d::count_launch(), k_maxpy<R><<<gb, kBlock, 0, c->stream>>>(V, ldv, kp1, h, w, len, sign, flag, c->part, c->red_cnt, fin); break;
+      P4D_MAXPY_CASE(0) P4D_MAXPY_CASE(1) P4D_MAXPY_CASE(2) P4D_MAXPY_CASE(3)
+      P4D_MAXPY_CASE(4) P4D_MAXPY_CASE(5) P4D_MAXPY_CASE(6) P4D_MAXPY_CASE(7)
+#undef P4D_MAXPY_CASE
+    }
+  }
+  static Fin norm_to(double* out, int zero_if_skipped = 0) {
+    Fin f;
+    f.mode = kFinNorm;
+    f.norm = out;
+    f.zero_if_skipped = zero_if_skipped;
+    return f;
   }
 };
 
+// Blocks of a sum over len entries (four per thread and trip).
+inline int norm_blocks(int64_t len) {
+  return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, len / (4 * kRedThreads)));
+}
 
 }  // namespace
 
@@ -472,15 +714,6 @@ namespace {
 // synchronization for all, then every cell's read phase, with the Arnoldi
 // steps of all cells in one graph per Krylov column.
 
-// Status of Arnoldi step k into dst[0..1] (residual estimate, status): the
-// batched step graphs gather every cell's pair in one device array.
-__global__ void k_put_status(const double* __restrict__ src, double* __restrict__ dst) {
-  if (threadIdx.x == 0) {
-    dst[0] = src[0];
-    dst[1] = src[1];
-  }
-}
-
 // Condition of a cell's conditional (IF) node in a batched step graph.
 __global__ void k_set_active(cudaGraphConditionalHandle h, const int* __restrict__ active) {
   if (threadIdx.x == 0) cudaGraphSetConditional(h, *active ? 1u : 0u);
@@ -491,18 +724,12 @@ __global__ void k_set_active(cudaGraphConditionalHandle h, const int* __restrict
 // step, [4] step limit of the cycle, [5] ||s.b_k||, [6] rtol.
 constexpr int kGateOff = 48;
 
-__global__ void k_gate(cudaGraphConditionalHandle h, const double* __restrict__ gate, int k) {
-  if (threadIdx.x == 0) cudaGraphSetConditional(h, (gate[0] == 0.0 && (double)k < gate[4]) ? 1u : 0u);
-}
-
-// After Arnoldi step k (whose estimate and status k_put_status left in
-// gate[2..3]): the cycle stops on a breakdown, a non-finite scalar or a
-// converged estimate, the same tests the host applies to a step's status.
-__global__ void k_step_done(double* gate, int k) {
-  if (threadIdx.x != 0) return;
-  gate[1] = k + 1;
-  if (gate[3] != 0.0 || gate[2] / gate[5] <= gate[6]) gate[0] = 1.0;
-}
+// Pinned mirror (hs_h): [0..11] right-hand-side norms at the start, [0..32]
+// the report at the end, [0..1] a step's status when stepped from the host,
+// then
+constexpr int kBetaOff = 40;   // beta of a cycle
+constexpr int kTrueOff = 41;   // squared true residual at a cycle's end
+constexpr int kGateRead = 44;  // gate[0..5] after a segment of a cycle
 
 struct FgRun;
 void fg_release(FgRun& r);
@@ -561,10 +788,9 @@ p4d_status fg_begin(FgRun& r, p4d_ctx* c, const double* b, double* x, int trans)
   P4D_TRY(cudaEventRecord(r.ev0, c->stream));
   // per-field weights from the full right-hand side
   {
-    const int nb = kRedBlocks;
-    ::p4d::count_launch(), k_field_norms<<<nb, kRedThreads, 0, c->stream>>>(b, c->rsqd, r.nn, c->ndof, c->part);
-    ::p4d::count_launch(), k_weights<<<1, 128, 0, c->stream>>>(c->part, nb, c->unorm2, 1e-14 / c->prm.rtol, trans,
-                                                             c->wf, c->iwf, hs + L.misc + 2 * L.m + 8);
+    ::p4d::count_launch(), k_field_norms<<<norm_blocks(c->ndof), kRedThreads, 0, c->stream>>>(
+        b, c->rsqd, r.nn, c->ndof, c->part, c->red_cnt, c->unorm2, 1e-14 / c->prm.rtol, trans, c->wf, c->iwf,
+        hs + L.misc + 2 * L.m + 8);
   }
   r.bk = b;
   if (!r.full) {
@@ -575,14 +801,15 @@ p4d_status fg_begin(FgRun& r, p4d_ctx* c, const double* b, double* x, int trans)
         c->bred, trans);
     r.bk = c->bred;
   }
-  ::p4d::count_launch(), k_field_norms<<<kRedBlocks, kRedThreads, 0, c->stream>>>(r.bk, c->rsqd, r.nn, r.len, c->part);
-  ::p4d::count_launch(), k_sum4<<<1, 128, 0, c->stream>>>(c->part, kRedBlocks, hs + L.misc + 2 * L.m + 16);
+  ::p4d::count_launch(), k_field_norms<<<norm_blocks(r.len), kRedThreads, 0, c->stream>>>(
+      r.bk, c->rsqd, r.nn, r.len, c->part, c->red_cnt, nullptr, 0.0, 0, nullptr, nullptr, hs + L.misc + 2 * L.m + 16);
   P4D_TRY(cudaMemcpyAsync(c->hs_h, hs + L.misc + 2 * L.m + 8, sizeof(double) * 12, cudaMemcpyDeviceToHost, c->stream));
+  P4D_TRY(cudaMemsetAsync(r.misc() + 2 * L.m + 7, 0, sizeof(double), c->stream));   // second passes
   return P4D_OK;
 }
 
 // ||s.b_k|| = sqrt(sum_f w_f^2 ||(b_k / sqrt(d))_f||^2); b_k = 0 gives x = 0.
-p4d_status fg_bnorm(FgRun& r) {
+p4d_status fg_bnorm(FgRun& r, bool gated = false) {
   p4d_ctx* c = r.c;
   const double* bn2 = c->hs_h;        // full-b field norms^2 (weights)
   const double* bk2 = c->hs_h + 8;    // Krylov-rhs field norms^2
@@ -592,17 +819,18 @@ p4d_status fg_bnorm(FgRun& r) {
     bnorm += wf * wf * bk2[f];
   }
   r.bnorm = std::sqrt(bnorm);
+  if (gated) r.bnorm = c->hs_h[kGateRead + 5];   // the value the device gate tests with
   if (r.bnorm == 0.0) {
     P4D_TRY(cudaMemsetAsync(r.x, 0, sizeof(double) * c->ndof, c->stream));
     r.st = P4D_OK;
     r.est = 0.0;
   }
-  P4D_TRY(cudaMemsetAsync(r.misc() + 2 * r.L.m + 7, 0, sizeof(double), c->stream));
   return P4D_OK;
 }
 
 // Start of a restart cycle: V0 = s.(b_k - A x), beta = ||V0||, V0 /= beta.
-p4d_status fg_cycle_launch(FgRun& r) {
+// gate: also prepare the device gate of a graph-driven cycle.
+p4d_status fg_cycle_launch(FgRun& r, bool gate = false) {
   p4d_ctx* c = r.c;
   Reducer R{c};
   double* misc = r.misc();
@@ -611,14 +839,24 @@ p4d_status fg_cycle_launch(FgRun& r) {
   if (r.full) P4D_TRYS(jvp_full(c, r.x, c->V, r.trans, r.bk, true));
   else P4D_TRYS(jvp_reduced(c, r.x, c->V, r.trans, r.bk, true));
   R.mdot(c->V, 0, 0, c->V, r.len, true, misc + 2 * L.m + 2);
-  ::p4d::count_launch(), k_init_cycle<<<1, 1, 0, c->stream>>>(c->hs, L, c->kdev);
-  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(c->V, c->V, r.len, misc + 2 * L.m + 5, 1);
-  P4D_TRY(cudaMemcpyAsync(c->hs_h, misc + 2 * L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  Tail t;
+  t.mode = 1;
+  t.hs = c->hs;
+  t.L = L;
+  t.kdev = c->kdev;
+  if (gate) {
+    t.gate = misc + 2 * L.m + kGateOff;
+    t.nf = r.full ? 4 : 3;
+    t.limit = (double)std::min(r.m, c->prm.maxit - r.iters);
+    t.rtol = c->prm.rtol;
+  }
+  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(c->V, c->V, r.len, misc + 2 * L.m + 2, t);
+  P4D_TRY(cudaMemcpyAsync(c->hs_h + kBetaOff, misc + 2 * L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
 }
 
 void fg_cycle_read(FgRun& r) {
-  const double beta = r.c->hs_h[0];
+  const double beta = r.c->hs_h[kBetaOff];
   r.est = beta / r.bnorm;
   r.kk = 0;
   r.cycle_done = false;
@@ -634,8 +872,9 @@ void fg_cycle_read(FgRun& r) {
 
 // Arnoldi step k: z_k = P^-1 (s^-1 v_k), w = s.J z_k, CGS (second pass only
 // when needed), Givens, v_{k+1} = w / h_{k+1,k}; the residual estimate and
-// status go to the host mirror (stat == nullptr) or to stat[0..1] (device).
-p4d_status fg_step_body(FgRun& r, int k, bool graph_precond, double* stat) {
+// status go where t says (batch status or cycle gate on the device), or to
+// the host mirror.
+p4d_status fg_step_body(FgRun& r, int k, bool graph_precond, Tail t) {
   p4d_ctx* c = r.c;
   Reducer R{c};
   double* misc = r.misc();
@@ -651,19 +890,31 @@ p4d_status fg_step_body(FgRun& r, int k, bool graph_precond, double* stat) {
   prof_mark(c, 1);
   prof_mark(c, 2);
   const double* flag = misc + 2 * L.m + 6;
-  R.mdot(c->V, r.len, k + 1, w, r.len, true, misc);                                        // h1, ||w||^2 before
-  R.maxpy(c->V, r.len, k + 1, misc, w, r.len, 1.0, nullptr, misc + 2 * L.m + 2, r.gb);     // ||w||^2 after
-  if (c->prm.cgs_refine > 0) {
-    ::p4d::count_launch(), k_reorth_flag<<<1, 1, 0, c->stream>>>(c->hs, L, k, c->prm.cgs_refine == 2 ? 2.0 : 0.49);
+  const int refine = c->prm.cgs_refine;
+  Fin fin = Reducer::norm_to(misc + 2 * L.m + 2);
+  fin.hs = c->hs;
+  fin.L = L;
+  fin.k = k;
+  fin.eta2 = refine == 2 ? 2.0 : 0.49;
+  fin.kdev = c->kdev;
+  fin.refine = refine;
+  R.mdot(c->V, r.len, k + 1, w, r.len, true, misc);   // h1, ||w||^2 before
+  fin.mode = refine > 0 ? kFinReorth : kFinGivens;
+  R.maxpy(c->V, r.len, k + 1, misc, w, r.len, 1.0, nullptr, fin, r.gb);   // ||w||^2 after
+  if (refine > 0) {
     R.mdot(c->V, r.len, k + 1, w, r.len, false, misc + L.m + 1, flag, 1);   // h2 (or 0)
     // ||w||^2 after the second pass (left unchanged when it is skipped)
-    R.maxpy(c->V, r.len, k + 1, misc + L.m + 1, w, r.len, 1.0, flag, misc + 2 * L.m + 2, r.gb);
+    fin.mode = kFinGivens;
+    R.maxpy(c->V, r.len, k + 1, misc + L.m + 1, w, r.len, 1.0, flag, fin, r.gb);
   }
-  ::p4d::count_launch(), k_givens<<<1, 1, 0, c->stream>>>(c->hs, L, k, c->kdev, c->prm.cgs_refine);
-  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(w, w, r.len, misc + 2 * L.m + 2, 2);
+  const bool host = !t.stat && !t.gate;
+  t.mode = 2;
+  t.hs = c->hs;
+  t.L = L;
+  t.k = k;
+  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(w, w, r.len, misc + 2 * L.m + 2, t);
   prof_mark(c, 2);
-  if (stat) ::p4d::count_launch(), k_put_status<<<1, 32, 0, c->stream>>>(misc + 2 * L.m + 3, stat);
-  else P4D_TRY(cudaMemcpyAsync(c->hs_h, misc + 2 * L.m + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  if (host) P4D_TRY(cudaMemcpyAsync(c->hs_h, misc + 2 * L.m + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
 }
 
@@ -686,15 +937,15 @@ p4d_status fg_cycle_end_launch(FgRun& r) {
   double* misc = r.misc();
   const HLay& L = r.L;
   if (r.kk > 0) {
-    ::p4d::count_launch(), k_backsolve<<<1, 1, 0, c->stream>>>(c->hs, L, r.kk);
+    ::p4d::count_launch(), k_backsolve<<<1, 32, 0, c->stream>>>(c->hs, L, r.kk);
     // x += Z y  (k_maxpy computes w -= sum h_i V_i; use sign -1)
-    R.maxpy(c->Z, r.len, r.kk, c->hs + L.y, r.x, r.len, -1.0, nullptr, nullptr, r.gb);
+    R.maxpy(c->Z, r.len, r.kk, c->hs + L.y, r.x, r.len, -1.0, nullptr, Fin{}, r.gb);
   }
   if (r.st == P4D_OK) {
     if (r.full) P4D_TRYS(jvp_full(c, r.x, c->V, r.trans, r.bk, true));
     else P4D_TRYS(jvp_reduced(c, r.x, c->V, r.trans, r.bk, true));
     R.mdot(c->V, 0, 0, c->V, r.len, true, misc + 2 * L.m + 2);
-    P4D_TRY(cudaMemcpyAsync(c->hs_h, misc + 2 * L.m + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    P4D_TRY(cudaMemcpyAsync(c->hs_h + kTrueOff, misc + 2 * L.m + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   }
   return P4D_OK;
 }
@@ -702,7 +953,7 @@ p4d_status fg_cycle_end_launch(FgRun& r) {
 // Confirmation by the true residual (only after st == OK was launched).
 void fg_cycle_end_read(FgRun& r) {
   if (r.st != P4D_OK) return;
-  r.est = std::sqrt(r.c->hs_h[0]) / r.bnorm;
+  r.est = std::sqrt(r.c->hs_h[kTrueOff]) / r.bnorm;
   if (!(r.est <= r.c->prm.rtol) && r.iters < r.c->prm.maxit) r.st = P4D_ERR_NOT_CONVERGED;
   if (!std::isfinite(r.est)) r.st = P4D_ERR_NONFINITE;
 }
@@ -720,13 +971,9 @@ p4d_status fg_finish_launch(FgRun& r) {
   }
   // final true residual of the full system in the scaled norm
   P4D_TRYS(jvp_full(c, r.x, c->r0, r.trans, r.b, true));
-  ::p4d::count_launch(), k_field_norms_plain<<<kRedBlocks, kRedThreads, 0, c->stream>>>(c->r0, nn, c->ndof, c->part);
-  ::p4d::count_launch(), k_sum4<<<1, 128, 0, c->stream>>>(c->part, kRedBlocks, r.misc() + 2 * L.m + 24);
   // and unscaled: ||(b - J x)_f||^2 = ||(sqrt(d) r0)_f||^2 / w_f^2, ||b_f||^2
-  ::p4d::count_launch(), k_field_norms<<<kRedBlocks, kRedThreads, 0, c->stream>>>(c->r0, c->sqd, nn, c->ndof, c->part);
-  ::p4d::count_launch(), k_sum4<<<1, 128, 0, c->stream>>>(c->part, kRedBlocks, r.misc() + 2 * L.m + 32);
-  ::p4d::count_launch(), k_field_norms_plain<<<kRedBlocks, kRedThreads, 0, c->stream>>>(r.b, nn, c->ndof, c->part);
-  ::p4d::count_launch(), k_sum4<<<1, 128, 0, c->stream>>>(c->part, kRedBlocks, r.misc() + 2 * L.m + 36);
+  ::p4d::count_launch(), k_final_norms<<<norm_blocks(c->ndof), kRedThreads, 0, c->stream>>>(
+      c->r0, c->sqd, r.b, nn, c->ndof, c->part, c->red_cnt, r.misc() + 2 * L.m + 24);
   P4D_TRY(cudaEventRecord(r.ev1, c->stream));
   P4D_TRY(cudaMemcpyAsync(c->hs_h, r.misc() + 2 * L.m + 7, sizeof(double) * 33, cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
@@ -801,93 +1048,103 @@ p4d_status capture_body(p4d_ctx* c, cudaGraph_t* out, long long* kernels, F&& bo
   return st;
 }
 
-// The restart cycle of r as one graph: for k < m, gate(k) -> IF { Arnoldi
-// step k; its status into the gate }.
-p4d_status cycle_graph(FgRun& r, p4d_ctx::CycleGraph*& out) {
+// Steps [k0, k0 + kSegSteps) of a restart cycle as one graph: each Arnoldi
+// step under a conditional (IF) node, the first one's condition set by
+// k_gate from the device gate, the others' by the step before (default 0).
+// A cycle is launched segment by segment: an IF node that is not taken costs
+// 10 us, so the 17 idle steps of a 13-iteration solve in one graph of
+// restart 30 cost 0.2 of 2.1 ms, while the host's check between segments
+// costs about 15 us per eight steps; and only the segments in use are captured.
+constexpr int kSegSteps = 8;
+
+p4d_status segment_graph(FgRun& r, int k0, p4d_ctx::CycleGraph::Seg*& out) {
   p4d_ctx* c = r.c;
   p4d_ctx::CycleGraph& cg = c->cyc[r.trans ? 1 : 0][r.full ? 1 : 0];
-  out = &cg;
-  if (cg.exec && cg.m == r.m) return P4D_OK;
-  if (cg.exec) cudaGraphExecDestroy(cg.exec);
-  cg.exec = nullptr;
-  cg.kernels.assign(r.m, 0);
+  const size_t si = (size_t)(k0 / kSegSteps);
+  if (cg.m != r.m) {   // another restart length: the last segment may end elsewhere
+    for (auto& sg : cg.seg)
+      if (sg.exec) cudaGraphExecDestroy(sg.exec);
+    cg.seg.clear();
+    cg.m = r.m;
+  }
+  if (cg.seg.size() <= si) cg.seg.resize(si + 1);
+  p4d_ctx::CycleGraph::Seg& sg = cg.seg[si];
+  out = &sg;
+  if (sg.exec) return P4D_OK;
+  const int n = std::min(kSegSteps, r.m - k0);
+  sg.kernels.assign(n, 0);
   double* gate = r.misc() + 2 * r.L.m + kGateOff;
   cudaGraph_t G = nullptr;
   P4D_TRY(cudaGraphCreate(&G, 0));
   p4d_status st = P4D_OK;
+  cudaGraphConditionalHandle h[kSegSteps];
+  for (int q = 0; q < n && st == P4D_OK; ++q)
+    if (cudaGraphConditionalHandleCreate(&h[q], G, 0, cudaGraphCondAssignDefault) != cudaSuccess) st = P4D_ERR_CUDA;
   cudaGraphNode_t prev = nullptr;
-  for (int k = 0; k < r.m && st == P4D_OK; ++k) {
-    cudaGraph_t step = nullptr;
-    long long kc = 0;
-    st = capture_body(c, &step, &kc, [&]() -> p4d_status {
-      P4D_TRYS(fg_step_body(r, k, false, gate + 2));
-      ::p4d::count_launch(), k_step_done<<<1, 32, 0, c->stream>>>(gate, k);
-      return P4D_OK;
-    });
-    if (st != P4D_OK) break;
-    cudaGraphConditionalHandle h;
-    cudaGraphNode_t kn = nullptr, cn = nullptr, ch = nullptr;
+  if (st == P4D_OK) {
     const double* gc = gate;
-    int kk = k;
-    void* args[] = {&h, &gc, &kk};
+    int kk = k0;
+    void* args[] = {&h[0], &gc, &kk};
     cudaKernelNodeParams kp = {};
     kp.func = (void*)k_gate;
     kp.gridDim = dim3(1);
     kp.blockDim = dim3(32);
     kp.kernelParams = args;
+    if (cudaGraphAddKernelNode(&prev, G, nullptr, 0, &kp) != cudaSuccess) st = P4D_ERR_CUDA;
+  }
+  for (int q = 0; q < n && st == P4D_OK; ++q) {
+    cudaGraph_t step = nullptr;
+    long long kc = 0;
+    Tail t;
+    t.gate = gate;
+    t.next = q + 1 < n;
+    if (t.next) t.handle = h[q + 1];
+    st = capture_body(c, &step, &kc, [&]() { return fg_step_body(r, k0 + q, false, t); });
+    if (st != P4D_OK) break;
+    cudaGraphNode_t cn = nullptr, ch = nullptr;
     cudaGraphNodeParams cp = {};
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.type = cudaGraphCondTypeIf;
     cp.conditional.size = 1;
-    if (cudaGraphConditionalHandleCreate(&h, G, 0, cudaGraphCondAssignDefault) != cudaSuccess ||
-        cudaGraphAddKernelNode(&kn, G, prev ? &prev : nullptr, prev ? 1 : 0, &kp) != cudaSuccess)
-      st = P4D_ERR_CUDA;
-    cp.conditional.handle = h;
-    if (st == P4D_OK && cudaGraphAddNode(&cn, G, &kn, nullptr, 1, &cp) != cudaSuccess) st = P4D_ERR_CUDA;
+    cp.conditional.handle = h[q];
+    if (cudaGraphAddNode(&cn, G, &prev, nullptr, 1, &cp) != cudaSuccess) st = P4D_ERR_CUDA;
     if (st == P4D_OK && cudaGraphAddChildGraphNode(&ch, cp.conditional.phGraph_out[0], nullptr, 0, step) != cudaSuccess)
       st = P4D_ERR_CUDA;
     cudaGraphDestroy(step);
     prev = cn;
-    cg.kernels[k] = kc;
+    sg.kernels[q] = kc;
   }
-  if (st == P4D_OK && cudaGraphInstantiate(&cg.exec, G, 0) != cudaSuccess) st = P4D_ERR_CUDA;
+  if (st == P4D_OK && cudaGraphInstantiate(&sg.exec, G, 0) != cudaSuccess) st = P4D_ERR_CUDA;
   cudaGraphDestroy(G);
   if (st != P4D_OK) {
     cudaGetLastError();
-    cg.exec = nullptr;
-    return st;
+    sg.exec = nullptr;
   }
-  cg.m = r.m;
+  return st;
+}
+
+// Launch the segment that starts at step k0, and read the gate after it.
+p4d_status fg_segment_launch(FgRun& r, int k0) {
+  p4d_ctx* c = r.c;
+  p4d_ctx::CycleGraph::Seg* sg = nullptr;
+  P4D_TRYS(segment_graph(r, k0, sg));
+  P4D_TRY(cudaGraphLaunch(sg->exec, c->stream));
+  P4D_TRY(cudaMemcpyAsync(c->hs_h + kGateRead, r.misc() + 2 * r.L.m + kGateOff, 6 * sizeof(double),
+                          cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
 }
 
-// The Arnoldi steps of one restart cycle by its graph: the host uploads the
-// gate, launches the graph, and reads the gate once at the end.
-p4d_status fg_cycle_steps_graph(FgRun& r) {
+// After the synchronization: the steps the segment ran.
+p4d_status fg_segment_read(FgRun& r, int k0) {
   p4d_ctx* c = r.c;
-  p4d_ctx::CycleGraph* cg = nullptr;
-  P4D_TRYS(cycle_graph(r, cg));
-  double* gate = r.misc() + 2 * r.L.m + kGateOff;
-  double* stage = c->hs_h + kGateOff;
-  stage[0] = 0.0;
-  stage[1] = 0.0;
-  stage[2] = 0.0;
-  stage[3] = 0.0;
-  stage[4] = (double)std::min(r.m, c->prm.maxit - r.iters);
-  stage[5] = r.bnorm;
-  stage[6] = c->prm.rtol;
-  P4D_TRY(cudaMemcpyAsync(gate, stage, 7 * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  P4D_TRY(cudaGraphLaunch(cg->exec, c->stream));
-  P4D_TRY(cudaMemcpyAsync(c->hs_h, gate, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  P4D_TRY(cudaStreamSynchronize(c->stream));
-  const int nrun = (int)c->hs_h[1];
-  long long launched = cg->m;
-  for (int k = 0; k < nrun; ++k) launched += cg->kernels[k];
+  const p4d_ctx::CycleGraph::Seg& sg = c->cyc[r.trans ? 1 : 0][r.full ? 1 : 0].seg[k0 / kSegSteps];
+  const int nrun = (int)c->hs_h[kGateRead + 1] - k0;
+  long long launched = 1;
+  for (int q = 0; q < nrun && q < (int)sg.kernels.size(); ++q) launched += sg.kernels[q];
   count_launches(launched);
-  if (nrun < 1) return P4D_ERR_CUDA;   // the first step always runs (limit >= 1, no stop)
-  const double s2[2] = {c->hs_h[2], c->hs_h[3]};
+  if (nrun < 1 || nrun > (int)sg.kernels.size()) return P4D_ERR_CUDA;   // the first step always runs (limit > k0, no stop)
   r.iters += nrun - 1;
-  fg_step_read(r, nrun - 1, s2);
+  fg_step_read(r, k0 + nrun - 1, c->hs_h + kGateRead + 2);
   return P4D_OK;
 }
 
@@ -895,33 +1152,59 @@ p4d_status fg_cycle_steps_graph(FgRun& r) {
 
 p4d_status fgmres(p4d_ctx* c, const double* b, double* x, p4d_info* info, int trans) {
   FgRun r;
+  const bool graph = !c->prm.profile;   // per-kernel events cannot sit inside a graph
   P4D_TRYS(fg_begin(r, c, b, x, trans));
-  P4D_TRY(cudaStreamSynchronize(c->stream));
-  P4D_TRYS(fg_bnorm(r));
-  while (r.active()) {
-    P4D_TRYS(fg_cycle_launch(r));
+  bool begun = false, finished = false;
+  if (!graph) {
     P4D_TRY(cudaStreamSynchronize(c->stream));
+    P4D_TRYS(fg_bnorm(r));
+    begun = true;
+  }
+  while (r.active()) {
+    // the first segment is launched before the host has seen the norms: the
+    // device gate makes the same tests and lets none of its steps run
+    // when there is nothing to solve
+    P4D_TRYS(fg_cycle_launch(r, graph));
+    if (graph) P4D_TRYS(fg_segment_launch(r, 0));
+    P4D_TRY(cudaStreamSynchronize(c->stream));
+    if (!begun) {
+      P4D_TRYS(fg_bnorm(r, true));
+      begun = true;
+      if (r.st == P4D_OK) {   // b_k = 0
+        r.restarts = 0;
+        break;
+      }
+    }
     fg_cycle_read(r);
     if (r.stop) break;
-    if (c->prm.profile) {
-      // per-kernel events cannot sit inside a graph: step by step
+    if (graph) {
+      P4D_TRYS(fg_segment_read(r, 0));
+      for (int k = kSegSteps; !r.cycle_done; k += kSegSteps) {
+        P4D_TRYS(fg_segment_launch(r, k));
+        P4D_TRY(cudaStreamSynchronize(c->stream));
+        P4D_TRYS(fg_segment_read(r, k));
+      }
+    } else {
       for (int k = 0; !r.cycle_done; ++k) {
-        P4D_TRYS(fg_step_body(r, k, true, nullptr));
+        P4D_TRYS(fg_step_body(r, k, true, Tail{}));
         P4D_TRY(cudaStreamSynchronize(c->stream));
         fg_step_read(r, k, c->hs_h);
       }
-    } else {
-      P4D_TRYS(fg_cycle_steps_graph(r));
     }
     P4D_TRYS(fg_cycle_end_launch(r));
     if (r.st == P4D_ERR_NONFINITE) break;
     if (r.st == P4D_OK) {
+      // the report's work runs with the confirmation (again when it fails)
+      P4D_TRYS(fg_finish_launch(r));
       P4D_TRY(cudaStreamSynchronize(c->stream));
       fg_cycle_end_read(r);
+      finished = r.st != P4D_ERR_NOT_CONVERGED;
     }
   }
-  P4D_TRYS(fg_finish_launch(r));
-  P4D_TRY(cudaStreamSynchronize(c->stream));
+  if (!finished) {
+    P4D_TRYS(fg_finish_launch(r));
+    P4D_TRY(cudaStreamSynchronize(c->stream));
+  }
   fg_finish_read(r, info);
   return r.st;
 }
@@ -949,7 +1232,9 @@ p4d_status batch_step_graph(p4d_batch_ctx* B, std::vector<FgRun>& R, int k, int 
     if (k >= r.m) continue;
     cudaGraph_t step = nullptr;
     long long kc = 0;
-    st = capture_body(r.c, &step, &kc, [&]() { return fg_step_body(r, k, false, B->stat_dev + 2 * i); });
+    Tail t;
+    t.stat = B->stat_dev + 2 * i;
+    st = capture_body(r.c, &step, &kc, [&]() { return fg_step_body(r, k, false, t); });
     if (st != P4D_OK) break;
     cudaGraphConditionalHandle h;
     cudaGraphNode_t kn = nullptr, cn = nullptr, ch = nullptr;
@@ -1119,9 +1404,9 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
   // field weights of the whole cell's right-hand side
   for (int p = 0; p < P; ++p) {
     p4d_ctx* c = D->parts[p];
-    ::p4d::count_launch(), k_field_norms<<<kRedBlocks, kRedThreads, 0, D->stream>>>(D->bw[p], c->rsqd, R[p].nn, c->ndof,
-                                                                                   c->part);
-    ::p4d::count_launch(), k_sum4<<<1, 128, 0, D->stream>>>(c->part, kRedBlocks, R[p].misc() + 2 * R[p].L.m + 8);
+    ::p4d::count_launch(), k_field_norms<<<norm_blocks(c->ndof), kRedThreads, 0, D->stream>>>(
+        D->bw[p], c->rsqd, R[p].nn, c->ndof, c->part, c->red_cnt, nullptr, 0.0, 0, nullptr, nullptr,
+        R[p].misc() + 2 * R[p].L.m + 8);
   }
   P4D_TRYS(reduce(at_off(2, 8), 4));
   for (int p = 0; p < P; ++p) {
@@ -1138,8 +1423,8 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
         c->g, c->nc, r.tau, c->eidx, c->label, c->Aj, c->Mj, c->betaj, c->ge, c->gc, c->gs, r.b, c->tmp + 3 * r.nn,
         c->bred, 0);
     r.bk = c->bred;
-    ::p4d::count_launch(), k_field_norms<<<kRedBlocks, kRedThreads, 0, D->stream>>>(r.bk, c->rsqd, r.nn, r.len, c->part);
-    ::p4d::count_launch(), k_sum4<<<1, 128, 0, D->stream>>>(c->part, kRedBlocks, r.misc() + 2 * r.L.m + 16);
+    ::p4d::count_launch(), k_field_norms<<<norm_blocks(r.len), kRedThreads, 0, D->stream>>>(
+        r.bk, c->rsqd, r.nn, r.len, c->part, c->red_cnt, nullptr, 0.0, 0, nullptr, nullptr, r.misc() + 2 * r.L.m + 16);
   }
   P4D_TRYS(reduce(at_off(2, 16), 4));
   P4D_TRY(cudaMemcpyAsync(c0->hs_h, r0.misc() + 2 * r0.L.m + 8, sizeof(double) * 12, cudaMemcpyDeviceToHost, D->stream));
@@ -1147,9 +1432,10 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
   for (int p = 0; p < P; ++p) {
     if (p > 0) std::memcpy(D->parts[p]->hs_h, c0->hs_h, sizeof(double) * 12);
     P4D_TRYS(fg_bnorm(R[p]));
+    P4D_TRY(cudaMemsetAsync(R[p].misc() + 2 * R[p].L.m + 7, 0, sizeof(double), D->stream));
   }
-  auto share_host = [&](int n) {
-    for (int p = 1; p < P; ++p) std::memcpy(D->parts[p]->hs_h, c0->hs_h, sizeof(double) * n);
+  auto share_host = [&](int at) {
+    for (int p = 1; p < P; ++p) D->parts[p]->hs_h[at] = c0->hs_h[at];
   };
   // V_0 = s.(b_k - J x), ||V_0|| and the true residual use the same sequence
   auto residual_norm = [&]() -> p4d_status {
@@ -1168,12 +1454,16 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
       FgRun& r = R[p];
       p4d_ctx* c = r.c;
       ++r.restarts;
-      ::p4d::count_launch(), k_init_cycle<<<1, 1, 0, D->stream>>>(c->hs, r.L, c->kdev);
-      ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(c->V, c->V, r.len, r.misc() + 2 * r.L.m + 5, 1);
+      Tail t;
+      t.mode = 1;
+      t.hs = c->hs;
+      t.L = r.L;
+      t.kdev = c->kdev;
+      ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(c->V, c->V, r.len, r.misc() + 2 * r.L.m + 2, t);
     }
-    P4D_TRY(cudaMemcpyAsync(c0->hs_h, r0.misc() + 2 * r0.L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, D->stream));
+    P4D_TRY(cudaMemcpyAsync(c0->hs_h + kBetaOff, r0.misc() + 2 * r0.L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, D->stream));
     P4D_TRY(cudaStreamSynchronize(D->stream));
-    share_host(1);
+    share_host(kBetaOff);
     for (int p = 0; p < P; ++p) fg_cycle_read(R[p]);
     if (r0.stop) break;
     for (int k = 0; !r0.cycle_done; ++k) {
@@ -1211,7 +1501,7 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
         p4d_ctx* c = D->parts[p];
         FgRun& r = R[p];
         Reducer{c}.maxpy(c->V, r.len, k + 1, r.misc(), c->V + (int64_t)(k + 1) * r.len, r.len, 1.0, nullptr,
-                         r.misc() + 2 * r.L.m + 2, r.gb);
+                         Reducer::norm_to(r.misc() + 2 * r.L.m + 2), r.gb);
       }
       P4D_TRYS(reduce(at_off(2, 2), 1));
       if (refine > 0) {
@@ -1229,11 +1519,8 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
           p4d_ctx* c = D->parts[p];
           FgRun& r = R[p];
           const double* flag = r.misc() + 2 * r.L.m + 6;
-          ::p4d::count_launch(), k_maxpy<<<r.gb, kBlock, 0, D->stream>>>(c->V, r.len, k + 1, r.misc() + r.L.m + 1,
-                                                                         c->V + (int64_t)(k + 1) * r.len, r.len, 1.0,
-                                                                         flag, c->part);
-          ::p4d::count_launch(), k_reduce_partials<<<1, 256, 0, D->stream>>>(c->part, (int)r.gb, 1, 1,
-                                                                             r.misc() + 2 * r.L.m + 44, flag, 1);
+          Reducer{c}.maxpy(c->V, r.len, k + 1, r.misc() + r.L.m + 1, c->V + (int64_t)(k + 1) * r.len, r.len, 1.0, flag,
+                           Reducer::norm_to(r.misc() + 2 * r.L.m + 44, 1), r.gb);
         }
         P4D_TRYS(reduce(at_off(2, 44), 1));
         for (int p = 0; p < P; ++p)
@@ -1245,8 +1532,8 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
         p4d_ctx* c = D->parts[p];
         FgRun& r = R[p];
         double* w = c->V + (int64_t)(k + 1) * r.len;
-        ::p4d::count_launch(), k_givens<<<1, 1, 0, D->stream>>>(c->hs, r.L, k, c->kdev, refine);
-        ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(w, w, r.len, r.misc() + 2 * r.L.m + 2, 2);
+        ::p4d::count_launch(), k_givens<<<1, 32, 0, D->stream>>>(c->hs, r.L, k, c->kdev, refine);
+        ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(w, w, r.len, r.misc() + 2 * r.L.m + 2, Tail{});
       }
       P4D_TRY(cudaMemcpyAsync(c0->hs_h, r0.misc() + 2 * r0.L.m + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                               D->stream));
@@ -1258,17 +1545,17 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
       FgRun& r = R[p];
       p4d_ctx* c = r.c;
       if (r.kk > 0) {
-        ::p4d::count_launch(), k_backsolve<<<1, 1, 0, D->stream>>>(c->hs, r.L, r.kk);
-        Reducer{c}.maxpy(c->Z, r.len, r.kk, c->hs + r.L.y, r.x, r.len, -1.0, nullptr, nullptr, r.gb);
+        ::p4d::count_launch(), k_backsolve<<<1, 32, 0, D->stream>>>(c->hs, r.L, r.kk);
+        Reducer{c}.maxpy(c->Z, r.len, r.kk, c->hs + r.L.y, r.x, r.len, -1.0, nullptr, Fin{}, r.gb);
       }
     }
     if (r0.st == P4D_ERR_NONFINITE) break;
     if (r0.st == P4D_OK) {
       P4D_TRYS(residual_norm());
-      P4D_TRY(cudaMemcpyAsync(c0->hs_h, r0.misc() + 2 * r0.L.m + 2, sizeof(double), cudaMemcpyDeviceToHost,
+      P4D_TRY(cudaMemcpyAsync(c0->hs_h + kTrueOff, r0.misc() + 2 * r0.L.m + 2, sizeof(double), cudaMemcpyDeviceToHost,
                               D->stream));
       P4D_TRY(cudaStreamSynchronize(D->stream));
-      share_host(1);
+      share_host(kTrueOff);
       for (int p = 0; p < P; ++p) fg_cycle_end_read(R[p]);
     }
   }
@@ -1287,12 +1574,8 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
     double* m = r.misc() + 2 * r.L.m;
     P4D_TRYS(jvp_full(c, r.x, c->r0, 0, r.b, true));
     P4D_TRYS(dd_zero_ghost(D, p, c->r0, true));
-    ::p4d::count_launch(), k_field_norms_plain<<<kRedBlocks, kRedThreads, 0, D->stream>>>(c->r0, r.nn, c->ndof, c->part);
-    ::p4d::count_launch(), k_sum4<<<1, 128, 0, D->stream>>>(c->part, kRedBlocks, m + 24);
-    ::p4d::count_launch(), k_field_norms<<<kRedBlocks, kRedThreads, 0, D->stream>>>(c->r0, c->sqd, r.nn, c->ndof, c->part);
-    ::p4d::count_launch(), k_sum4<<<1, 128, 0, D->stream>>>(c->part, kRedBlocks, m + 32);
-    ::p4d::count_launch(), k_field_norms_plain<<<kRedBlocks, kRedThreads, 0, D->stream>>>(r.b, r.nn, c->ndof, c->part);
-    ::p4d::count_launch(), k_sum4<<<1, 128, 0, D->stream>>>(c->part, kRedBlocks, m + 36);
+    ::p4d::count_launch(), k_final_norms<<<norm_blocks(c->ndof), kRedThreads, 0, D->stream>>>(
+        c->r0, c->sqd, r.b, r.nn, c->ndof, c->part, c->red_cnt, m + 24);
   }
   P4D_TRYS(reduce(at_off(2, 24), 4));
   P4D_TRYS(reduce(at_off(2, 32), 8));

@@ -236,7 +236,8 @@ struct p4d_ctx {
   double* r0 = nullptr;                // [ndof]
   double* tmp = nullptr;               // [ndof]
   double* bred = nullptr;              // [ndof] reduced right-hand side / scratch
-  double* part = nullptr;              // [nparts][kry dots] partial sums
+  double* part = nullptr;              // block partial sums of a reduction
+  unsigned* red_cnt = nullptr;         // blocks of the running reduction that have finished (0 between launches)
   double* hs = nullptr;                // device Hessenberg / Givens state
   double* hs_h = nullptr;              // pinned host mirror of small scalars
 
@@ -253,13 +254,16 @@ struct p4d_ctx {
     cudaGraphExec_t exec = nullptr;
     long long kernels = 0;             // kernel nodes (added to the launch counter per launch)
   } pcg[2][2];
-  // One FGMRES restart cycle as one graph, [transpose][full]: Arnoldi step k
-  // inside a conditional (IF) node whose condition a one-thread kernel sets
-  // from the device gate (no stop yet, k below the cycle's step limit).
+  // An FGMRES restart cycle as graphs of a few Arnoldi steps each
+  // (segments, captured at first use), [transpose][full]: step k inside a
+  // conditional (IF) node whose condition the step before sets.
   struct CycleGraph {
-    cudaGraphExec_t exec = nullptr;
-    int m = 0;                         // steps in the graph
-    std::vector<long long> kernels;    // kernel launches of step k (gate kernels not included)
+    struct Seg {
+      cudaGraphExec_t exec = nullptr;
+      std::vector<long long> kernels;  // kernel launches of each of its steps (the gate kernel not included)
+    };
+    std::vector<Seg> seg;
+    int m = 0;                         // restart length of the segments
   } cyc[2][2];
   unsigned graph_gen = 0;              // incremented whenever the captured graphs are dropped
   cudaStream_t cap_stream = nullptr;

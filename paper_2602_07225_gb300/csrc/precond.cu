@@ -420,10 +420,10 @@ void drop_graphs(p4d_ctx* c) {
     for (auto& g : row) drop(g);
   for (auto& row : c->cyc)
     for (auto& g : row) {
-      if (g.exec) cudaGraphExecDestroy(g.exec);
-      g.exec = nullptr;
+      for (auto& sg : g.seg)
+        if (sg.exec) cudaGraphExecDestroy(sg.exec);
+      g.seg.clear();
       g.m = 0;
-      g.kernels.clear();
     }
 }
 
