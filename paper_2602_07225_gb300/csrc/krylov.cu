@@ -89,6 +89,25 @@ __device__ __forceinline__ double warp_sum(const double* p, int n, int lane) {
   return s;
 }
 
+// Sum of p[0..n) by one warp in the order of a 256-thread block (thread t
+// sums p[t], p[t + 256], ..., then a halving tree): lane l holds threads l,
+// l + 32, ..., l + 224.  Lane 0 has the result.
+__device__ __forceinline__ double warp_tree_sum(const double* p, int n, int lane) {
+  double s[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    s[q] = 0.0;
+    for (int b = lane + 32 * q; b < n; b += 256) s[q] += __ldcg(p + b);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) s[q] += s[q + 4];
+  s[0] += s[2];
+  s[1] += s[3];
+  double t = s[0] + s[1];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  return t;
+}
+
 // out[g0 + i] = V_{g0+i} . w (i < NG), out[kp1] = w . w (WW), summed over the
 // blocks by the last one.  flag (optional): skipped when *flag == 0, out
 // then zeroed (zero_if_skipped) or left as it is.
@@ -151,7 +170,7 @@ __global__ void __launch_bounds__(kRedThreads) k_mdot(const double* __restrict__
   }
   if (!last_block(cnt)) return;
   for (int i = warp; i < NA; i += kRedThreads / 32) {
-    const double sum = warp_sum(partial + (int64_t)i * kRedBlocks, gridDim.x, lane);
+    const double sum = warp_tree_sum(partial + (int64_t)i * kRedBlocks, gridDim.x, lane);
     if (lane == 0) out[i < NG ? g0 + i : kp1] = sum;
   }
 }
@@ -317,15 +336,21 @@ __global__ void __launch_bounds__(kBlock) k_maxpy(const double* __restrict__ V, 
     partial[blockIdx.x] = t;
   }
   if (!last_block(cnt)) return;
-  // each warp sums every eighth run of 32 partials; then the warps in order
+  // strided sums per thread, then a halving tree over the 256 threads
   double t = 0.0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) t += __ldcg(partial + b);
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __shared__ double tree[kBlock];
+  tree[threadIdx.x] = t;
   __syncthreads();
+  for (int off = kBlock / 2; off >= 32; off >>= 1) {
+    if ((int)threadIdx.x < off) tree[threadIdx.x] += tree[threadIdx.x + off];
+    __syncthreads();
+  }
+  if (threadIdx.x < 32) {
+    t = tree[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  }
   if (threadIdx.x == 0) {
-    t = 0.0;
-    for (int i = 0; i < kBlock / 32; ++i) t += red[i];
     *fin.norm = t;
     if (fin.mode == kFinReorth) reorth_test(fin.hs, fin.L, fin.k, fin.eta2);
   }
@@ -557,36 +582,41 @@ __global__ void k_reorth_flag(double* hs, HLay L, int k, double eta2) {
   if (threadIdx.x == 0) reorth_test(hs, L, k, eta2);
 }
 
-// H y = g by one warp, column by column from the last: lane j keeps rows
-// j, j + 32, ... of g; the diagonal's reciprocals are formed side by side
-// (a serial row-wise substitution took 24 us at 13 columns).
+// H y = g by one warp, row by row from the last: the lanes load the next row
+// (strided: columns are contiguous) while lane 0 runs the current row's
+// dependent chain out of shared memory.  With lane 0 loading for itself the
+// substitution took 24 us at 13 columns.
 __global__ void __launch_bounds__(32) k_backsolve(double* hs, HLay L, int kk) {
+  __shared__ double row[2][130], y[130];
   const int lane = threadIdx.x, ld = L.m + 1;
   const double* H = hs + L.H;
-  double g[4], rd[4], nx[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = lane + 32 * q;
-    g[q] = i < kk ? hs[L.g + i] : 0.0;
-    const double d = i < kk ? H[(int64_t)i * ld + i] : 0.0;
-    rd[q] = d != 0.0 ? 1.0 / d : 0.0;
-    nx[q] = i < kk - 1 ? H[(int64_t)(kk - 1) * ld + i] : 0.0;
-  }
+  for (int j = kk - 1 + lane; j < kk; j += 32) row[(kk - 1) & 1][j] = H[(int64_t)j * ld + kk - 1];
+  double gi = lane == 0 ? hs[L.g + kk - 1] : 0.0;
+  __syncwarp();
   for (int i = kk - 1; i >= 0; --i) {
-    double c[4];
+    double nx[4], gn = 0.0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      c[q] = nx[q];
-      const int j = lane + 32 * q;
-      nx[q] = j < i - 1 ? H[(int64_t)(i - 1) * ld + j] : 0.0;   // the next column's load is in flight
+      const int j = i - 1 + lane + 32 * q;
+      nx[q] = i > 0 && j < kk ? H[(int64_t)j * ld + i - 1] : 0.0;
     }
-    const int iq = i >> 5;
-    const double mine = iq == 0 ? g[0] * rd[0] : (iq == 1 ? g[1] * rd[1] : (iq == 2 ? g[2] * rd[2] : g[3] * rd[3]));
-    const double y = __shfl_sync(0xffffffffu, mine, i & 31);
-    if (lane == 0) hs[L.y + i] = y;
+    if (lane == 0) {
+      if (i > 0) gn = hs[L.g + i - 1];
+      const double* r = row[i & 1];
+      double s = gi;
+      for (int j = i + 1; j < kk; ++j) s -= r[j] * y[j];
+      const double d = r[i];
+      y[i] = d != 0.0 ? s / d : 0.0;
+      gi = gn;
+    }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) g[q] -= c[q] * y;   // rows j >= i: c = 0
+    for (int q = 0; q < 4; ++q) {
+      const int j = i - 1 + lane + 32 * q;
+      if (i > 0 && j < kk) row[(i - 1) & 1][j] = nx[q];
+    }
+    __syncwarp();
   }
+  for (int i = lane; i < kk; i += 32) hs[L.y + i] = y[i];
 }
 
 // Reduced-mode condensation / back-substitution helpers (per node).
@@ -640,13 +670,18 @@ __global__ void k_surface_coupling(int64_t NE, double tau, const int32_t* __rest
   }
 }
 
+// Vectors up to the size of a cell whose whole V-cycle is one launch (8,192
+// nodes, three fields) are partitioned finer: their kernels are latency
+// bound.  Above it the sums keep one partition at every size.
+constexpr int64_t kSmallLen = 3 * 8192;
+
 struct Reducer {
   p4d_ctx* c;
-  // one element per thread and trip on small vectors (a block per 512
-  // elements: eight per thread left 3 blocks at 6,075 elements and 14 us),
-  // kRedBlocks blocks on large ones
+  // eight elements per thread; on the smallest vectors two (eight left 3
+  // blocks at 6,075 elements and 14 us per multi-dot)
   int nblk(int64_t len) const {
-    const int64_t want = (len + (int64_t)kRedThreads * 2 - 1) / ((int64_t)kRedThreads * 2);
+    const int64_t per = (int64_t)kRedThreads * (len <= kSmallLen ? 2 : 8);
+    const int64_t want = (len + per - 1) / per;
     return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, want));
   }
   // out[0..kp1) = V^T w, out[kp1] = w.w (optional)
@@ -697,9 +732,10 @@ struct Reducer {
   }
 };
 
-// Blocks of a sum over len entries (four per thread and trip).
+// Blocks of a sum over len entries: four per thread on the smallest vectors
+// (608 blocks took 13 us for 24 k entries, mostly in the last sum).
 inline int norm_blocks(int64_t len) {
-  return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, len / (4 * kRedThreads)));
+  return len <= 4 * kSmallLen ? (int)std::max<int64_t>(1, len / (4 * kRedThreads)) : kRedBlocks;
 }
 
 }  // namespace

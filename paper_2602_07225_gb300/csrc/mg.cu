@@ -750,7 +750,7 @@ __device__ __forceinline__ void stencil_rows(const TS* __restrict__ st, const T*
       if (9 * pz + t == 13) continue;
 #pragma unroll
       for (int q = 0; q < kNpt; ++q)
-        if (on[q]) ax[q] += (T)tof(sv[t][q]) * (xv[t][q] - xn[q]);
+        if (on[q]) ax[q] = fma((T)tof(sv[t][q]), xv[t][q] - xn[q], ax[q]);
     }
   }
 }
@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(256) k_cheb(LevelDims dd, LvlPtrs<TS, T> P, HL
     T res = bq[q];
     if (!first) res -= ax[q];
     const T z = iq[q] * res;
-    const T dn = step == 0 ? c0 * z : ca * dq[q] + cb * z;
+    const T dn = step == 0 ? c0 * z : fma(cb, z, ca * dq[q]);   // contraction as in k_tail
     d[m] = dn;
     xo[m] = (first ? (T)0 : x[m]) + dn;
   }
@@ -1017,8 +1017,9 @@ __global__ void __launch_bounds__(32 * kCoarseWarps) k_coarse_solve(int n, const
 // most kTailThreads rows runs on the first block alone (block barriers); the
 // coarsest dense solve, FP64 and bound by the FP64 rate of an SM, is spread
 // over the cluster.  Only the x of level l0 goes back to global memory.  Per
-// row the arithmetic and its order are those of k_cheb, k_resid, k_restrict,
-// k_prolong and k_coarse_solve.
+// row the arithmetic, its order and its contractions are those of k_cheb,
+// k_resid, k_restrict, k_prolong and k_coarse_solve: the results are
+// bit-identical to the level-by-level cycle's.
 constexpr int kTailThreads = 512;
 constexpr int kTailMaxCluster = 16;
 // Rows per block before a level takes another block of the cluster: one per
@@ -1175,9 +1176,9 @@ __device__ __forceinline__ void row_coef(const void* st, int N, int n, T (&c)[27
 }
 template <typename T>
 __device__ __forceinline__ T row_apply(const T (&c)[27], const T* x, int sy, int sz, int n, T xn) {
-  T ax = c[13] * xn;
+  T ax = fma(c[0], x[n - 1 - sy - sz] - xn, c[13] * xn);
 #pragma unroll
-  for (int o = 0; o < 27; ++o)
+  for (int o = 1; o < 27; ++o)
     if (o != 13) ax += c[o] * (x[n + (o % 3 - 1) + ((o / 3) % 3 - 1) * sy + (o / 9 - 1) * sz] - xn);
   return ax;
 }
@@ -1320,7 +1321,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
         if (s < a.deg) {
           const T z = iq * res;
           const T* cf = ch + (q * a.deg + s) * 3;
-          dq = s == 0 ? cf[0] * z : cf[1] * dq + cf[2] * z;
+          dq = s == 0 ? cf[0] * z : fma(cf[2], z, cf[1] * dq);
           xq += dq;
           val = xq;
         }
