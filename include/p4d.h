@@ -139,7 +139,8 @@ typedef struct {
                            refinement), 1 when the first pass leaves ||w|| < 0.7 ||w_0||
                            (default), 2 always */
   int32_t mf_zchunk;    /* node planes per block of the matrix-free level-0 kernel (the
-                           z depth of its tile; 0 = 8, at most 64).  Fixed at p4d_setup */
+                           z depth of its tile; 0 = by the cell's size, at most 64; the
+                           results do not depend on it).  Fixed at p4d_setup */
 } p4d_params;
 
 /* A linearization state.  All [device], FP64; cs / cs_prev are [nelec][nc]. */

@@ -194,8 +194,12 @@ __device__ inline bool kinetics(const Kin& kn, int et, double phis, double phie,
   return true;
 }
 
+// With ue: also the inputs of the residual's stencils, ue = phi_e + gamma ln
+// c_e and dce = c_e - c_e_prev (formed per node instead of per neighbour).
 __global__ void k_node_ln(int64_t nn, const double* __restrict__ ce, double gamma, double* __restrict__ lnce,
-                          double* __restrict__ gdc, unsigned* flags) {
+                          double* __restrict__ gdc, const double* __restrict__ phie,
+                          const double* __restrict__ ce_prev, double* __restrict__ ue, double* __restrict__ dce,
+                          unsigned* flags) {
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= nn) return;
   const double c = ce[n];
@@ -205,7 +209,12 @@ __global__ void k_node_ln(int64_t nn, const double* __restrict__ ce, double gamm
     if (gdc) gdc[n] = 0.0;
     return;
   }
-  lnce[n] = log(c);
+  const double l = log(c);
+  lnce[n] = l;
+  if (ue) {
+    ue[n] = fma(gamma, l, phie[n]);
+    dce[n] = c - ce_prev[n];
+  }
   if (gdc) gdc[n] = gamma / c;
 }
 
@@ -343,36 +352,22 @@ __global__ void k_fixed_sums(Grid g, const double* __restrict__ Jst, const uint8
   }
 }
 
-template <typename F>
-__device__ inline double stencil_apply(const double* __restrict__ st, int64_t nn, const Grid& g, int64_t n,
-                                       int i, int j, int k, F val) {
-  double acc = 0.0;
-#pragma unroll
-  for (int o = 0; o < 27; ++o) {
-    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    const int ii = i + dx, jj = j + dy, kk = k + dz;
-    if (ii < 0 || jj < 0 || kk < 0 || ii >= g.nnx || jj >= g.nny || kk >= g.nnz) continue;
-    const int64_t m = n + dx + (int64_t)g.nnx * (dy + (int64_t)g.nny * dz);
-    acc += st[o * nn + n] * val(m);
-  }
-  return acc;
-}
-
-// Nonlinear residual (paper section 4, block residual) -- macro rows.
-__global__ void k_residual_macro(Grid g, Kin kn, const double* __restrict__ Jst,
+// Nonlinear residual (paper section 4, block residual) -- macro rows.  Every
+// neighbour is loaded without a test, as in k_jvp_macro: the stencils hold
+// exact zeros for neighbours outside the grid and, for phi_s, without an
+// unknown.
+__global__ void __launch_bounds__(128) k_residual_macro(Grid g, Kin kn, const double* __restrict__ Jst,
                                  const uint8_t* __restrict__ label, const int32_t* __restrict__ eidx,
                                  const double* __restrict__ Aj, const double* __restrict__ gpw,
-                                 const double* __restrict__ phis, const double* __restrict__ phie,
-                                 const double* __restrict__ ce, const double* __restrict__ ce_prev,
-                                 const double* __restrict__ lnce, const double* __restrict__ rin,
+                                 const double* __restrict__ phis, const double* __restrict__ ue,
+                                 const double* __restrict__ ce, const double* __restrict__ dce,
+                                 const double* __restrict__ rin,
                                  const double* __restrict__ sfix, const double* __restrict__ trows,
                                  double* __restrict__ r) {
-  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;   // 27 nn < 2^31 (checked at setup)
   const int64_t nn = g.nn;
-  if (n >= nn) return;
-  const int i = (int)(n % g.nnx);
-  const int j = (int)((n / g.nnx) % g.nny);
-  const int k = (int)(n / ((int64_t)g.nnx * g.nny));
+  const int N = (int)nn;
+  if (n >= N) return;
   const int32_t e = eidx[n];
   const double ain = e >= 0 ? Aj[e] * rin[e] : 0.0;
   const bool act = label[n] & kLabActive;
@@ -381,46 +376,49 @@ __global__ void k_residual_macro(Grid g, Kin kn, const double* __restrict__ Jst,
   // of the lifted stencil (exactly 0 where no coupling was dropped): the
   // collector-shell rows couple nodes whose potentials agree to microvolts
   // through conductances ~1e7 times the bulk ones, and the standard form
-  // would leave rounding of those large products in the residual
-  if (act) {
-    const double* Ks = Jst;
-    const double pn = phis[n];
-    double s = sfix[n] * pn;
+  // would leave rounding of those large products in the residual.
+  // c_e: mass part on (c_e - c_e_prev), diffusion part (C - M_eps/dt) on c_e:
+  // no cancellation between the two time levels.  Transport rows: the fixed
+  // stencils, or (concentration-dependent coefficients) the element
+  // integrals at this state, trows[0..1][n]
+  const double* Ks = Jst;
+  const double* Kk = Jst + 1 * 27 * nn;
+  const double* Cc = Jst + 2 * 27 * nn;
+  const double* Mm = Jst + 3 * 27 * nn;
+  const double pn = phis[n];
+  double s = act ? sfix[n] * pn : 0.0, se = 0.0, sc = 0.0;
 #pragma unroll
-    for (int o = 0; o < 27; ++o) {
-      if (o == 13) continue;
-      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-      const int ii = i + dx, jj = j + dy, kk = k + dz;
-      if (ii < 0 || jj < 0 || kk < 0 || ii >= g.nnx || jj >= g.nny || kk >= g.nnz) continue;
-      const int64_t m = n + dx + (int64_t)g.nnx * (dy + (int64_t)g.nny * dz);
-      if (label[m] & kLabActive) s += Ks[o * nn + n] * (phis[m] - pn);
+  for (int l = 0; l < 9; ++l) {
+    const int mid = n + g.nnx * ((l % 3 - 1) + g.nny * (l / 3 - 1));
+    double ks[3], kk[3], cc[3], mm[3], vs[3], vu[3], vc[3], vd[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int o = 3 * l + d;
+      const int m = min(max(mid + d - 1, 0), N - 1);
+      if (act) {
+        ks[d] = Ks[o * N + n];
+        vs[d] = phis[m];
+      }
+      mm[d] = Mm[o * N + n];
+      vd[d] = dce[m];
+      if (!trows) {
+        kk[d] = Kk[o * N + n];
+        vu[d] = ue[m];
+        cc[d] = Cc[o * N + n];
+        vc[d] = ce[m];
+      }
     }
-    r[n] = s + ain - kn.i_app * gpw[n];
-  } else {
-    r[n] = phis[n];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (act && 3 * l + d != 13) s += ks[d] * (vs[d] - pn);
+      if (!trows) se += kk[d] * vu[d];
+      const double mo = mm[d];
+      sc += mo * vd[d] + (trows ? 0.0 : (cc[d] - mo) * vc[d]);
+    }
   }
-  // transport rows: the fixed stencils, or (concentration-dependent
-  // coefficients) the element integrals at this state, trows[0..1][n]
-  const double se = trows ? trows[n]
-                          : stencil_apply(Jst + 1 * 27 * nn, nn, g, n, i, j, k,
-                                          [&](int64_t m) { return phie[m] + kn.gamma * lnce[m]; });
+  r[n] = act ? s + ain - kn.i_app * gpw[n] : pn;
+  if (trows) se = trows[n];
   r[nn + n] = se - ain;
-  // mass part on (c_e - c_e_prev), diffusion part (C - M_eps/dt) on c_e: no cancellation between
-  // the two time levels
-  double sc = 0.0;
-  {
-    const double* Cc = Jst + 2 * 27 * nn;
-    const double* Mm = Jst + 3 * 27 * nn;
-#pragma unroll
-    for (int o = 0; o < 27; ++o) {
-      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-      const int ii = i + dx, jj = j + dy, kk = k + dz;
-      if (ii < 0 || jj < 0 || kk < 0 || ii >= g.nnx || jj >= g.nny || kk >= g.nnz) continue;
-      const int64_t m = n + dx + (int64_t)g.nnx * (dy + (int64_t)g.nny * dz);
-      const double mo = Mm[o * nn + n];
-      sc += mo * (ce[m] - ce_prev[m]) + (trows ? 0.0 : (Cc[o * nn + n] - mo) * ce[m]);
-    }
-  }
   if (trows) sc += trows[nn + n];
   r[2 * nn + n] = sc - kn.tau * ain;
 }
@@ -511,7 +509,7 @@ p4d_status linearize(p4d_ctx* c, const p4d_state* st) {
   const int nc = c->nc;
   Kin kn = make_kin(c->prm);
   P4D_TRY(cudaMemsetAsync(c->flags, 0, sizeof(unsigned), c->stream));
-  ::p4d::count_launch(), k_node_ln<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, st->ce, kn.gamma, c->lnce, c->gdc, c->flags);
+  ::p4d::count_launch(), k_node_ln<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, st->ce, kn.gamma, c->lnce, c->gdc, nullptr, nullptr, nullptr, nullptr, c->flags);
   P4D_TRYS(transport_linearize(c, st));   // K_kappa, C at the state (transport_model 1)
   if (NE > 0)
     ::p4d::count_launch(), k_linearize<<<nblocks(NE), kBlock, 0, c->stream>>>(NE, nc, kn, c->enode, c->label, c->etype,
@@ -533,14 +531,16 @@ p4d_status residual(p4d_ctx* c, const p4d_state* st, double* r) {
   const int nc = c->nc;
   Kin kn = make_kin(c->prm);
   P4D_TRY(cudaMemsetAsync(c->flags, 0, sizeof(unsigned), c->stream));
-  ::p4d::count_launch(), k_node_ln<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, st->ce, kn.gamma, c->lnce_r, nullptr, c->flags);
+  ::p4d::count_launch(), k_node_ln<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, st->ce, kn.gamma, c->lnce_r, nullptr, st->phie,
+                                                                 st->ce_prev, c->ue_r, c->dce_r, c->flags);
   if (NE > 0)
     ::p4d::count_launch(), k_kinetics_only<<<nblocks(NE), kBlock, 0, c->stream>>>(NE, nc, kn, c->enode, c->label, c->etype, st->phis,
                                                             st->phie, st->ce, st->cs, c->rin, c->flags);
   const double* trows = transport_residual_rows(c, st, c->lnce_r);
-  ::p4d::count_launch(), k_residual_macro<<<nblocks(nn, 128), 128, 0, c->stream>>>(c->g, kn, c->Jst, c->label, c->eidx, c->Aj, c->gpw,
-                                                             st->phis, st->phie, st->ce, st->ce_prev,
-                                                             c->lnce_r, c->rin, c->sfix, trows, r);
+  int bt = 128;   // as the Jacobian product's rows (jvp.cu)
+  while (bt > 32 && nn < (int64_t)2 * 152 * bt) bt /= 2;
+  ::p4d::count_launch(), k_residual_macro<<<nblocks(nn, bt), bt, 0, c->stream>>>(c->g, kn, c->Jst, c->label, c->eidx, c->Aj, c->gpw,
+                                                             st->phis, c->ue_r, st->ce, c->dce_r, c->rin, c->sfix, trows, r);
   if (NE > 0)
     ::p4d::count_launch(), k_residual_particle<<<nblocks(NE * nc), kBlock, 0, c->stream>>>(NE, nc, 1.0 / c->prm.dt, st->cs, st->cs_prev, c->Mj,
                                                                     c->kapj, c->betaj, c->rref, c->rin,

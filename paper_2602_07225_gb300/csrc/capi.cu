@@ -275,6 +275,8 @@ p4d_status setup_impl(p4d_ctx* c, const p4d_mesh* m, const p4d_params* prm) {
   // ---- linearization workspace
   P4D_TRYS(dalloc_t(c, &c->lnce, nn));
   P4D_TRYS(dalloc_t(c, &c->lnce_r, nn));
+  P4D_TRYS(dalloc_t(c, &c->ue_r, nn));
+  P4D_TRYS(dalloc_t(c, &c->dce_r, nn));
   P4D_TRYS(dalloc_t(c, &c->rin, NE));
   P4D_TRYS(dalloc_t(c, &c->gdc, nn));
   P4D_TRYS(dalloc_t(c, &c->in_, NE));

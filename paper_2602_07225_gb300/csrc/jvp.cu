@@ -45,16 +45,18 @@ __global__ void k_jvp_combine(int64_t nn, const double* __restrict__ x, const do
 }
 
 // Macro rows.  reduced: Schur operator on [phi_s | phi_e | c_e] only.
+// Large cells are bound by the FP64 rate, small ones by the latency of the
+// loads: every neighbour is loaded without a test (the stencils hold exact
+// zeros in the slots of neighbours outside the grid, the index is clamped to
+// the vector), one stencil line of three offsets at a time.
 template <bool TRANS, bool REDUCED>
 __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __restrict__ x,
                                                    const double* __restrict__ b, double* __restrict__ y,
                                                    bool scaled) {
   const int64_t nn = a.g.nn;
-  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (n >= nn) return;
-  const int i = (int)(n % a.g.nnx);
-  const int j = (int)((n / a.g.nnx) % a.g.nny);
-  const int k = (int)(n / ((int64_t)a.g.nnx * a.g.nny));
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;   // 27 nn < 2^31 (checked at setup)
+  const int N = (int)nn;
+  if (n >= N) return;
   const double* xs = x;
   const double* xe = x + nn;
   const double* xc = x + 2 * nn;
@@ -63,18 +65,32 @@ __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __re
   const double* Cc = a.Jst + 2 * 27 * nn;
   double ys = 0.0, ye = 0.0, yc = 0.0;
   const bool act = a.label[n] & kLabActive;
+  const double* ue = !TRANS && a.u ? a.u : xe;
+  const bool comb = !TRANS && !a.u;
 #pragma unroll
-  for (int o = 0; o < 27; ++o) {
-    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-    const int ii = i + dx, jj = j + dy, kk = k + dz;
-    if (ii < 0 || jj < 0 || kk < 0 || ii >= a.g.nnx || jj >= a.g.nny || kk >= a.g.nnz) continue;
-    const int64_t m = n + dx + (int64_t)a.g.nnx * (dy + (int64_t)a.g.nny * dz);
-    const int64_t so = o * nn + n;
-    if (act) ys += Ks[so] * xs[m];
-    const double kk_ = Kk[so];
-    if (!TRANS) ye += kk_ * (a.u ? a.u[m] : fma(a.gdc[m], xc[m], xe[m]));
-    else ye += kk_ * xe[m];
-    yc += Cc[so] * xc[m];
+  for (int l = 0; l < 9; ++l) {
+    const int mid = n + a.g.nnx * ((l % 3 - 1) + a.g.nny * (l / 3 - 1));
+    double k0[3], k1[3], k2[3], v0[3], v1[3], v2[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int o = 3 * l + d;
+      const int m = min(max(mid + d - 1, 0), N - 1);
+      k1[d] = Kk[o * N + n];
+      k2[d] = Cc[o * N + n];
+      v1[d] = ue[m];
+      v2[d] = xc[m];
+      if (comb) v1[d] = fma(a.gdc[m], v2[d], v1[d]);
+      if (act) {
+        k0[d] = Ks[o * N + n];
+        v0[d] = xs[m];
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (act) ys += k0[d] * v0[d];
+      ye += k1[d] * v1[d];
+      yc += k2[d] * v2[d];
+    }
   }
   if (TRANS) yc += a.gdc[n] * ye;   // (K_kappa diag(gamma/c_e))^T = diag(gamma/c_e) K_kappa
   if (!act) ys = xs[n];
@@ -154,15 +170,35 @@ JvpArgs make_args(p4d_ctx* c) {
 
 }  // namespace
 
-p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled) {
+// The input combination phi_e + gamma/c_e c_e: already in c->ujvp (u_ready:
+// the preconditioner's store left it there), formed per node, or on small
+// cells (latency: one launch less) inside the stencil loop; the values are
+// the same.
+static void jvp_input(p4d_ctx* c, JvpArgs& a, const double* x, bool u_ready) {
+  const int64_t nn = c->g.nn;
+  if (!u_ready && nn <= 8192) return;
+  if (!u_ready)
+    ::p4d::count_launch(), k_jvp_combine<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, x, c->gdc, c->ujvp);
+  a.u = c->ujvp;
+}
+
+// Threads per block of the macro rows: 128, fewer while that leaves SMs
+// without a block (the rows of a block share an SM's FP64 units; the reduced
+// product of 2,025 nodes took 17 us with 128 and its own combination pass,
+// 11 us with 32, launch gaps included).
+static int jvp_threads(int64_t nn) {
+  int t = 128;
+  while (t > 32 && nn < (int64_t)2 * 152 * t) t /= 2;
+  return t;
+}
+
+p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled, bool u_ready) {
   JvpArgs a = make_args(c);
   const int64_t nn = c->g.nn;
-  if (!transpose) {
-    ::p4d::count_launch(), k_jvp_combine<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, x, c->gdc, c->ujvp);
-    a.u = c->ujvp;
-  }
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, 128), 128, 0, c->stream>>>(a, x, b, y, scaled);
-  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, 128), 128, 0, c->stream>>>(a, x, b, y, scaled);
+  const int bt = jvp_threads(nn);
+  if (!transpose) jvp_input(c, a, x, u_ready);
+  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
+  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
   if (c->NE > 0) {
     const int64_t np = c->NE * c->nc;
     if (transpose) ::p4d::count_launch(), k_jvp_particle<true><<<nblocks(np), kBlock, 0, c->stream>>>(a, x, b, y, scaled);
@@ -173,15 +209,14 @@ p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const
   return P4D_OK;
 }
 
-p4d_status jvp_reduced(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled) {
+p4d_status jvp_reduced(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled,
+                       bool u_ready) {
   JvpArgs a = make_args(c);
   const int64_t nn = c->g.nn;
-  if (!transpose) {
-    ::p4d::count_launch(), k_jvp_combine<<<nblocks(nn), kBlock, 0, c->stream>>>(nn, x, c->gdc, c->ujvp);
-    a.u = c->ujvp;
-  }
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, true><<<nblocks(nn, 128), 128, 0, c->stream>>>(a, x, b, y, scaled);
-  else ::p4d::count_launch(), k_jvp_macro<false, true><<<nblocks(nn, 128), 128, 0, c->stream>>>(a, x, b, y, scaled);
+  const int bt = jvp_threads(nn);
+  if (!transpose) jvp_input(c, a, x, u_ready);
+  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
+  else ::p4d::count_launch(), k_jvp_macro<false, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
   P4D_TRYS(transport_jvp(c, x, y, transpose, b, scaled));
   P4D_TRY(cudaGetLastError());
   return P4D_OK;
@@ -240,8 +275,8 @@ extern "C" p4d_status p4d_jvp_noalloc(p4d_handle h, const double* x, double* y, 
   JvpArgs a = make_args(h);
   a.tloc = tloc;   // each entry read by the particle rows is written first by the macro rows
   const int64_t nn = h->g.nn;
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, 128), 128, 0, h->stream>>>(a, x, nullptr, y, false);
-  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, 128), 128, 0, h->stream>>>(a, x, nullptr, y, false);
+  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
+  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
   if (h->NE > 0) {
     const int64_t np = h->NE * h->nc;
     if (transpose) ::p4d::count_launch(), k_jvp_particle<true><<<nblocks(np), kBlock, 0, h->stream>>>(a, x, nullptr, y, false);

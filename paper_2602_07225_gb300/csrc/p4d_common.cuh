@@ -177,6 +177,8 @@ struct p4d_ctx {
   // linearization
   double* lnce = nullptr;              // [nn] ln c_e
   double* lnce_r = nullptr;            // [nn] ln c_e at the state of a residual evaluation
+  double* ue_r = nullptr;              // [nn] phi_e + gamma ln c_e there
+  double* dce_r = nullptr;             // [nn] c_e - c_e_prev there
   double* rin = nullptr;               // [NE] i_n at the state of a residual evaluation
   double* gdc = nullptr;               // [nn] gamma / c_e
   double* in_ = nullptr;               // [NE] reaction current
@@ -439,10 +441,11 @@ p4d_status check_flags(p4d_ctx* c);
 
 // ---- operator application (jvp.cu)
 // y[i] = sc_out[i] * ((b ? b[i] : 0) +/- (J x)[i]); sign = -1 with b for residual form.
+// u_ready: c->ujvp already holds the combination phi_e + gamma/c_e c_e of x.
 p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const double* b,
-                    bool scaled);
+                    bool scaled, bool u_ready = false);
 p4d_status jvp_reduced(p4d_ctx* c, const double* x, double* y, int transpose, const double* b,
-                       bool scaled);
+                       bool scaled, bool u_ready = false);
 
 // ---- particle elimination (particle.cu)
 p4d_status particle_solve64(p4d_ctx* c, const double* rc, double* yc, const double* tN, int transpose);

@@ -198,9 +198,12 @@ __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref
 }
 
 // x0c: phi_s of the cathode (x0, or the cathode hierarchy's own iterate).
+// u (optional, with the last fields stored): the combination z_phie +
+// gamma/c_e z_ce that the Jacobian product of z reads next.
 template <typename T>
 __global__ void k_store(Grid g, const uint8_t* __restrict__ label, int fmask, const T* __restrict__ x0,
-                        const T* __restrict__ x0c, const T* __restrict__ x1, const T* __restrict__ x2, VRef zref_) {
+                        const T* __restrict__ x0c, const T* __restrict__ x1, const T* __restrict__ x2, VRef zref_,
+                        const double* __restrict__ gdc, double* __restrict__ u) {
   double* __restrict__ zm = zref_.get();
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t nn = g.nn;
@@ -214,6 +217,11 @@ __global__ void k_store(Grid g, const uint8_t* __restrict__ label, int fmask, co
       continue;
     }
     zm[f * nn + n] = (double)xs[f][n];
+  }
+  if (u) {
+    const double ze = (fmask & 2) ? (double)x1[n] : zm[nn + n];
+    const double zc = (fmask & 4) ? (double)x2[n] : zm[2 * nn + n];
+    u[n] = fma(gdc[n], zc, ze);
   }
 }
 
@@ -302,7 +310,7 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
     const int hs[4] = {0, 1, 2, 3};
     P4D_TRYS(mg_vcycle(c, hs, 4));
     ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 7, (const T*)l0.x[0], (const T*)l0.x[1], (const T*)l0.x[2],
-                                                      (const T*)l0.x[3], z);
+                                                      (const T*)l0.x[3], z, c->gdc, TRANS ? nullptr : c->ujvp);
   } else {
     int done = 0;
     for (int t = 0; t < 3; ++t) {
@@ -315,7 +323,8 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
         if (kHOfField[f][q] >= 0) hs[nh++] = kHOfField[f][q];
       P4D_TRYS(mg_vcycle(c, hs, nh));
       ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 1 << f, (const T*)l0.x[0], (const T*)l0.x[1], (const T*)l0.x[2],
-                                                        (const T*)l0.x[3], z);
+                                                        (const T*)l0.x[3], z, c->gdc,
+                                                        TRANS || t < 2 ? nullptr : c->ujvp);
       done |= 1 << f;
     }
   }
