@@ -287,12 +287,13 @@ __global__ void k_linearize(int64_t NE, int nc, Kin kn, const int32_t* __restric
 // residual and the preconditioner's input weighting, both of which are free
 // to be any positive diagonal, so a relative 1e-7 perturbation changes
 // nothing but that definition.
-__device__ __forceinline__ void put_scale(double d, double* sqd, double* rsqd, int64_t row) {
+__device__ __forceinline__ float put_scale(double d, double* sqd, double* rsqd, int64_t row) {
   float a = (float)fabs(d);
   if (!(a > 0.f) || !isfinite(a)) a = 1.f;
   const float r = sqrtf(a);
   sqd[row] = (double)r;
   rsqd[row] = (double)(1.0f / r);
+  return r;
 }
 
 __global__ void k_diag(Grid g, int64_t NE, int nc, double tau, double idt, const double* __restrict__ Jst,
@@ -301,15 +302,15 @@ __global__ void k_diag(Grid g, int64_t NE, int nc, double tau, double idt, const
                        const double* __restrict__ kapj, const double* __restrict__ betaj,
                        const double* __restrict__ rref, const double* __restrict__ ge,
                        const double* __restrict__ gc, const double* __restrict__ gs, double* __restrict__ sqd,
-                       double* __restrict__ rsqd) {
+                       double* __restrict__ rsqd, float* __restrict__ sqd32) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t nn = g.nn;
   if (t < nn) {
     const int64_t n = t;
     const int32_t e = eidx[n];
-    put_scale((label[n] & kLabActive) ? Jst[(0 * 27 + 13) * nn + n] + Aj[e] * ge[e] : 1.0, sqd, rsqd, n);
-    put_scale(Jst[(1 * 27 + 13) * nn + n] + (e >= 0 ? Aj[e] * ge[e] : 0.0), sqd, rsqd, nn + n);
-    put_scale(Jst[(2 * 27 + 13) * nn + n] - (e >= 0 ? tau * Aj[e] * gc[e] : 0.0), sqd, rsqd, 2 * nn + n);
+    sqd32[n] = put_scale((label[n] & kLabActive) ? Jst[(0 * 27 + 13) * nn + n] + Aj[e] * ge[e] : 1.0, sqd, rsqd, n);
+    sqd32[nn + n] = put_scale(Jst[(1 * 27 + 13) * nn + n] + (e >= 0 ? Aj[e] * ge[e] : 0.0), sqd, rsqd, nn + n);
+    sqd32[2 * nn + n] = put_scale(Jst[(2 * 27 + 13) * nn + n] - (e >= 0 ? tau * Aj[e] * gc[e] : 0.0), sqd, rsqd, 2 * nn + n);
   } else if (t < nn + NE * nc) {
     const int64_t q = t - nn;
     const int64_t e = (uint32_t)q / (uint32_t)nc;   // NE nc < 2^31 (checked at setup)
@@ -518,7 +519,7 @@ p4d_status linearize(p4d_ctx* c, const p4d_state* st) {
                                                         c->tfac, c->tfac32, c->flags);
   ::p4d::count_launch(), k_diag<<<nblocks(nn + NE * nc), kBlock, 0, c->stream>>>(c->g, NE, nc, kn.tau, 1.0 / c->prm.dt, c->Jst, c->label,
                                                           c->eidx, c->Aj, c->Mj, c->kapj, c->betaj, c->rref,
-                                                          c->ge, c->gc, c->gs, c->sqd, c->rsqd);
+                                                          c->ge, c->gc, c->gs, c->sqd, c->rsqd, c->sqd32);
   ::p4d::count_launch(), k_state_scale<<<4 * 152, kBlock, 0, c->stream>>>(nn, NE * nc, c->sqd, st->phis, st->phie, st->ce,
                                                                          st->cs, c->part);
   ::p4d::count_launch(), k_state_sum<<<1, 128, 0, c->stream>>>(c->part, 4 * 152, c->unorm2);

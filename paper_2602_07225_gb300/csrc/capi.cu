@@ -290,6 +290,7 @@ p4d_status setup_impl(p4d_ctx* c, const p4d_mesh* m, const p4d_params* prm) {
   if (prm->precision != 0) P4D_TRYS(dalloc_t(c, &c->tfac32, (size_t)2 * std::max<int64_t>(1, NE) * nc));
   P4D_TRYS(dalloc_t(c, &c->sqd, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->rsqd, c->ndof));
+  P4D_TRYS(dalloc_t(c, &c->sqd32, (size_t)3 * nn));
   P4D_TRYS(dalloc_t(c, &c->iwf, 4));
   P4D_TRYS(dalloc_t(c, &c->unorm2, 4));
   P4D_TRYS(dalloc_t(c, &c->ujvp, nn));

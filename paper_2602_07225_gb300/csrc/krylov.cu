@@ -66,10 +66,13 @@ __device__ __forceinline__ void warp_transpose_reduce(double (&a)[P], int lane) 
 }
 
 // True in every thread of the block that finishes its kernel last, with the
-// other blocks' writes visible; it resets the counter for the next launch.
+// partial sums of the other blocks visible; it resets the counter for the
+// next launch.  The partial sums are written by the first warp, which alone
+// orders its writes (a fence in every warp held the blocks of an update back
+// by several microseconds).
 __device__ __forceinline__ bool last_block(unsigned* cnt) {
   __shared__ bool last;
-  __threadfence();
+  if (threadIdx.x < 32) __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     last = atomicAdd(cnt, 1u) == gridDim.x - 1;
@@ -284,15 +287,16 @@ struct Fin {
 
 // w[n] -= sum_i h[i] V[i][n] (h on the device), the products subtracted in
 // order of i; the loads of eight basis vectors are in flight at a time (R:
-// kp1 mod 8).  With fin.mode, each block also sums the updated w[n]^2 and
-// the last block finishes as fin says.  One element per thread and a grid of
-// up to 16 blocks per SM: 14 us at 614 k elements and 7 vectors against 20
-// us with one load per product in flight.
+// kp1 mod 8).  With fin.mode, the updated w[n]^2 are summed over nvb runs of
+// 256 elements (grid-strided; the partition of the sums does not depend on
+// the launch), four runs per block, and the last block finishes as fin says.
+// With a block per run and every warp fencing, the arrival of 2,432 blocks at
+// the counter took 10-15 of 25 us at 614 k elements.
 template <int R>
 __global__ void __launch_bounds__(kBlock) k_maxpy(const double* __restrict__ V, int64_t ldv, int kp1,
                                                   const double* __restrict__ h, double* __restrict__ w,
                                                   int64_t len, double sign, const double* __restrict__ flag,
-                                                  double* __restrict__ partial, unsigned* cnt, Fin fin) {
+                                                  double* __restrict__ partial, unsigned* cnt, int nvb, Fin fin) {
   if (flag && *flag == 0.0) {
     if (blockIdx.x == 0) {
       if (fin.mode == kFinGivens) givens_block(fin.hs, fin.L, fin.k, fin.kdev, fin.refine);
@@ -301,44 +305,48 @@ __global__ void __launch_bounds__(kBlock) k_maxpy(const double* __restrict__ V, 
     return;
   }
   __shared__ double hs[130];
-  __shared__ double red[kBlock / 32];
+  __shared__ double red[2][kBlock / 32];
   for (int i = threadIdx.x; i < kp1; i += blockDim.x) hs[i] = sign * h[i];
   __syncthreads();
-  double ss = 0.0;
-  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x) {
-    double acc = w[n];
-    const double* v = V + n;
-    int i = 0;
-    for (; i + 8 <= kp1; i += 8) {
-      double a[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int vb = blockIdx.x, it = 0; vb < nvb; vb += gridDim.x, ++it) {
+    double ss = 0.0;
+    for (int64_t n = vb * (int64_t)kBlock + threadIdx.x; n < len; n += (int64_t)nvb * kBlock) {
+      double acc = w[n];
+      const double* v = V + n;
+      int i = 0;
+      for (; i + 8 <= kp1; i += 8) {
+        double a[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) a[q] = v[(int64_t)(i + q) * ldv];
+        for (int q = 0; q < 8; ++q) a[q] = v[(int64_t)(i + q) * ldv];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc -= hs[i + q] * a[q];
+        for (int q = 0; q < 8; ++q) acc -= hs[i + q] * a[q];
+      }
+      if (R > 0) {
+        double a[R > 0 ? R : 1];
+#pragma unroll
+        for (int q = 0; q < R; ++q) a[q] = v[(int64_t)(i + q) * ldv];
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc -= hs[i + q] * a[q];
+      }
+      w[n] = acc;
+      if (fin.mode) ss = fma(acc, acc, ss);
     }
-    if (R > 0) {
-      double a[R > 0 ? R : 1];
-#pragma unroll
-      for (int q = 0; q < R; ++q) a[q] = v[(int64_t)(i + q) * ldv];
-#pragma unroll
-      for (int q = 0; q < R; ++q) acc -= hs[i + q] * a[q];
+    if (!fin.mode) continue;
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) red[it & 1][warp] = ss;   // two buffers: one barrier per run
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int i = 0; i < kBlock / 32; ++i) t += red[it & 1][i];
+      partial[vb] = t;
     }
-    w[n] = acc;
-    if (fin.mode) ss = fma(acc, acc, ss);
   }
   if (!fin.mode) return;
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int i = 0; i < kBlock / 32; ++i) t += red[i];
-    partial[blockIdx.x] = t;
-  }
   if (!last_block(cnt)) return;
   // strided sums per thread, then a halving tree over the 256 threads
   double t = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) t += __ldcg(partial + b);
+  for (int b = threadIdx.x; b < nvb; b += kBlock) t += __ldcg(partial + b);
   __shared__ double tree[kBlock];
   tree[threadIdx.x] = t;
   __syncthreads();
@@ -432,14 +440,26 @@ __global__ void k_scale(const double* x, double* y, int64_t len, const double* _
   // the factor once per block (an FP64 divide and square root per thread
   // cost more than the scaling itself on this GPU)
   __shared__ double sfac;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // four elements in flight, the first four over the factor's latency
+  double a[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) a[q] = n + q * stride < len ? x[n + q * stride] : 0.0;
   if (threadIdx.x == 0) {
     const double v = *sp;
     sfac = v != 0.0 ? 1.0 / sqrt(v) : 0.0;
   }
   __syncthreads();
   const double s = sfac;
-  for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < len; n += (int64_t)gridDim.x * blockDim.x)
-    y[n] = x[n] * s;
+  while (n < len) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (n + q * stride < len) y[n + q * stride] = a[q] * s;
+    n += 4 * stride;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = n + q * stride < len ? x[n + q * stride] : 0.0;
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (t.mode == 1) init_cycle(t);
     else if (t.mode == 2) step_done(t);
@@ -717,7 +737,7 @@ struct Reducer {
              const double* flag, const Fin& fin, unsigned gb) {
     switch (kp1 & 7) {
 #define P4D_MAXPY_CASE(R) \
-  case R: ::p4d::count_launch(), k_maxpy<R><<<gb, kBlock, 0, c->stream>>>(V, ldv, kp1, h, w, len, sign, flag, c->part, c->red_cnt, fin); break;
+  case R: ::p4d::count_launch(), k_maxpy<R><<<std::min(gb, 4u * 152u), kBlock, 0, c->stream>>>(V, ldv, kp1, h, w, len, sign, flag, c->part, c->red_cnt, (int)gb, fin); break;
       P4D_MAXPY_CASE(0) P4D_MAXPY_CASE(1) P4D_MAXPY_CASE(2) P4D_MAXPY_CASE(3)
       P4D_MAXPY_CASE(4) P4D_MAXPY_CASE(5) P4D_MAXPY_CASE(6) P4D_MAXPY_CASE(7)
 #undef P4D_MAXPY_CASE
@@ -886,7 +906,7 @@ p4d_status fg_cycle_launch(FgRun& r, bool gate = false) {
     t.limit = (double)std::min(r.m, c->prm.maxit - r.iters);
     t.rtol = c->prm.rtol;
   }
-  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(c->V, c->V, r.len, misc + 2 * L.m + 2, t);
+  ::p4d::count_launch(), k_scale<<<std::min(r.gb, 4u * 152u), kBlock, 0, c->stream>>>(c->V, c->V, r.len, misc + 2 * L.m + 2, t);
   P4D_TRY(cudaMemcpyAsync(c->hs_h + kBetaOff, misc + 2 * L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
 }
@@ -948,7 +968,7 @@ p4d_status fg_step_body(FgRun& r, int k, bool graph_precond, Tail t) {
   t.hs = c->hs;
   t.L = L;
   t.k = k;
-  ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, c->stream>>>(w, w, r.len, misc + 2 * L.m + 2, t);
+  ::p4d::count_launch(), k_scale<<<std::min(r.gb, 4u * 152u), kBlock, 0, c->stream>>>(w, w, r.len, misc + 2 * L.m + 2, t);
   prof_mark(c, 2);
   if (host) P4D_TRY(cudaMemcpyAsync(c->hs_h, misc + 2 * L.m + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return P4D_OK;
@@ -1495,7 +1515,7 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
       t.hs = c->hs;
       t.L = r.L;
       t.kdev = c->kdev;
-      ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(c->V, c->V, r.len, r.misc() + 2 * r.L.m + 2, t);
+      ::p4d::count_launch(), k_scale<<<std::min(r.gb, 4u * 152u), kBlock, 0, D->stream>>>(c->V, c->V, r.len, r.misc() + 2 * r.L.m + 2, t);
     }
     P4D_TRY(cudaMemcpyAsync(c0->hs_h + kBetaOff, r0.misc() + 2 * r0.L.m + 5, sizeof(double), cudaMemcpyDeviceToHost, D->stream));
     P4D_TRY(cudaStreamSynchronize(D->stream));
@@ -1569,7 +1589,7 @@ p4d_status fgmres_dd(p4d_dd_ctx* D, const double* const* b, double* const* x, p4
         FgRun& r = R[p];
         double* w = c->V + (int64_t)(k + 1) * r.len;
         ::p4d::count_launch(), k_givens<<<1, 32, 0, D->stream>>>(c->hs, r.L, k, c->kdev, refine);
-        ::p4d::count_launch(), k_scale<<<r.gb, kBlock, 0, D->stream>>>(w, w, r.len, r.misc() + 2 * r.L.m + 2, Tail{});
+        ::p4d::count_launch(), k_scale<<<std::min(r.gb, 4u * 152u), kBlock, 0, D->stream>>>(w, w, r.len, r.misc() + 2 * r.L.m + 2, Tail{});
       }
       P4D_TRY(cudaMemcpyAsync(c0->hs_h, r0.misc() + 2 * r0.L.m + 3, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                               D->stream));

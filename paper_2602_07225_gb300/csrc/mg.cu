@@ -895,89 +895,98 @@ __device__ __forceinline__ int par_of(const Axis1& a, int i, int q, T& w) {
 // Full-weighting restriction (P^T r)_C over the fine nodes of the mask.
 // The phi_e / c_e masks are all ones (no mask load); elsewhere a masked-out
 // residual is selected away (never multiplied: it may hold stale values).
+// Node planes of the listed hierarchies that hold rows of their masks.
+struct PRange {
+  int lo[kNH];
+  int cnt[kNH];
+};
+
+// Restriction by planes: the block's coarse plane K (and with it the z
+// support) is uniform, one integer division per node is left; absent
+// support nodes of an axis get weight 0 on a node of the plane (acc + 0 r =
+// acc; the support is summed in increasing node order).
 template <typename T>
-__device__ __forceinline__ T restrict_row(const LevelDims& fd, const LevelDims& cd, const Xfer1& X, const T* r,
-                                          const uint8_t* __restrict__ m, bool all_on, int C) {
-  int I, J, K;
-  node_ijk_i32(cd, C, I, J, K);
+__global__ void __launch_bounds__(256) k_restrict(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> fr,
+                                                  Ptr4<const uint8_t> fm, Ptr4<T> cb, HList hl, PRange pr) {
+  const int h = pk(hl.h, blockIdx.z);
+  if ((int)blockIdx.y >= pk(pr.cnt, h)) return;
+  const int K = pk(pr.lo, h) + (int)blockIdx.y;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= cd.nnx * cd.nny) return;
+  const int J = q / cd.nnx, I = q - J * cd.nnx;
+  const T* __restrict__ r = pk(fr.p, h);
+  const uint8_t* __restrict__ m = pk(fm.p, h);
+  const bool all_on = h >= 2;
+  int fx[3], fy[3];
+  T wx[3], wy[3];
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    fx[t] = sup_of<T>(X.a[0], I, t, wx[t]);
+    if (fx[t] < 0) { fx[t] = 0; wx[t] = (T)0; }
+    fy[t] = sup_of<T>(X.a[1], J, t, wy[t]);
+    if (fy[t] < 0) { fy[t] = 0; wy[t] = (T)0; }
+    fy[t] *= fd.nnx;
+  }
   T acc = 0;
 #pragma unroll
   for (int tz = 0; tz < 3; ++tz) {
     T wz;
     const int fk = sup_of<T>(X.a[2], K, tz, wz);
-    if (fk < 0) continue;
+    if (fk < 0) continue;   // uniform
+    const int o = fd.nnx * fd.nny * fk;
+    T v[9];
+    bool on[9];
 #pragma unroll
-    for (int ty = 0; ty < 3; ++ty) {
-      T wy;
-      const int fj = sup_of<T>(X.a[1], J, ty, wy);
-      if (fj < 0) continue;
-#pragma unroll
-      for (int tx = 0; tx < 3; ++tx) {
-        T wx;
-        const int fi = sup_of<T>(X.a[0], I, tx, wx);
-        if (fi < 0) continue;
-        const int f = fi + fd.nnx * (fj + fd.nny * fk);
-        const T v = r[f];
-        const bool on = all_on || m[f];
-        acc += on ? wx * wy * wz * v : (T)0;
-      }
+    for (int t = 0; t < 9; ++t) {
+      const int f = o + fy[t / 3] + fx[t % 3];
+      v[t] = r[f];
+      on[t] = all_on || m[f];
     }
+#pragma unroll
+    for (int t = 0; t < 9; ++t) acc += on[t] && wx[t % 3] * wy[t / 3] != (T)0 ? wx[t % 3] * wy[t / 3] * wz * v[t] : (T)0;
   }
-  return acc;
+  pk(cb.p, h)[K * (cd.nnx * cd.nny) + q] = acc;
 }
 
+// Prolongation by planes, as k_restrict.
 template <typename T>
-__global__ void k_restrict(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> fr, Ptr4<const uint8_t> fm, Ptr4<T> cb,
-                           HList hl, BRange br) {
-  const int h = pk(hl.h, blockIdx.y);
-  if ((int)blockIdx.x >= pk(br.cnt, h)) return;   // coarse blocks without rows of the coarse mask
-  const int C = (pk(br.lo, h) + (int)blockIdx.x) * blockDim.x + threadIdx.x;
-  if (C >= (int)cd.n) return;
-  const T* __restrict__ r = pk(fr.p, h);
-  pk(cb.p, h)[C] = restrict_row<T>(fd, cd, X, r, pk(fm.p, h), h >= 2, C);
-}
-
-// (P x_c)_f: trilinear interpolation of the coarse correction at fine node f.
-template <typename T>
-__device__ __forceinline__ T prolong_row(const LevelDims& fd, const LevelDims& cd, const Xfer1& X, const T* cx, int f) {
-  int i, j, k;
-  node_ijk_i32(fd, f, i, j, k);
-  T acc = 0;
-#pragma unroll
-  for (int c3 = 0; c3 < 2; ++c3) {
-    T wz;
-    const int pz = par_of<T>(X.a[2], k, c3, wz);
-    if (pz < 0) continue;
-#pragma unroll
-    for (int c2 = 0; c2 < 2; ++c2) {
-      T wy;
-      const int py = par_of<T>(X.a[1], j, c2, wy);
-      if (py < 0) continue;
-#pragma unroll
-      for (int c1 = 0; c1 < 2; ++c1) {
-        T wx;
-        const int px = par_of<T>(X.a[0], i, c1, wx);
-        if (px < 0) continue;
-        acc += wx * wy * wz * cx[px + cd.nnx * (py + cd.nny * pz)];
-      }
-    }
-  }
-  return acc;
-}
-
-template <typename T>
-__global__ void k_prolong(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> cx_, Ptr4<const uint8_t> fm, Ptr4<T> fx,
-                          HList hl, BRange br) {
-  const int h = pk(hl.h, blockIdx.y);
-  if ((int)blockIdx.x >= pk(br.cnt, h)) return;   // fine blocks without rows of the mask
-  const int f = (pk(br.lo, h) + (int)blockIdx.x) * blockDim.x + threadIdx.x;
-  if (f >= (int)fd.n) return;
+__global__ void __launch_bounds__(256) k_prolong(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> cx_,
+                                                 Ptr4<const uint8_t> fm, Ptr4<T> fx, HList hl, PRange pr) {
+  const int h = pk(hl.h, blockIdx.z);
+  if ((int)blockIdx.y >= pk(pr.cnt, h)) return;
+  const int k = pk(pr.lo, h) + (int)blockIdx.y;
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= fd.nnx * fd.nny) return;
+  const int j = q / fd.nnx, i = q - j * fd.nnx;
+  const int f = k * (fd.nnx * fd.nny) + q;
   // the mask gates only the write: the interpolation's loads do not wait on it
   // (phi_e / c_e masks are all ones)
   const bool on = h >= 2 || pk(fm.p, h)[f];
   const T xf = pk(fx.p, h)[f];
   const T* __restrict__ cx = pk(cx_.p, h);
-  const T acc = prolong_row<T>(fd, cd, X, cx, f);
+  int px[2], py[2];
+  T wx[2], wy[2];
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    px[t] = par_of<T>(X.a[0], i, t, wx[t]);
+    if (px[t] < 0) { px[t] = 0; wx[t] = (T)0; }
+    py[t] = par_of<T>(X.a[1], j, t, wy[t]);
+    if (py[t] < 0) { py[t] = 0; wy[t] = (T)0; }
+    py[t] *= cd.nnx;
+  }
+  T acc = 0;
+#pragma unroll
+  for (int c3 = 0; c3 < 2; ++c3) {
+    T wz;
+    const int pz = par_of<T>(X.a[2], k, c3, wz);
+    if (pz < 0) continue;   // uniform
+    const T* __restrict__ p = cx + pz * (cd.nnx * cd.nny);
+    T v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = p[py[t >> 1] + px[t & 1]];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) acc += wx[t & 1] * wy[t >> 1] * wz * v[t];
+  }
   if (on) pk(fx.p, h)[f] = xf + acc;
 }
 
@@ -1091,9 +1100,8 @@ __device__ __forceinline__ void tail_ijk(const TailLv& L, int n, int (&id)[3]) {
   id[0] = r - id[1] * L.d.nnx;
 }
 
-// restrict_row and prolong_row with the axes' entries formed once and absent
-// entries as weight 0 on an index inside the level (acc + 0 r = acc): 27 and
-// 8 independent loads.
+// The transfers of k_restrict and k_prolong for one row, the axes' entries
+// formed once, absent entries as weight 0 on an index inside the level.
 template <typename T>
 __device__ __forceinline__ T tail_restrict(const TailLv& F, const TailLv& C, const T* r, int c) {
   int id[3];
@@ -1416,6 +1424,32 @@ template <> const float* cheb_tab<float>(const p4d_ctx* c) { return c->cheb_dev3
 // grid width (the widest range).  The transfer kernels take one row per
 // thread in blocks of kBlock and share these ranges.
 static_assert(kNpt == 1, "block ranges are shared by the one-row-per-thread transfer kernels");
+// Threads per block of the transfers: a multiple of 64 that wastes little of
+// the plane's last block.
+int plane_threads(const MGLevel& L) {
+  const int sxy = L.nnx * L.nny;
+  int best = 256, waste = 1 << 30;
+  for (int t = 256; t >= 128; t -= 64) {
+    const int w = (int)nblocks(sxy, t) * t - sxy;
+    if (w < waste) { waste = w; best = t; }
+  }
+  return best;
+}
+
+PRange prange(const MGLevel& A, const int* hs, int nhs, unsigned* gy) {
+  PRange r{};
+  int w = 1;
+  const int sxy = A.nnx * A.nny;
+  for (int h = 0; h < kNH; ++h) {
+    const int lo = A.blo[h] * kBlock, hi = (int)std::min<int64_t>(A.n, (int64_t)(A.blo[h] + A.bcnt[h]) * kBlock);
+    r.lo[h] = lo / sxy;
+    r.cnt[h] = A.bcnt[h] ? (hi - 1) / sxy - r.lo[h] + 1 : 0;
+  }
+  for (int t = 0; t < nhs; ++t) w = std::max(w, r.cnt[hs[t]]);
+  *gy = (unsigned)w;
+  return r;
+}
+
 BRange brange(const MGLevel& A, const int* hs, int nhs, unsigned* gx) {
   BRange r{};
   int w = 1;
@@ -1549,9 +1583,9 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
     const dim3 grid(gx, nhs);
     for (int s = 0; s < deg; ++s) {
       if (l == 0 && s > 0) prof_mark(c, 3);
+      // (level 0, step 0: with the right-hand side, see mg_first_by_load)
       if (l == 0 && s > 0) P4D_TRYS((level0_stencil_step<TS0, T>(c, A, hs, nhs, hl, br, grid, 0, s)));
-      else if (l == 0) ::p4d::count_launch(), k_cheb<TS0, T><<<grid, kBlock, 0, c->stream>>>(dims(A), ptrs<TS0, T>(A), hl, br, cheb_tab<T>(c), l, s, 1);
-      else ::p4d::count_launch(), k_cheb<TS, T><<<grid, kBlock, 0, c->stream>>>(dims(A), ptrs<TS, T>(A), hl, br, cheb_tab<T>(c), l, s, s == 0);
+      else if (l > 0) ::p4d::count_launch(), k_cheb<TS, T><<<grid, kBlock, 0, c->stream>>>(dims(A), ptrs<TS, T>(A), hl, br, cheb_tab<T>(c), l, s, s == 0);
       if (l == 0 && s > 0) prof_mark(c, 3);
       swap_x(A, hs, nhs);
     }
@@ -1561,9 +1595,10 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
     Ptr4<const uint8_t> fm;
     Ptr4<T> cb;
     for (int h = 0; h < kNH; ++h) { fr.p[h] = (const T*)A.r[h]; fm.p[h] = A.mask[h]; cb.p[h] = (T*)B.b[h]; }
-    unsigned gxc = 1;
-    const BRange brc = brange(B, hs, nhs, &gxc);
-    ::p4d::count_launch(), k_restrict<T><<<dim3(gxc, nhs), kBlock, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fr, fm, cb, hl, brc);
+    unsigned gy = 1;
+    const PRange pr = prange(B, hs, nhs, &gy);
+    const int bt = plane_threads(B);
+    ::p4d::count_launch(), k_restrict<T><<<dim3(nblocks(B.nnx * B.nny, bt), gy, nhs), bt, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fr, fm, cb, hl, pr);
   }
   if (c->tail_l0 >= 0) {
     P4D_TRYS((tail_launch<TS0, TS, T>(c, hs, nhs, LT)));
@@ -1585,7 +1620,10 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs) {
     unsigned gx = 1;
     const BRange br = brange(A, hs, nhs, &gx);
     const dim3 grid(gx, nhs);
-    ::p4d::count_launch(), k_prolong<T><<<grid, kBlock, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), cxp, fm, fx, hl, br);
+    unsigned gy = 1;
+    const PRange pr = prange(A, hs, nhs, &gy);
+    const int bt = plane_threads(A);
+    ::p4d::count_launch(), k_prolong<T><<<dim3(nblocks(A.nnx * A.nny, bt), gy, nhs), bt, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), cxp, fm, fx, hl, pr);
     for (int s = 0; s < deg; ++s) {
       if (l == 0) prof_mark(c, 3);
       if (l == 0) P4D_TRYS((level0_stencil_step<TS0, T>(c, A, hs, nhs, hl, br, grid, 0, s)));

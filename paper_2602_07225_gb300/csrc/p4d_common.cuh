@@ -194,6 +194,7 @@ struct p4d_ctx {
   double* ujvp = nullptr;              // [nn] phi_e + gamma/c_e * c_e combination of a JVP input
   double* sqd = nullptr;               // [ndof] sqrt(|diag J|)
   double* rsqd = nullptr;              // [ndof] 1 / sqrt(|diag J|)
+  float* sqd32 = nullptr;              // [3 nn] the macro rows of sqd (its values are FP32 numbers)
   double* iwf = nullptr;               // [4] 1 / w_f
   double* unorm2 = nullptr;            // [4] ||(sqrt(d) u)_f||^2 of the linearization state
   double* wf = nullptr;                // [4] per-field Krylov weights (device)
@@ -492,6 +493,9 @@ p4d_status mg_update(p4d_ctx* c);
 p4d_status mg_fetch_lam(p4d_ctx* c);
 // run the V-cycles of the listed hierarchies on the level-0 right-hand sides already in place
 p4d_status mg_vcycle(p4d_ctx* c, const int* hs, int nhs);
+// whether the first Chebyshev step of level 0 comes with the right-hand side
+// (into d and x2): level 0 is smoothed by launches of its own
+inline bool mg_first_by_load(const p4d_ctx* c) { return c->nlev > 1 && c->tail_l0 != 0; }
 // matrix-free level 0 (mf.cu): setup after mg_setup_fixed; whether field f
 // (0 phi_s, 1 phi_e, 2 c_e) is applied matrix-free; one launch over the
 // fields in fmask: mode 0 Chebyshev step `step` (x -> x2, d), mode 1 r = b - A x

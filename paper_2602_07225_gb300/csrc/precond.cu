@@ -26,6 +26,7 @@ struct PcArgs {
   const int32_t* enode;
   const double *Aj, *Mj, *iMj, *betaj, *kapj, *rref;
   const double *ge, *gc, *gs, *zeta, *sqd, *iwf;
+  const float* sqd32;   // the macro rows of sqd (FP32 values)
   const double* Kk;     // K_kappa stencil [27][nn] (FP64, fixed)
   const double* gdc;    // gamma / c_e per node
   double sc[3];
@@ -138,21 +139,50 @@ __device__ __forceinline__ void local_uv(const PcArgs& a, int64_t e, bool act, d
   v[0] = act ? ge : 0.0; v[1] = -ge; v[2] = a.gc[e]; v[3] = a.gs[e];
 }
 
+// First Chebyshev step of level 0 from x = 0 (d = c0 D^-1 b, x = d), done
+// with the load when `on` (the level is launched on its own): per field 1/diag,
+// d and x (ctab: the Chebyshev table).
+template <typename T>
+struct First {
+  bool on;
+  const T* dinv[3];
+  T* d[3];
+  T* x[3];
+  const T* ctab;
+};
+
+template <typename T>
+__device__ __forceinline__ void first_step(const First<T>& s, int f, int64_t n, uint8_t lab, T b) {
+  const int h = f == 0 ? ((lab & kLabCathode) ? 1 : 0) : f + 1;
+  const T dn = s.ctab[h] * (s.dinv[f][n] * b);   // table entry (level 0, step 0, c0)
+  s.d[f][n] = dn;
+  s.x[f][n] = dn;
+}
+
 // Load the level-0 multigrid right-hand sides of the fields in `fmask`
 // (bit f): r_f = s^-1 r - condensation (FULL) - BGS couplings to the fields
 // in `done` (bits, their z already written to zm).  phi_s rows without an
 // unknown are identity rows: z = r directly.
 template <typename T, bool TRANS, bool FULL>
 __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref_, int fmask, int done, bool scaled,
-                       T* b0, T* b1, T* b2) {
+                       T* b0, T* b1, T* b2, First<T> first) {
   const double* __restrict__ r = rref_.get();
+  // the fields' factors once per block: conversions between FP64 and FP32
+  // run at the FP64 rate, and twelve per node were this kernel's time (37 us
+  // at 1.6 M nodes, three per node XX us with the first smoothing step)
+  __shared__ float wsh[3];
+  if (sizeof(T) == sizeof(float) && scaled) {
+    if (threadIdx.x < 3) wsh[threadIdx.x] = (float)(a.iwf[threadIdx.x] * a.sc[threadIdx.x]);
+    __syncthreads();
+  }
   const double* zm = zref_.get();
   double* zout = zref_.get();
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t nn = a.g.nn;
   if (n >= nn) return;
   const int32_t e = a.eidx[n];
-  const bool act = a.label[n] & kLabActive;
+  const uint8_t lab = a.label[n];
+  const bool act = lab & kLabActive;
   // the node couplings are needed only for the FULL condensation and for
   // BGS corrections (the reduced block-Jacobi load is a pure scaling, and
   // FP64 arithmetic is the cost of this kernel)
@@ -177,8 +207,9 @@ __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref
     if (sizeof(T) == sizeof(float) && scaled && !coupled && !dpc && !(f == 0 && !act)) {
       // FP32 right-hand side of an FP32 cycle: the scaling in FP32 (FP64
       // multiplies are this kernel's cost)
-      const float w = (float)(a.iwf[f] * a.sc[f]);
-      bs[f][n] = (T)(((float)r[row] * (float)a.sqd[row]) * w);
+      const T bv = (T)(((float)r[row] * a.sqd32[row]) * wsh[f]);
+      bs[f][n] = bv;
+      if (first.on) first_step(first, f, n, lab, bv);
       continue;
     }
     double rf = scaled ? (r[row] * a.sqd[row]) * a.iwf[f] : r[row];
@@ -193,7 +224,9 @@ __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref
       zout[n] = rf;   // identity row
       continue;
     }
-    bs[f][n] = (T)(a.sc[f] * rf);
+    const T bv = (T)(a.sc[f] * rf);
+    bs[f][n] = bv;
+    if (first.on) first_step(first, f, n, lab, bv);
   }
 }
 
@@ -283,7 +316,7 @@ PcArgs make_pc(p4d_ctx* c) {
   a.tau = (1.0 - c->prm.tplus) / c->prm.F; a.dt = c->prm.dt; a.idt = 1.0 / c->prm.dt;
   a.label = c->label; a.eidx = c->eidx; a.enode = c->enode;
   a.Aj = c->Aj; a.Mj = c->Mj; a.iMj = c->iMj; a.betaj = c->betaj; a.kapj = c->kapj; a.rref = c->rref;
-  a.ge = c->ge; a.gc = c->gc; a.gs = c->gs; a.zeta = c->zeta; a.sqd = c->sqd; a.iwf = c->iwf;
+  a.ge = c->ge; a.gc = c->gc; a.gs = c->gs; a.zeta = c->zeta; a.sqd = c->sqd; a.iwf = c->iwf; a.sqd32 = c->sqd32;
   a.Kk = c->Jst + 27 * c->g.nn; a.gdc = c->gdc;
   for (int f = 0; f < 3; ++f) a.sc[f] = c->scale_f[f];
   return a;
@@ -305,8 +338,17 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
     ::p4d::count_launch(), k_part_fwd<T, TRANS><<<nblocks(c->NE, kPartBlock), kPartBlock, 0, c->stream>>>(a, F, r, yc, scaled);
   MGLevel& l0 = c->lev[0];
   T* b[3] = {(T*)l0.b[0], (T*)l0.b[2], (T*)l0.b[3]};
+  const int hf[3] = {0, 2, 3};
+  First<T> first;
+  first.on = mg_first_by_load(c);
+  for (int f = 0; f < 3; ++f) {
+    first.dinv[f] = (const T*)l0.dinv[hf[f]];
+    first.d[f] = (T*)l0.d[hf[f]];
+    first.x[f] = (T*)l0.x2[hf[f]];
+  }
+  first.ctab = sizeof(T) == sizeof(double) ? (const T*)c->cheb_dev : (const T*)c->cheb_dev32;
   if (c->prm.combine == 0) {
-    ::p4d::count_launch(), k_load<T, TRANS, FULL><<<nblocks(nn), kBlock, 0, c->stream>>>(a, r, yc, z, 7, 0, scaled, b[0], b[1], b[2]);
+    ::p4d::count_launch(), k_load<T, TRANS, FULL><<<nblocks(nn), kBlock, 0, c->stream>>>(a, r, yc, z, 7, 0, scaled, b[0], b[1], b[2], first);
     const int hs[4] = {0, 1, 2, 3};
     P4D_TRYS(mg_vcycle(c, hs, 4));
     ::p4d::count_launch(), k_store<T><<<nblocks(nn), kBlock, 0, c->stream>>>(c->g, c->label, 7, (const T*)l0.x[0], (const T*)l0.x[1], (const T*)l0.x[2],
@@ -316,7 +358,7 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
     for (int t = 0; t < 3; ++t) {
       const int f = TRANS ? c->prm.order[2 - t] : c->prm.order[t];
       ::p4d::count_launch(), k_load<T, TRANS, FULL><<<nblocks(nn), kBlock, 0, c->stream>>>(a, r, yc, z, 1 << f, done, scaled, b[0], b[1],
-                                                                   b[2]);
+                                                                   b[2], first);
       int hs[2];
       int nh = 0;
       for (int q = 0; q < 2; ++q)
