@@ -456,7 +456,6 @@ p4d_status p4d_jacobian_update(p4d_handle h, const p4d_state* st) {
   h->linearized = false;
   P4D_TRYS(linearize(h, st));
   P4D_TRYS(mg_update(h));
-  P4D_TRYS(check_flags(h));
   P4D_TRYS(mg_fetch_lam(h));
   h->linearized = true;
   return P4D_OK;

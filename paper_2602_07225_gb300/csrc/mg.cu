@@ -102,6 +102,51 @@ __global__ void k_mask_coarse(LevelDims fd, LevelDims cd, Xfer X, Ptr4<const uin
   pk(cm.p, h)[C] = any ? 1 : 0;
 }
 
+// 32-bit (i, j, k) of node n of a level (every level has < 2^31 nodes).
+__device__ __forceinline__ void node_ijk_i32(const LevelDims& d, int n, int& i, int& j, int& k) {
+  const int sxy = d.nnx * d.nny;
+  k = n / sxy;
+  const int r = n - k * sxy;
+  j = r / d.nnx;
+  i = r - j * d.nnx;
+}
+
+// Interpolation between a level and its coarsening, computed instead of read
+// from the tables of struct Axis (same rule and weights; the weights 1/2 and
+// 1 are exact, so the sums round identically): a table entry is a dependent
+// load in front of every transferred value, and the transfers are bound by
+// that latency.  Coarse node I of a coarsened axis sits on fine node 2 I;
+// with an odd element count the last fine node keeps its own coarse node.
+struct Axis1 {
+  int nf, nc, c;   // fine nodes, coarse nodes, coarsened
+};
+struct Xfer1 {
+  Axis1 a[3];
+};
+
+// Entry t of the support of coarse node I: fine node (-1: none) and weight.
+template <typename T>
+__device__ __forceinline__ int sup_of(const Axis1& a, int I, int t, T& w) {
+  w = (T)1;
+  if (!a.c) return t == 0 ? I : -1;
+  const int f = 2 * I - 1 + t;
+  if (f < 0 || f >= a.nf) return -1;
+  if (f == a.nf - 1 && !(a.nf & 1)) return I == a.nc - 1 ? f : -1;   // the last fine node of an odd element count
+  if (t != 1) w = (T)0.5;
+  return f;
+}
+
+// Parent q (0, 1) of fine node i: coarse node (-1: none) and weight.
+template <typename T>
+__device__ __forceinline__ int par_of(const Axis1& a, int i, int q, T& w) {
+  w = (T)1;
+  if (!a.c) return q == 0 ? i : -1;
+  if (i == a.nf - 1 && !(a.nf & 1)) return q == 0 ? a.nc - 1 : -1;
+  if (!(i & 1)) return q == 0 ? i >> 1 : -1;
+  w = (T)0.5;
+  return (i >> 1) + q;
+}
+
 // ---------------------------------------------------------------- Galerkin
 // Source operator in difference form: off-diagonals O[o][n] (o != 13) and
 // row sums s[n] (slot 13, or a separate array at level 0).
@@ -231,6 +276,109 @@ __global__ void __launch_bounds__(32 * kRapWarps) k_rap(LevelDims fd, LevelDims 
   }
   __syncwarp();
   rap_finish<TV>(my, rs_l, cin, identity_out, lane, pk(out.p, h), cd.n, C);
+}
+
+// The same product in FP32, without scattering: per axis the parents of the
+// neighbours f + o of a support node lie on the coarse offsets d in {-1, 0,
+// 1} of I, so the lane multiplies its row with 3 x 3 weight maps per axis
+// held in registers (absent parents: weight 0, acc + 0 = acc) and adds to 27
+// register accumulators, offset by offset as the scatter does; only the 27
+// slots then pass through shared memory, summed over the lanes in the same
+// order.  The scatter updates shared memory up to 216 times per lane (109 us
+// at level 2 of a 65 x 65 x 49 cell, 751 + 188 us at levels 2 and 3 of 129 x
+// 129 x 97); with this kernel and the coarsest solve below the linearization
+// of the two cells takes 0.51 and 2.27 ms instead of 0.70 and 2.88.  In FP64
+// the extra products cost more than the scatter.
+struct RapAxis {
+  float m[3][3];   // [o][d]: weight from fine node f + o - 1 to coarse node I + d - 1
+};
+__device__ __forceinline__ RapAxis rap_axis(const Axis1& a, int I, int t, int& f, float& w) {
+  RapAxis r;
+  f = sup_of<float>(a, I, t, w);
+#pragma unroll
+  for (int o = 0; o < 3; ++o) {
+    const int g = f + o - 1;
+    const bool in = f >= 0 && g >= 0 && g < a.nf;
+    float w0 = 0.f, w1 = 0.f;
+    const int p0 = in ? par_of<float>(a, g, 0, w0) : -9, p1 = in ? par_of<float>(a, g, 1, w1) : -9;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r.m[o][d] = p0 == I + d - 1 && p0 >= 0 ? w0 : (p1 == I + d - 1 && p1 >= 0 ? w1 : 0.f);
+  }
+  return r;
+}
+
+__global__ void __launch_bounds__(32 * kRapWarps) k_rap32(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const float> fst,
+                                                          Ptr4<const uint8_t> fm, Ptr4<const uint8_t> cm,
+                                                          Ptr4<float> out) {
+  __shared__ float part[kRapWarps][27 * kRapLd];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int C = blockIdx.x * kRapWarps + warp;
+  const int h = blockIdx.y;
+  if (C >= (int)cd.n) return;   // per warp
+  float* my = part[warp];
+  int I, J, K;
+  node_ijk_i32(cd, C, I, J, K);
+  const bool cin = pk(cm.p, h)[C];
+  const float* __restrict__ st = pk(fst.p, h);
+  const uint8_t* __restrict__ m = pk(fm.p, h);
+  const int fn = (int)fd.n;
+  float acc[27];
+#pragma unroll
+  for (int q = 0; q < 27; ++q) acc[q] = 0.f;
+  float rs_l = 0.f;
+  if (cin && lane < 27) {
+    int fi, fj, fk;
+    float wx, wy, wz;
+    const RapAxis ax = rap_axis(X.a[0], I, lane % 3, fi, wx);
+    const RapAxis ay = rap_axis(X.a[1], J, lane / 3 % 3, fj, wy);
+    const RapAxis az = rap_axis(X.a[2], K, lane / 9, fk, wz);
+    const int f = fi + fd.nnx * (fj + fd.nny * fk);
+    if (fi >= 0 && fj >= 0 && fk >= 0 && m[f]) {
+      const float wf = wx * (wy * wz);
+      float a[27];
+#pragma unroll
+      for (int o = 0; o < 27; ++o) a[o] = st[o * fn + f];
+      unsigned in = 0;   // neighbours inside the grid and the mask
+#pragma unroll
+      for (int o = 0; o < 27; ++o) {
+        const int gi = fi + o % 3 - 1, gj = fj + (o / 3) % 3 - 1, gk = fk + o / 9 - 1;
+        const bool g = gi >= 0 && gj >= 0 && gk >= 0 && gi < fd.nnx && gj < fd.nny && gk < fd.nnz;
+        if (g && m[gi + fd.nnx * (gj + fd.nny * gk)]) in |= 1u << o;
+      }
+      const float sf = a[13];
+      rs_l = wf * sf;
+      float diag = sf;   // full-form diagonal of row f
+#pragma unroll
+      for (int o = 0; o < 27; ++o)
+        if (o != 13) diag -= a[o];
+      a[13] = diag;
+#pragma unroll
+      for (int oz = 0; oz < 3; ++oz)
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy) {
+          float wzy[9];
+#pragma unroll
+          for (int q = 0; q < 9; ++q) wzy[q] = az.m[oz][q / 3] * ay.m[oy][q % 3];
+#pragma unroll
+          for (int ox = 0; ox < 3; ++ox) {
+            const int o = ox + 3 * oy + 9 * oz;
+            const float v = (in >> o) & 1 ? a[o] * wf : 0.f;
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              const float t = v * ax.m[ox][dx];
+#pragma unroll
+              for (int q = 0; q < 9; ++q) acc[3 * q + dx] += t * wzy[q];
+            }
+          }
+        }
+    }
+  }
+  if (lane < 27) {
+#pragma unroll
+    for (int o = 0; o < 27; ++o) my[o * kRapLd + lane] = acc[o];
+  }
+  __syncwarp();
+  rap_finish<float>(my, rs_l, cin, 0, lane, pk(out.p, h), cd.n, C);
 }
 
 // V_1 = P^T diag(m s) P by gathering: with a diagonal operator and a
@@ -439,17 +587,20 @@ __global__ void k_level_combine(LevelDims d, Ptr4<const double> F, Ptr4<const TV
   double gl = 0.0;
   if (n < d.n) {
     const double sc = h == 0 ? sc0 : (h == 1 ? sc1 : (h == 2 ? sc2 : sc3));
-    const double* f = pk(F.p, h);
-    const TV* v = pk(V.p, h);
+    const double* __restrict__ f = pk(F.p, h);
+    const TV* __restrict__ v = pk(V.p, h);
     if (std::is_same<T, float>::value) {
       // FP32 cycle: the sum of the fixed and variable parts, the scaling, the
       // diagonal and the Gershgorin sums in FP32 (the results are stored in
       // FP32 or BF16; the row sum in slot 13 adds its two parts directly)
       const float scf = (float)sc;
       float diag = 0.f, absoff = 0.f, s = 0.f;
+      float as[27];   // all loads before the first store
+#pragma unroll
+      for (int o = 0; o < 27; ++o) as[o] = (float)f[o * d.n + n] + (float)v[o * d.n + n];
 #pragma unroll
       for (int o = 0; o < 27; ++o) {
-        const float a = (float)f[o * d.n + n] + (float)v[o * d.n + n];
+        const float a = as[o];
         pk(st.p, h)[o * d.n + n] = (TS)(scf * a);
         if (o == 13) s = a;
         else { diag -= a; absoff += fabsf(a); }
@@ -460,8 +611,12 @@ __global__ void k_level_combine(LevelDims d, Ptr4<const double> F, Ptr4<const TV
       if (pk(mask.p, h)[n]) gl = (double)((absoff + fabsf(diag)) / diag);
     } else {
       double diag = 0.0, absoff = 0.0, s = 0.0;
+      double as[27];
+#pragma unroll
+      for (int o = 0; o < 27; ++o) as[o] = f[o * d.n + n] + (double)v[o * d.n + n];
+#pragma unroll
       for (int o = 0; o < 27; ++o) {
-        const double a = f[o * d.n + n] + (double)v[o * d.n + n];
+        const double a = as[o];
         pk(st.p, h)[o * d.n + n] = fromd<TS>(sc * a);
         if (o == 13) s = a;
         else { diag -= a; absoff += fabs(a); }
@@ -534,23 +689,68 @@ __global__ void k_dense0(Grid g, const double* __restrict__ Jst, const double* _
   A[n * nn + n] = sc * diag;
 }
 
-// In-place Gauss-Jordan inversion with partial pivoting, one block per matrix.
 // Coarsest-level inverse, n <= kLuMax: LU with partial pivoting of each
-// hierarchy's matrix in one block (row-major, in place in lu; perm[i] = the
-// original row now at row i), then the columns of the inverse, one warp
-// each, by forward and backward substitution.  FP64 throughout.
+// hierarchy's matrix in one block (perm[i] = the original row now at row i),
+// then the columns of the inverse, one warp each, by forward and backward
+// substitution.  FP64 throughout.  Up to kLuSmem rows the matrix stays in
+// shared memory (rows padded by one entry); larger ones in global memory.  A
+// pivot step is a pivot search by one warp and the update of the rows below,
+// two block barriers; the elements of the multiplier column are formed by the
+// row's warp.  With the matrix in global memory and five barriers per step
+// the two kernels took 132 + 75 us at n = 63; the factorization is bound by
+// the FP64 rate of one SM (n^3 / 6 clocks) from n ~ 100 on.
 constexpr int kLuMax = 256;
+constexpr int kLuSmem = 160;
+constexpr int kLuThreads = 512;
+inline size_t lu_smem(int n) { return n <= kLuSmem ? sizeof(double) * n * (n + 1) : 0; }
 
-__global__ void __launch_bounds__(256) k_lu_factor(int n, const double* __restrict__ mats, double* __restrict__ lu,
-                                                   int* __restrict__ perm) {
-  const double* A0 = mats + (size_t)blockIdx.x * n * n;
-  double* A = lu + (size_t)blockIdx.x * n * n;
-  int* P = perm + (size_t)blockIdx.x * n;
+// Row n of the dense scaled coarsest operator, from difference form.
+struct DenseRows {
+  LevelDims d;
+  double sc[kNH];
+};
+
+template <typename TV>
+__global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, Ptr4<const double> F, Ptr4<const TV> V,
+                                                          const double* __restrict__ mats, double* __restrict__ lu,
+                                                          int* __restrict__ perm) {
+  extern __shared__ double lu_s[];
+  const int h = blockIdx.x;
+  double* G = lu + (size_t)h * n * n;
+  const bool sm = n <= kLuSmem;
+  double* A = sm ? lu_s : G;
+  const int ld = sm ? n + 1 : n;
+  int* P = perm + (size_t)h * n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __shared__ int piv;
   __shared__ double inv_d;
-  for (int r = warp; r < n; r += nw)
-    for (int cc = lane; cc < n; cc += 32) A[(size_t)r * n + cc] = A0[(size_t)r * n + cc];
+  if (mats) {
+    const double* A0 = mats + (size_t)h * n * n;
+    for (int r = warp; r < n; r += nw)
+      for (int cc = lane; cc < n; cc += 32) A[(size_t)r * ld + cc] = A0[(size_t)r * n + cc];
+  } else {
+    for (int r = warp; r < n; r += nw)
+      for (int cc = lane; cc < n; cc += 32) A[(size_t)r * ld + cc] = 0.0;
+    __syncthreads();
+    const double sc = pk(dr.sc, h);
+    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+      int i, j, k;
+      node_ijk(dr.d, r, i, j, k);
+      double a[27];
+#pragma unroll
+      for (int o = 0; o < 27; ++o) a[o] = pk(F.p, h)[o * dr.d.n + r] + (double)pk(V.p, h)[o * dr.d.n + r];
+      double diag = 0.0;
+#pragma unroll
+      for (int o = 0; o < 27; ++o) {
+        if (o == 13) { diag += a[o]; continue; }
+        diag -= a[o];
+        const int ii = i + o % 3 - 1, jj = j + (o / 3) % 3 - 1, kk = k + o / 9 - 1;
+        if (ii < 0 || jj < 0 || kk < 0 || ii >= dr.d.nnx || jj >= dr.d.nny || kk >= dr.d.nnz) continue;
+        A[(size_t)r * ld + ii + dr.d.nnx * (jj + dr.d.nny * kk)] = sc * a[o];
+      }
+      A[(size_t)r * ld + r] = sc * diag;
+    }
+  }
   for (int r = threadIdx.x; r < n; r += blockDim.x) P[r] = r;
   __syncthreads();
   for (int k = 0; k < n; ++k) {
@@ -558,7 +758,7 @@ __global__ void __launch_bounds__(256) k_lu_factor(int n, const double* __restri
       double best = -1.0;
       int idx = k;
       for (int r = k + lane; r < n; r += 32) {
-        const double v = fabs(A[(size_t)r * n + k]);
+        const double v = fabs(A[(size_t)r * ld + k]);
         if (v > best) { best = v; idx = r; }
       }
       for (int o = 16; o > 0; o >>= 1) {
@@ -568,67 +768,83 @@ __global__ void __launch_bounds__(256) k_lu_factor(int n, const double* __restri
       }
       if (lane == 0) {
         piv = idx;
-        const double d = A[(size_t)idx * n + k];
+        const double d = A[(size_t)idx * ld + k];
         inv_d = d != 0.0 ? 1.0 / d : 0.0;
       }
     }
     __syncthreads();
     const int p = piv;
-    if (p != k) {
+    if (p != k) {   // uniform
       for (int cc = threadIdx.x; cc < n; cc += blockDim.x) {
-        const double t = A[(size_t)k * n + cc];
-        A[(size_t)k * n + cc] = A[(size_t)p * n + cc];
-        A[(size_t)p * n + cc] = t;
+        const double t = A[(size_t)k * ld + cc];
+        A[(size_t)k * ld + cc] = A[(size_t)p * ld + cc];
+        A[(size_t)p * ld + cc] = t;
       }
       if (threadIdx.x == 0) {
         const int t = P[k];
         P[k] = P[p];
         P[p] = t;
       }
+      __syncthreads();
     }
-    __syncthreads();
     const double id = inv_d;
-    for (int r = k + 1 + threadIdx.x; r < n; r += blockDim.x) A[(size_t)r * n + k] *= id;
-    __syncthreads();
     for (int r = k + 1 + warp; r < n; r += nw) {
-      const double l = A[(size_t)r * n + k];
+      const double l = A[(size_t)r * ld + k] * id;
+      __syncwarp();
+      if (lane == 0) A[(size_t)r * ld + k] = l;
       if (l == 0.0) continue;
-      for (int cc = k + 1 + lane; cc < n; cc += 32) A[(size_t)r * n + cc] -= l * A[(size_t)k * n + cc];
+      for (int cc = k + 1 + lane; cc < n; cc += 32) A[(size_t)r * ld + cc] -= l * A[(size_t)k * ld + cc];
     }
     __syncthreads();
   }
+  if (sm)
+    for (int r = warp; r < n; r += nw)
+      for (int cc = lane; cc < n; cc += 32) G[(size_t)r * n + cc] = A[(size_t)r * ld + cc];
 }
 
-__global__ void __launch_bounds__(128) k_lu_inverse(int n, const double* __restrict__ lu, const int* __restrict__ perm,
-                                                    double* __restrict__ inv) {
-  __shared__ double xs[4][kLuMax];
+// Columns of the inverse: four warps of a block, a column each at a time.
+constexpr int kLuCols = 4;
+__global__ void __launch_bounds__(32 * kLuCols) k_lu_inverse(int n, const double* __restrict__ lu,
+                                                             const int* __restrict__ perm, double* __restrict__ inv) {
+  extern __shared__ double lu_s[];
+  __shared__ double xs[kLuCols][kLuMax];
+  __shared__ double rd[kLuMax];   // the diagonal
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = blockIdx.x * 4 + warp;
+  const int j = blockIdx.x * kLuCols + warp;
+  const double* G = lu + (size_t)blockIdx.y * n * n;
+  const bool sm = n <= kLuSmem;
+  const int ld = sm ? n + 1 : n;
+  if (sm)
+    for (int r = warp; r < n; r += kLuCols)
+      for (int cc = lane; cc < n; cc += 32) lu_s[(size_t)r * ld + cc] = G[(size_t)r * n + cc];
+  const double* A = sm ? lu_s : G;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) rd[r] = G[(size_t)r * n + r];
+  __syncthreads();
   if (j >= n) return;   // per warp
-  const double* A = lu + (size_t)blockIdx.y * n * n;
   const int* P = perm + (size_t)blockIdx.y * n;
   double* x = xs[warp];
   // x = P e_j, then L y = x (unit lower), then U x = y
-  for (int i = lane; i < n; i += 32) x[i] = P[i] == j ? 1.0 : 0.0;
+  int k0 = n;
+  for (int i = lane; i < n; i += 32) {
+    const bool one = P[i] == j;
+    x[i] = one ? 1.0 : 0.0;
+    if (one) k0 = i;
+  }
+  for (int o = 16; o > 0; o >>= 1) k0 = min(k0, __shfl_xor_sync(0xffffffffu, k0, o));
   __syncwarp();
-  for (int k = 0; k < n - 1; ++k) {
+  for (int k = k0; k < n - 1; ++k) {   // x is zero above its unit entry
     const double xk = x[k];
     __syncwarp();
     if (xk != 0.0)
-      for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[(size_t)i * n + k] * xk;
+      for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[(size_t)i * ld + k] * xk;
     __syncwarp();
   }
   for (int k = n - 1; k >= 0; --k) {
-    double xk = 0.0;
-    if (lane == 0) {
-      const double d = A[(size_t)k * n + k];
-      xk = d != 0.0 ? x[k] / d : 0.0;
-      x[k] = xk;
-    }
-    xk = __shfl_sync(0xffffffffu, xk, 0);
+    const double d = rd[k], xk = d != 0.0 ? x[k] / d : 0.0;
     __syncwarp();
+    if (lane == 0) x[k] = xk;
     if (xk != 0.0)
-      for (int i = lane; i < k; i += 32) x[i] -= A[(size_t)i * n + k] * xk;
+      for (int i = lane; i < k; i += 32) x[i] -= A[(size_t)i * ld + k] * xk;
     __syncwarp();
   }
   double* Inv = inv + (size_t)blockIdx.y * n * n;
@@ -846,51 +1062,6 @@ __global__ void __launch_bounds__(256) k_resid(LevelDims dd, LvlPtrs<TS, T> P, H
     if (on[q]) r[n[q]] = b[n[q]] - ax[q];
 }
 
-
-// 32-bit (i, j, k) of node n of a level (every level has < 2^31 nodes).
-__device__ __forceinline__ void node_ijk_i32(const LevelDims& d, int n, int& i, int& j, int& k) {
-  const int sxy = d.nnx * d.nny;
-  k = n / sxy;
-  const int r = n - k * sxy;
-  j = r / d.nnx;
-  i = r - j * d.nnx;
-}
-
-// Interpolation between a level and its coarsening, computed instead of read
-// from the tables of struct Axis (same rule and weights; the weights 1/2 and
-// 1 are exact, so the sums round identically): a table entry is a dependent
-// load in front of every transferred value, and the transfers are bound by
-// that latency.  Coarse node I of a coarsened axis sits on fine node 2 I;
-// with an odd element count the last fine node keeps its own coarse node.
-struct Axis1 {
-  int nf, nc, c;   // fine nodes, coarse nodes, coarsened
-};
-struct Xfer1 {
-  Axis1 a[3];
-};
-
-// Entry t of the support of coarse node I: fine node (-1: none) and weight.
-template <typename T>
-__device__ __forceinline__ int sup_of(const Axis1& a, int I, int t, T& w) {
-  w = (T)1;
-  if (!a.c) return t == 0 ? I : -1;
-  const int f = 2 * I - 1 + t;
-  if (f < 0 || f >= a.nf) return -1;
-  if (f == a.nf - 1 && !(a.nf & 1)) return I == a.nc - 1 ? f : -1;   // the last fine node of an odd element count
-  if (t != 1) w = (T)0.5;
-  return f;
-}
-
-// Parent q (0, 1) of fine node i: coarse node (-1: none) and weight.
-template <typename T>
-__device__ __forceinline__ int par_of(const Axis1& a, int i, int q, T& w) {
-  w = (T)1;
-  if (!a.c) return q == 0 ? i : -1;
-  if (i == a.nf - 1 && !(a.nf & 1)) return q == 0 ? a.nc - 1 : -1;
-  if (!(i & 1)) return q == 0 ? i >> 1 : -1;
-  w = (T)0.5;
-  return (i >> 1) + q;
-}
 
 // Full-weighting restriction (P^T r)_C over the fine nodes of the mask.
 // The phi_e / c_e masks are all ones (no mask load); elsewhere a masked-out
@@ -1767,13 +1938,19 @@ p4d_status mg_plan(p4d_ctx* c) {
     nnz = cn[2];
   }
   c->nlev = L;
+  // process-wide attributes: the largest sizes the kernels use
+  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
+  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
+  P4D_TRY(cudaFuncSetAttribute(k_lu_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
   if (c->lev[L - 1].n > 4096) return P4D_ERR_INVALID_ARG;   // coarsest level too large for a dense inverse
   P4D_TRYS(tail_plan(c));
+  double* lam = nullptr;
+  P4D_TRYS(dalloc_t(c, &lam, (size_t)kNH * L));
   for (int l = 0; l < L; ++l) {
     MGLevel& lv = c->lev[l];
     const int64_t n = lv.n;
     const size_t ts = tsize(prec, l);
-    P4D_TRYS(dalloc_t(c, &lv.lam, kNH));
+    lv.lam = lam + (size_t)l * kNH;
     for (int h = 0; h < kNH; ++h) P4D_TRYS(dalloc_t(c, &lv.mask[h], n));
     if (l == 0) {
       // fields: phi_s (hierarchies 0,1 share), phi_e (2), c_e (3)
@@ -1913,20 +2090,6 @@ p4d_status mg_setup_fixed(p4d_ctx* c) {
   return P4D_OK;
 }
 
-// Inverse of the coarsest dense matrices in mats (overwritten with it);
-// work: scratch of the same size.
-p4d_status coarse_inverse(p4d_ctx* c, MGLevel& C, double* mats, double* work) {
-  const int n = (int)C.n;
-  if (n <= kLuMax) {
-    ::p4d::count_launch(), k_lu_factor<<<kNH, 256, 0, c->stream>>>(n, mats, work, C.perm);
-    ::p4d::count_launch(), k_lu_inverse<<<dim3((n + 3) / 4, kNH), 128, 0, c->stream>>>(n, work, C.perm, mats);
-  } else {
-    ::p4d::count_launch(), k_gauss_jordan<<<kNH, 256, 0, c->stream>>>(n, mats, work);
-  }
-  P4D_TRY(cudaGetLastError());
-  return P4D_OK;
-}
-
 // Variable part of levels >= 1 (Galerkin products in precision TV), the
 // stored level operators, and the coarsest dense inverse (FP64).
 template <typename TV>
@@ -1947,8 +2110,13 @@ p4d_status mg_update_levels(p4d_ctx* c, const double* svar, const double* sch) {
       ::p4d::count_launch(), k_rap_diag_g<TV><<<dim3(nblocks(B.n, 128), kNH), 128, 0, c->stream>>>(dims(A), dims(B), A.X, s, fm, cm, out);
     } else {
       Ptr4<const TV> fst, frs;
+      if constexpr (std::is_same<TV, float>::value) {
+        for (int h = 0; h < kNH; ++h) fst.p[h] = (const float*)A.Vvar + (size_t)h * 27 * A.n;
+        ::p4d::count_launch(), k_rap32<<<dim3(nblocks(B.n, kRapWarps), kNH), 32 * kRapWarps, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fst, fm, cm, out);
+      } else {
       for (int h = 0; h < kNH; ++h) { fst.p[h] = (const TV*)A.Vvar + (size_t)h * 27 * A.n; frs.p[h] = nullptr; }
       ::p4d::count_launch(), k_rap<TV><<<dim3(nblocks(B.n, kRapWarps), kNH), 32 * kRapWarps, 0, c->stream>>>(dims(A), dims(B), A.X, fst, frs, fm, cm, out, 0);
+      }
     }
     Ptr4<const double> F;
     Ptr4<const TV> V;
@@ -1983,16 +2151,28 @@ p4d_status mg_update_levels(p4d_ctx* c, const double* svar, const double* sch) {
     for (int h = 0; h < kNH; ++h) m.p[h] = C.mask[h];
     ::p4d::count_launch(), k_dense0<<<dim3(nblocks(C.n), kNH), kBlock, 0, c->stream>>>(c->g, c->Jst, c->sfix, svar, m, sf[0], sf[1], sf[2],
                                                                  mats);
-  } else {
-    Ptr4<const double> F;
-    Ptr4<const TV> V;
-    for (int h = 0; h < kNH; ++h) {
+  }
+  // the inverse (into mats; work: the factors)
+  const int n = (int)C.n;
+  DenseRows dr{};
+  dr.d = dims(C);
+  Ptr4<const double> F{};
+  Ptr4<const TV> V{};
+  for (int h = 0; h < kNH; ++h) {
+    dr.sc[h] = sch[h];
+    if (c->nlev > 1) {
       F.p[h] = C.Ffix + (size_t)h * 27 * C.n;
       V.p[h] = (const TV*)C.Vvar + (size_t)h * 27 * C.n;
     }
-    ::p4d::count_launch(), k_dense<TV><<<dim3(nblocks(C.n), kNH), kBlock, 0, c->stream>>>(dims(C), F, V, sch[0], sch[1], sch[2], sch[3], mats);
   }
-  P4D_TRYS(coarse_inverse(c, C, mats, work));
+  if (n <= kLuMax) {
+    ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, lu_smem(n), c->stream>>>(n, dr, F, V, c->nlev == 1 ? mats : nullptr, work, C.perm);
+    ::p4d::count_launch(), k_lu_inverse<<<dim3((n + kLuCols - 1) / kLuCols, kNH), 32 * kLuCols, lu_smem(n), c->stream>>>(n, work, C.perm, mats);
+  } else {
+    if (c->nlev > 1)
+      ::p4d::count_launch(), k_dense<TV><<<dim3(nblocks(C.n), kNH), kBlock, 0, c->stream>>>(dims(C), F, V, sch[0], sch[1], sch[2], sch[3], mats);
+    ::p4d::count_launch(), k_gauss_jordan<<<kNH, 256, 0, c->stream>>>(n, mats, work);
+  }
   P4D_TRY(cudaGetLastError());
   return P4D_OK;
 }
@@ -2004,7 +2184,7 @@ p4d_status mg_update(p4d_ctx* c) {
   const double* sf = c->scale_f;
   const double sch[kNH] = {sf[0], sf[0], sf[1], sf[2]};
   double* svar = c->tmp;   // [3][nn] scratch (Krylov scratch is idle during an update)
-  for (int l = 0; l < c->nlev; ++l) P4D_TRY(cudaMemsetAsync(c->lev[l].lam, 0, kNH * sizeof(double), c->stream));
+  P4D_TRY(cudaMemsetAsync(c->lev[0].lam, 0, kNH * sizeof(double) * c->nlev, c->stream));   // one array over the levels
   MGLevel& l0 = c->lev[0];
   if (prec == 0)
     ::p4d::count_launch(), k_level0_update<double, double><<<nblocks(nn), kBlock, 0, c->stream>>>(
@@ -2023,22 +2203,20 @@ p4d_status mg_update(p4d_ctx* c) {
 }
 
 p4d_status mg_fetch_lam(p4d_ctx* c) {
-  for (int l = 0; l < c->nlev; ++l)
-    P4D_TRY(cudaMemcpyAsync(c->lam_pin + l * kNH, c->lev[l].lam, kNH * sizeof(double), cudaMemcpyDeviceToHost,
-                            c->stream));
-  P4D_TRY(cudaStreamSynchronize(c->stream));
+  P4D_TRY(cudaMemcpyAsync(c->lam_pin, c->lev[0].lam, kNH * sizeof(double) * c->nlev, cudaMemcpyDeviceToHost, c->stream));
+  P4D_TRYS(check_flags(c));   // (synchronizes the stream, once for both)
   for (int l = 0; l < c->nlev; ++l)
     for (int h = 0; h < kNH; ++h) c->lam_h[l][h] = c->lam_pin[l * kNH + h];
-  return cheb_upload(c);
+  return cheb_upload(c, true);
 }
 
 // Chebyshev(degree d) coefficients on [lam/ratio, lam] of D^-1 A for every
 // level, step and hierarchy (three-term recurrence of the shifted Chebyshev
 // polynomials), copied to the device table.
-p4d_status cheb_upload(p4d_ctx* c) {
+p4d_status cheb_upload(p4d_ctx* c, bool synced) {
   const double ratio = c->prm.cheb_ratio;
   double* t = c->cheb_pin;
-  P4D_TRY(cudaStreamSynchronize(c->stream));   // the previous copy from t has completed
+  if (!synced) P4D_TRY(cudaStreamSynchronize(c->stream));   // the previous copy from t has completed
   for (int l = 0; l < c->nlev; ++l)
     for (int h = 0; h < kNH; ++h) {
       const double lm = c->lam_h[l][h] > 0 ? c->lam_h[l][h] : 1.0;
@@ -2059,8 +2237,9 @@ p4d_status cheb_upload(p4d_ctx* c) {
   const size_t ne = (size_t)kMaxLevels * kMaxDeg * 3 * kNH;
   float* t32 = reinterpret_cast<float*>(t + ne);   // FP32 copy for the FP32 smoothers
   for (size_t q = 0; q < ne; ++q) t32[q] = (float)t[q];
-  P4D_TRY(cudaMemcpyAsync(c->cheb_dev, t, sizeof(double) * ne, cudaMemcpyHostToDevice, c->stream));
-  P4D_TRY(cudaMemcpyAsync(c->cheb_dev32, t32, sizeof(float) * ne, cudaMemcpyHostToDevice, c->stream));
+  // the smoothers read the table in their own precision
+  if (c->prm.precision == 0) P4D_TRY(cudaMemcpyAsync(c->cheb_dev, t, sizeof(double) * ne, cudaMemcpyHostToDevice, c->stream));
+  else P4D_TRY(cudaMemcpyAsync(c->cheb_dev32, t32, sizeof(float) * ne, cudaMemcpyHostToDevice, c->stream));
   return P4D_OK;
 }
 

@@ -484,7 +484,7 @@ p4d_status capture_graph(p4d_ctx* c, p4d_ctx::PcGraph& g, F&& body) {
   return P4D_OK;
 }
 void drop_graphs(p4d_ctx* c);
-p4d_status cheb_upload(p4d_ctx* c);
+p4d_status cheb_upload(p4d_ctx* c, bool synced = false);
 
 // ---- multigrid (mg.cu)
 p4d_status mg_plan(p4d_ctx* c);

