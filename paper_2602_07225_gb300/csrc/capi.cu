@@ -323,7 +323,7 @@ p4d_status setup_impl(p4d_ctx* c, const p4d_mesh* m, const p4d_params* prm) {
   P4D_TRYS(dalloc_t(c, &c->w, c->kry_len));
   P4D_TRYS(dalloc_t(c, &c->r0, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->nwork, (size_t)5 * c->ndof));
-  P4D_TRYS(dalloc_t(c, &c->nrm4, 4));
+  P4D_TRYS(dalloc_t(c, &c->nrm4, 8));
   P4D_TRYS(dalloc_t(c, &c->tmp, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->bred, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->part, (size_t)1024 * 136));

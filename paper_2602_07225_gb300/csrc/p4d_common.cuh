@@ -166,7 +166,7 @@ struct p4d_ctx {
   double* Rj = nullptr;                // [NE] particle radius
   double* nwork = nullptr;             // [4][ndof] Newton work (residual, step, trial state, trial residual)
   double gp_area = 0.0;                // area of Gamma_p
-  double* nrm4 = nullptr;              // [4] device scratch for Newton field norms
+  double* nrm4 = nullptr;              // [8] device scratch for Newton field norms
 
   // fixed FP64 stencils [4][27][nn]: 0 K_sigma (lifted), 1 K_kappa, 2 C = M_eps/dt + K_D, 3 M_eps/dt
   double* Jst = nullptr;
@@ -192,6 +192,7 @@ struct p4d_ctx {
   float* tfac32 = nullptr;             // FP32 copy of tfac (FP32 preconditioners)
   double* tloc = nullptr;              // [NE] node-local coupling scalar of the last operator application
   double* ujvp = nullptr;              // [nn] phi_e + gamma/c_e * c_e combination of a JVP input
+  bool diag_fixed = false;             // the interior particle rows of sqd, rsqd are in place
   double* sqd = nullptr;               // [ndof] sqrt(|diag J|)
   double* rsqd = nullptr;              // [ndof] 1 / sqrt(|diag J|)
   float* sqd32 = nullptr;              // [3 nn] the macro rows of sqd (its values are FP32 numbers)
