@@ -941,8 +941,9 @@ p4d_status fg_step_body(FgRun& r, int k, bool graph_precond, Tail t) {
   P4D_TRYS(precond_column(c, r.trans, graph_precond));   // k read from c->kdev
   prof_mark(c, 0);
   prof_mark(c, 1);
-  if (r.full) P4D_TRYS(jvp_full(c, zk, w, r.trans, nullptr, true, true));
-  else P4D_TRYS(jvp_reduced(c, zk, w, r.trans, nullptr, true, true));
+  const bool u = precond_leaves_u(c, r.trans);
+  if (r.full) P4D_TRYS(jvp_full(c, zk, w, r.trans, nullptr, true, u));
+  else P4D_TRYS(jvp_reduced(c, zk, w, r.trans, nullptr, true, u));
   prof_mark(c, 1);
   prof_mark(c, 2);
   const double* flag = misc + 2 * L.m + 6;

@@ -435,6 +435,19 @@ struct VRef {
   __device__ __forceinline__ double* get() const { return k ? base + stride * (int64_t)(*k) : base; }
 };
 
+// Input and output of a whole preconditioner application by the V-cycle's
+// single launch (mg.cu): rows of r (macro layout, scaled Krylov space) in,
+// rows of z out.
+struct TailIO {
+  int on = 0;
+  VRef r{}, z{};
+  const double* sqd = nullptr;
+  const float* sqd32 = nullptr;
+  const double* iwf = nullptr;
+  const uint8_t* label = nullptr;
+  double sc[3] = {1.0, 1.0, 1.0};
+};
+
 // ---- assembly / linearization (assemble.cu)
 p4d_status assemble_fixed(p4d_ctx* c, const double* eps, const double* eps_s, const uint8_t* region);
 p4d_status linearize(p4d_ctx* c, const p4d_state* st);
@@ -456,6 +469,8 @@ p4d_status precond_macro(p4d_ctx* c, const double* rm, double* zm, int transpose
 // Preconditioner applied to Krylov column *kdev of V into column *kdev of Z
 // (scaled space), through a CUDA graph unless profiling.
 p4d_status precond_column(p4d_ctx* c, int transpose, bool use_graph);
+// whether it leaves phi_e + gamma/c_e c_e of z_k in c->ujvp
+bool precond_leaves_u(const p4d_ctx* c, int transpose);
 
 // Captures what body() launches on c->stream into g (on c->cap_stream,
 // thread-local capture mode; launches are counted as g's kernel nodes).
@@ -494,6 +509,7 @@ p4d_status mg_update(p4d_ctx* c);
 p4d_status mg_fetch_lam(p4d_ctx* c);
 // run the V-cycles of the listed hierarchies on the level-0 right-hand sides already in place
 p4d_status mg_vcycle(p4d_ctx* c, const int* hs, int nhs);
+p4d_status mg_apply_tail(p4d_ctx* c, VRef r, VRef z);
 // whether the first Chebyshev step of level 0 comes with the right-hand side
 // (into d and x2): level 0 is smoothed by launches of its own
 inline bool mg_first_by_load(const p4d_ctx* c) { return c->nlev > 1 && c->tail_l0 != 0; }

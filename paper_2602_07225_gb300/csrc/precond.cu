@@ -325,6 +325,11 @@ PcArgs make_pc(p4d_ctx* c) {
 // fields of the multigrid hierarchies
 const int kHOfField[3][2] = {{0, 1}, {2, -1}, {3, -1}};
 
+// The reduced block-Jacobi application of a cell whose V-cycles are one launch.
+bool whole_in_tail(const p4d_ctx* c, bool full, bool scaled) {
+  return c->tail_l0 == 0 && c->prm.combine == 0 && !full && scaled;
+}
+
 template <typename T, bool TRANS, bool FULL>
 p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
   PcArgs a = make_pc(c);
@@ -347,7 +352,9 @@ p4d_status apply_t(p4d_ctx* c, VRef r, VRef z, bool scaled) {
     first.x[f] = (T*)l0.x2[hf[f]];
   }
   first.ctab = sizeof(T) == sizeof(double) ? (const T*)c->cheb_dev : (const T*)c->cheb_dev32;
-  if (c->prm.combine == 0) {
+  if (whole_in_tail(c, FULL, scaled)) {
+    P4D_TRYS(mg_apply_tail(c, r, z));
+  } else if (c->prm.combine == 0) {
     ::p4d::count_launch(), k_load<T, TRANS, FULL><<<nblocks(nn), kBlock, 0, c->stream>>>(a, r, yc, z, 7, 0, scaled, b[0], b[1], b[2], first);
     const int hs[4] = {0, 1, 2, 3};
     P4D_TRYS(mg_vcycle(c, hs, 4));
@@ -497,6 +504,10 @@ p4d_status precond_column(p4d_ctx* c, int transpose, bool use_graph) {
   count_launches(g.kernels);
   P4D_TRY(cudaGraphLaunch(g.exec, c->stream));
   return P4D_OK;
+}
+
+bool precond_leaves_u(const p4d_ctx* c, int transpose) {
+  return !transpose && !whole_in_tail(c, c->prm.mode == 0, true);
 }
 
 p4d_status particle_solve64(p4d_ctx* c, const double* rc, double* yc, const double* tN, int transpose) {
