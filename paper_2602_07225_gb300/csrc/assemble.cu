@@ -526,9 +526,10 @@ p4d_status linearize(p4d_ctx* c, const p4d_state* st) {
                                                           c->eidx, c->Aj, c->Mj, c->kapj, c->betaj, c->rref,
                                                           c->ge, c->gc, c->gs, c->sqd, c->rsqd, c->sqd32);
   c->diag_fixed = true;   // (stream order: set once the launch has been issued)
-  ::p4d::count_launch(), k_state_scale<<<4 * 152, kBlock, 0, c->stream>>>(nn, NE * nc, c->sqd, st->phis, st->phie, st->ce,
+  const int sb = nn <= 8192 ? (int)nblocks(c->ndof, 4 * kBlock) : 4 * 152;   // small cells: fewer partial sums
+  ::p4d::count_launch(), k_state_scale<<<sb, kBlock, 0, c->stream>>>(nn, NE * nc, c->sqd, st->phis, st->phie, st->ce,
                                                                          st->cs, c->part);
-  ::p4d::count_launch(), k_state_sum<<<1, 128, 0, c->stream>>>(c->part, 4 * 152, c->unorm2);
+  ::p4d::count_launch(), k_state_sum<<<1, 128, 0, c->stream>>>(c->part, sb, c->unorm2);
   P4D_TRY(cudaGetLastError());
   return P4D_OK;
 }

@@ -96,6 +96,11 @@ __device__ __forceinline__ double warp_sum(const double* p, int n, int lane) {
 // sums p[t], p[t + 256], ..., then a halving tree): lane l holds threads l,
 // l + 32, ..., l + 224.  Lane 0 has the result.
 __device__ __forceinline__ double warp_tree_sum(const double* p, int n, int lane) {
+  if (n <= 32) {   // one partial per lane at most: the tree above the lanes adds zeros
+    double t = lane < n ? __ldcg(p + lane) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    return t;
+  }
   double s[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -697,10 +702,11 @@ constexpr int64_t kSmallLen = 3 * 8192;
 
 struct Reducer {
   p4d_ctx* c;
-  // eight elements per thread; on the smallest vectors two (eight left 3
-  // blocks at 6,075 elements and 14 us per multi-dot)
+  // eight elements per thread; on the smallest vectors one: a warp's FP64
+  // instruction takes an SM's FP64 unit 20 clocks, so few elements per SM
+  // count (6,075 elements, 12 dots: 14 us with 3 blocks, 10 us with 12)
   int nblk(int64_t len) const {
-    const int64_t per = (int64_t)kRedThreads * (len <= kSmallLen ? 2 : 8);
+    const int64_t per = (int64_t)kRedThreads * (len <= kSmallLen ? 1 : 8);
     const int64_t want = (len + per - 1) / per;
     return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, want));
   }

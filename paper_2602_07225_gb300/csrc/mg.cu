@@ -695,10 +695,13 @@ __global__ void k_dense0(Grid g, const double* __restrict__ Jst, const double* _
 // substitution.  FP64 throughout.  Up to kLuSmem rows the matrix stays in
 // shared memory (rows padded by one entry); larger ones in global memory.  A
 // pivot step is a pivot search by one warp and the update of the rows below,
-// two block barriers; the elements of the multiplier column are formed by the
-// row's warp.  With the matrix in global memory and five barriers per step
-// the two kernels took 132 + 75 us at n = 63; the factorization is bound by
-// the FP64 rate of one SM (n^3 / 6 clocks) from n ~ 100 on.
+// four block barriers.  A warp's FP64 instruction occupies an SM's FP64 unit
+// for 20 clocks whatever its active lanes, so the trailing block is updated
+// as m^2 elements over full warps, one multiplication per multiplier, and
+// the substitutions divide through precomputed reciprocals.  A warp per row,
+// with the multiplier formed by every lane, and a division per row and
+// column took 145 + 75 us at 63 rows and 380 + 151 us at 120; this takes 111
+// + 50 and 353 + 107.
 constexpr int kLuMax = 256;
 constexpr int kLuSmem = 160;
 constexpr int kLuThreads = 512;
@@ -709,6 +712,11 @@ struct DenseRows {
   LevelDims d;
   double sc[kNH];
 };
+
+// Tests of doubles on their bits: a floating-point comparison is an FP64
+// instruction (20 clocks of an SM's FP64 unit per warp).
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 template <typename TV>
 __global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, Ptr4<const double> F, Ptr4<const TV> V,
@@ -755,14 +763,17 @@ __global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, P
   __syncthreads();
   for (int k = 0; k < n; ++k) {
     if (warp == 0) {
-      double best = -1.0;
+      // magnitudes compared as integers (the bits of non-negative doubles are
+      // ordered; a NaN is never chosen), the first of equal ones
+      long long best = -1;
       int idx = k;
       for (int r = k + lane; r < n; r += 32) {
-        const double v = fabs(A[(size_t)r * ld + k]);
+        long long v = __double_as_longlong(A[(size_t)r * ld + k]) & 0x7fffffffffffffffll;
+        if (v > 0x7ff0000000000000ll) v = -1;
         if (v > best) { best = v; idx = r; }
       }
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
         if (ob > best || (ob == best && oi < idx)) { best = ob; idx = oi; }
       }
@@ -787,13 +798,22 @@ __global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, P
       }
       __syncthreads();
     }
+    // multipliers, one row per thread
     const double id = inv_d;
-    for (int r = k + 1 + warp; r < n; r += nw) {
-      const double l = A[(size_t)r * ld + k] * id;
-      __syncwarp();
-      if (lane == 0) A[(size_t)r * ld + k] = l;
-      if (l == 0.0) continue;
-      for (int cc = k + 1 + lane; cc < n; cc += 32) A[(size_t)r * ld + cc] -= l * A[(size_t)k * ld + cc];
+    const int m = n - k - 1;
+    for (int r = threadIdx.x; r < m; r += blockDim.x) A[(size_t)(k + 1 + r) * ld + k] *= id;
+    __syncthreads();
+    // the trailing block, its m x m elements spread evenly over the lanes
+    const float rm = 1.0f / (float)max(1, m);
+    const double* rowk = A + (size_t)k * ld + k + 1;
+    for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+      int r = (int)((float)q * rm);   // q / m up to one, corrected (q < 2^16)
+      int cc = q - r * m;
+      if (cc < 0) { --r; cc += m; }
+      else if (cc >= m) { ++r; cc -= m; }
+      double* row = A + (size_t)(k + 1 + r) * ld;
+      const double l = row[k];
+      if (l != 0.0) row[k + 1 + cc] -= l * rowk[cc];
     }
     __syncthreads();
   }
@@ -802,23 +822,36 @@ __global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, P
       for (int cc = lane; cc < n; cc += 32) G[(size_t)r * n + cc] = A[(size_t)r * ld + cc];
 }
 
-// Columns of the inverse: four warps of a block, a column each at a time.
+// x / d from r = 1 / d (correctly rounded): one Newton correction of the
+// quotient by its exact remainder gives the correctly rounded quotient
+// (Markstein 1990) in three FP64 operations.
+__device__ __forceinline__ double div_by(double x, double d, double r) {
+  const double q = x * r;
+  return finite_bits(q) && finite_bits(r) ? fma(fma(-q, d, x), r, q) : x / d;
+}
+
+// Columns of the inverse, a column per warp.
 constexpr int kLuCols = 4;
+template <bool SM>
 __global__ void __launch_bounds__(32 * kLuCols) k_lu_inverse(int n, const double* __restrict__ lu,
                                                              const int* __restrict__ perm, double* __restrict__ inv) {
   extern __shared__ double lu_s[];
   __shared__ double xs[kLuCols][kLuMax];
-  __shared__ double rd[kLuMax];   // the diagonal
+  __shared__ double dg[kLuMax], rd[kLuMax];   // the diagonal and its reciprocals
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * kLuCols + warp;
   const double* G = lu + (size_t)blockIdx.y * n * n;
-  const bool sm = n <= kLuSmem;
-  const int ld = sm ? n + 1 : n;
-  if (sm)
+  const int ld = SM ? n + 1 : n;
+  if (SM)
+#pragma unroll 4
     for (int r = warp; r < n; r += kLuCols)
-      for (int cc = lane; cc < n; cc += 32) lu_s[(size_t)r * ld + cc] = G[(size_t)r * n + cc];
-  const double* A = sm ? lu_s : G;
-  for (int r = threadIdx.x; r < n; r += blockDim.x) rd[r] = G[(size_t)r * n + r];
+      for (int cc = lane; cc < n; cc += 32) lu_s[r * ld + cc] = G[(size_t)r * n + cc];
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    const double d = G[(size_t)r * n + r];
+    dg[r] = d;
+    rd[r] = d != 0.0 ? 1.0 / d : 0.0;
+  }
+  const double* A = SM ? lu_s : G;
   __syncthreads();
   if (j >= n) return;   // per warp
   const int* P = perm + (size_t)blockIdx.y * n;
@@ -835,16 +868,18 @@ __global__ void __launch_bounds__(32 * kLuCols) k_lu_inverse(int n, const double
   for (int k = k0; k < n - 1; ++k) {   // x is zero above its unit entry
     const double xk = x[k];
     __syncwarp();
-    if (xk != 0.0)
-      for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[(size_t)i * ld + k] * xk;
+    if (nonzero(xk))
+#pragma unroll 1
+      for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[i * ld + k] * xk;
     __syncwarp();
   }
   for (int k = n - 1; k >= 0; --k) {
-    const double d = rd[k], xk = d != 0.0 ? x[k] / d : 0.0;
+    const double d = dg[k], xk = nonzero(d) ? div_by(x[k], d, rd[k]) : 0.0;
     __syncwarp();
     if (lane == 0) x[k] = xk;
-    if (xk != 0.0)
-      for (int i = lane; i < k; i += 32) x[i] -= A[(size_t)i * ld + k] * xk;
+    if (nonzero(xk))
+#pragma unroll 1
+      for (int i = lane; i < k; i += 32) x[i] -= A[i * ld + k] * xk;
     __syncwarp();
   }
   double* Inv = inv + (size_t)blockIdx.y * n * n;
@@ -1975,7 +2010,7 @@ p4d_status mg_plan(p4d_ctx* c) {
   // process-wide attributes: the largest sizes the kernels use
   P4D_TRY(cudaFuncSetAttribute(k_lu_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
   P4D_TRY(cudaFuncSetAttribute(k_lu_factor<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
-  P4D_TRY(cudaFuncSetAttribute(k_lu_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
+  P4D_TRY(cudaFuncSetAttribute(k_lu_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
   if (c->lev[L - 1].n > 4096) return P4D_ERR_INVALID_ARG;   // coarsest level too large for a dense inverse
   P4D_TRYS(tail_plan(c));
   double* lam = nullptr;
@@ -2200,8 +2235,15 @@ p4d_status mg_update_levels(p4d_ctx* c, const double* svar, const double* sch) {
     }
   }
   if (n <= kLuMax) {
-    ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, lu_smem(n), c->stream>>>(n, dr, F, V, c->nlev == 1 ? mats : nullptr, work, C.perm);
-    ::p4d::count_launch(), k_lu_inverse<<<dim3((n + kLuCols - 1) / kLuCols, kNH), 32 * kLuCols, lu_smem(n), c->stream>>>(n, work, C.perm, mats);
+    const double* dense = c->nlev == 1 ? mats : nullptr;
+    const dim3 gi((n + kLuCols - 1) / kLuCols, kNH);
+    if (n <= kLuSmem) {
+      ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, lu_smem(n), c->stream>>>(n, dr, F, V, dense, work, C.perm);
+      ::p4d::count_launch(), k_lu_inverse<true><<<gi, 32 * kLuCols, lu_smem(n), c->stream>>>(n, work, C.perm, mats);
+    } else {
+      ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, 0, c->stream>>>(n, dr, F, V, dense, work, C.perm);
+      ::p4d::count_launch(), k_lu_inverse<false><<<gi, 32 * kLuCols, 0, c->stream>>>(n, work, C.perm, mats);
+    }
   } else {
     if (c->nlev > 1)
       ::p4d::count_launch(), k_dense<TV><<<dim3(nblocks(C.n), kNH), kBlock, 0, c->stream>>>(dims(C), F, V, sch[0], sch[1], sch[2], sch[3], mats);
