@@ -357,10 +357,10 @@ __global__ void k_fixed_sums(Grid g, const double* __restrict__ Jst, const uint8
   }
 }
 
-// Nonlinear residual (paper section 4, block residual) -- macro rows.  Every
-// neighbour is loaded without a test, as in k_jvp_macro: the stencils hold
-// exact zeros for neighbours outside the grid and, for phi_s, without an
-// unknown.
+// Nonlinear residual (paper section 4, block residual) -- macro rows.  A
+// stencil line's loads are issued together, without a branch; neighbours
+// outside the grid and, for phi_s, without an unknown are left out by
+// selects (their slots hold exact zeros, but 0 x Inf is NaN).
 __global__ void __launch_bounds__(128) k_residual_macro(Grid g, Kin kn, const double* __restrict__ Jst,
                                  const uint8_t* __restrict__ label, const int32_t* __restrict__ eidx,
                                  const double* __restrict__ Aj, const double* __restrict__ gpw,
@@ -373,6 +373,8 @@ __global__ void __launch_bounds__(128) k_residual_macro(Grid g, Kin kn, const do
   const int64_t nn = g.nn;
   const int N = (int)nn;
   if (n >= N) return;
+  const int q = (unsigned)n / (unsigned)g.nnx;
+  const int i = n - q * g.nnx, k = (unsigned)q / (unsigned)g.nny, j = q - k * g.nny;
   const int32_t e = eidx[n];
   const double ain = e >= 0 ? Aj[e] * rin[e] : 0.0;
   const bool act = label[n] & kLabActive;
@@ -394,23 +396,27 @@ __global__ void __launch_bounds__(128) k_residual_macro(Grid g, Kin kn, const do
   double s = act ? sfix[n] * pn : 0.0, se = 0.0, sc = 0.0;
 #pragma unroll
   for (int l = 0; l < 9; ++l) {
+    const int jj = j + l % 3 - 1, kz = k + l / 3 - 1;
+    const bool line = (unsigned)jj < (unsigned)g.nny && (unsigned)kz < (unsigned)g.nnz;
     const int mid = n + g.nnx * ((l % 3 - 1) + g.nny * (l / 3 - 1));
     double ks[3], kk[3], cc[3], mm[3], vs[3], vu[3], vc[3], vd[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int o = 3 * l + d;
-      const int m = min(max(mid + d - 1, 0), N - 1);
+      // no product with a neighbour outside the grid or (phi_s) inactive: 0 x Inf is NaN
+      const bool in = line && (unsigned)(i + d - 1) < (unsigned)g.nnx;
+      const int m = in ? mid + d - 1 : n;
       if (act) {
         ks[d] = Ks[o * N + n];
-        vs[d] = phis[m];
+        vs[d] = in && (label[m] & kLabActive) ? phis[m] : pn;
       }
       mm[d] = Mm[o * N + n];
-      vd[d] = dce[m];
+      vd[d] = in ? dce[m] : 0.0;
       if (!trows) {
         kk[d] = Kk[o * N + n];
-        vu[d] = ue[m];
+        vu[d] = in ? ue[m] : 0.0;
         cc[d] = Cc[o * N + n];
-        vc[d] = ce[m];
+        vc[d] = in ? ce[m] : 0.0;
       }
     }
 #pragma unroll

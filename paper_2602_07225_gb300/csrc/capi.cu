@@ -327,6 +327,7 @@ p4d_status setup_impl(p4d_ctx* c, const p4d_mesh* m, const p4d_params* prm) {
   P4D_TRYS(dalloc_t(c, &c->tmp, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->bred, c->ndof));
   P4D_TRYS(dalloc_t(c, &c->part, (size_t)1024 * 136));
+  P4D_TRYS(dalloc_t(c, &c->nzflag, 1));
   P4D_TRYS(dalloc_t(c, &c->red_cnt, 1));
   P4D_TRY(cudaMemset(c->red_cnt, 0, sizeof(unsigned)));
   P4D_TRYS(dalloc_t(c, &c->hs, (size_t)(c->mcap + 2) * (c->mcap + 8) + 64));

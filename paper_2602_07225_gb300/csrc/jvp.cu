@@ -11,6 +11,7 @@
 //
 // Output forms: y = sc .* (J x) or y = sc .* (b - J x), sc = w_f / sqrt(d) in
 // the scaled Krylov space, 1 otherwise.
+#include <algorithm>
 #include <mutex>
 #include "p4d_common.cuh"
 
@@ -29,6 +30,7 @@ struct JvpArgs {
   const double *ge, *gc, *gs, *zeta, *gdc, *rsqd, *wf;
   double* tloc;
   const double* u;     // optional precombined phi_e + gamma/c_e * c_e of the input (non-transposed)
+  const unsigned* nz;  // GATED: *nz == 0 says that the input is all zeros
 };
 
 __device__ __forceinline__ double outscale(const JvpArgs& a, bool scaled, int f, int64_t row) {
@@ -44,12 +46,20 @@ __global__ void k_jvp_combine(int64_t nn, const double* __restrict__ x, const do
   u[n] = fma(gdc[n], x[2 * nn + n], x[nn + n]);
 }
 
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
 // Macro rows.  reduced: Schur operator on [phi_s | phi_e | c_e] only.
 // Large cells are bound by the FP64 rate, small ones by the latency of the
 // loads: every neighbour is loaded without a test (the stencils hold exact
 // zeros in the slots of neighbours outside the grid, the index is clamped to
 // the vector), one stencil line of three offsets at a time.
-template <bool TRANS, bool REDUCED>
+// CHECK: an entry that is not finite must not reach a row that it does not
+// couple to (0 x Inf is NaN): a row that ends non-finite is summed again with
+// the tests.  The Krylov solves, whose vectors are finite or end the solve,
+// go without (reduced product 10.1 instead of 12.3 us on 2,025 nodes, 271
+// instead of 293 us on 129 x 129 x 97).
+// GATED: see jvp_start.
+template <bool TRANS, bool REDUCED, bool GATED = false, bool CHECK = false>
 __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __restrict__ x,
                                                    const double* __restrict__ b, double* __restrict__ y,
                                                    bool scaled) {
@@ -57,6 +67,11 @@ __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __re
   const int n = blockIdx.x * blockDim.x + threadIdx.x;   // 27 nn < 2^31 (checked at setup)
   const int N = (int)nn;
   if (n >= N) return;
+  if (GATED && *a.nz == 0) {
+#pragma unroll
+    for (int f = 0; f < 3; ++f) y[f * nn + n] = outscale(a, scaled, f, f * nn + n) * b[f * nn + n];
+    return;
+  }
   const double* xs = x;
   const double* xe = x + nn;
   const double* xc = x + 2 * nn;
@@ -92,36 +107,55 @@ __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __re
       yc += k2[d] * v2[d];
     }
   }
-  if (TRANS) yc += a.gdc[n] * ye;   // (K_kappa diag(gamma/c_e))^T = diag(gamma/c_e) K_kappa
-  if (!act) ys = xs[n];
-  const int32_t e = a.eidx[n];
-  if (e >= 0) {
-    const double A = a.Aj[e];
-    const double ge = a.ge[e];
-    if (!TRANS) {
-      // t = v . x  (c_s surface value only in the full operator)
-      double t = (act ? ge * xs[n] : 0.0) - ge * xe[n] + a.gc[e] * xc[n];
-      if (REDUCED) t *= a.zeta[e];
-      else t += a.gs[e] * x[3 * nn + (int64_t)e * a.nc + a.nc - 1];
-      if (act) ys += A * t;
-      ye -= A * t;
-      yc -= a.tau * A * t;
-      if (!REDUCED) a.tloc[e] = t;
-    } else {
-      // t = u . x
-      double t = (act ? A * xs[n] : 0.0) - A * xe[n] - a.tau * A * xc[n];
-      if (REDUCED) t *= a.zeta[e];
-      else t += a.Mj[e] * a.betaj[e] * x[3 * nn + (int64_t)e * a.nc + a.nc - 1];
-      if (act) ys += ge * t;
-      ye -= ge * t;
-      yc += a.gc[e] * t;
-      if (!REDUCED) a.tloc[e] = t;
+  auto couple = [&] {
+    if (TRANS) yc += a.gdc[n] * ye;   // (K_kappa diag(gamma/c_e))^T = diag(gamma/c_e) K_kappa
+    if (!act) ys = xs[n];
+    const int32_t e = a.eidx[n];
+    if (e >= 0) {
+      const double A = a.Aj[e];
+      const double ge = a.ge[e];
+      if (!TRANS) {
+        // t = v . x  (c_s surface value only in the full operator)
+        double t = (act ? ge * xs[n] : 0.0) - ge * xe[n] + a.gc[e] * xc[n];
+        if (REDUCED) t *= a.zeta[e];
+        else t += a.gs[e] * x[3 * nn + (int64_t)e * a.nc + a.nc - 1];
+        if (act) ys += A * t;
+        ye -= A * t;
+        yc -= a.tau * A * t;
+        if (!REDUCED) a.tloc[e] = t;
+      } else {
+        // t = u . x
+        double t = (act ? A * xs[n] : 0.0) - A * xe[n] - a.tau * A * xc[n];
+        if (REDUCED) t *= a.zeta[e];
+        else t += a.Mj[e] * a.betaj[e] * x[3 * nn + (int64_t)e * a.nc + a.nc - 1];
+        if (act) ys += ge * t;
+        ye -= ge * t;
+        yc += a.gc[e] * t;
+        if (!REDUCED) a.tloc[e] = t;
+      }
     }
-  }
-  if (b) {
-    ys = b[n] - ys;
-    ye = b[nn + n] - ye;
-    yc = b[2 * nn + n] - yc;
+    if (b) {
+      ys = b[n] - ys;
+      ye = b[nn + n] - ye;
+      yc = b[2 * nn + n] - yc;
+    }
+  };
+  couple();
+  if (CHECK && !(finite_bits(ys) && finite_bits(ye) && finite_bits(yc))) {
+    const int q = n / a.g.nnx, i = n - q * a.g.nnx, k = q / a.g.nny, j = q - k * a.g.nny;
+    ys = ye = yc = 0.0;
+#pragma unroll 1
+    for (int o = 0; o < 27; ++o) {
+      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+      if ((unsigned)(i + dx) >= (unsigned)a.g.nnx || (unsigned)(j + dy) >= (unsigned)a.g.nny ||
+          (unsigned)(k + dz) >= (unsigned)a.g.nnz)
+        continue;
+      const int m = n + dx + a.g.nnx * (dy + a.g.nny * dz);
+      if (act) ys += Ks[o * N + n] * xs[m];
+      ye += Kk[o * N + n] * (comb ? fma(a.gdc[m], xc[m], ue[m]) : ue[m]);
+      yc += Cc[o * N + n] * xc[m];
+    }
+    couple();
   }
   y[n] = outscale(a, scaled, 0, n) * ys;
   y[nn + n] = outscale(a, scaled, 1, nn + n) * ye;
@@ -165,6 +199,7 @@ JvpArgs make_args(p4d_ctx* c) {
   a.ge = c->ge; a.gc = c->gc; a.gs = c->gs; a.zeta = c->zeta; a.gdc = c->gdc; a.rsqd = c->rsqd; a.wf = c->wf;
   a.tloc = c->tloc;
   a.u = nullptr;
+  a.nz = nullptr;
   return a;
 }
 
@@ -197,14 +232,48 @@ p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const
   const int64_t nn = c->g.nn;
   const int bt = jvp_threads(nn);
   if (!transpose) jvp_input(c, a, x, u_ready);
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
-  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
+  auto k = scaled ? (transpose ? k_jvp_macro<true, false> : k_jvp_macro<false, false>)
+                  : (transpose ? k_jvp_macro<true, false, false, true> : k_jvp_macro<false, false, false, true>);
+  ::p4d::count_launch(), k<<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
   if (c->NE > 0) {
     const int64_t np = c->NE * c->nc;
     if (transpose) ::p4d::count_launch(), k_jvp_particle<true><<<nblocks(np), kBlock, 0, c->stream>>>(a, x, b, y, scaled);
     else ::p4d::count_launch(), k_jvp_particle<false><<<nblocks(np), kBlock, 0, c->stream>>>(a, x, b, y, scaled);
   }
   P4D_TRYS(transport_jvp(c, x, y, transpose, b, scaled));
+  P4D_TRY(cudaGetLastError());
+  return P4D_OK;
+}
+
+// Whether any entry of x[0..n) is not zero, into *nz (zeroed before).
+__global__ void __launch_bounds__(kBlock) k_nonzero(const double* __restrict__ x, int64_t n, unsigned* __restrict__ nz) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  long long any = 0;
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) any |= __double_as_longlong(x[i + q * stride]);
+  for (; i < n; i += stride) any |= __double_as_longlong(x[i]);
+  if (__any_sync(0xffffffffu, any != 0) && (threadIdx.x & 31) == 0) atomicOr(nz, 1u);
+}
+
+// Residual of the first restart cycle in the reduced mode: y = sc (b - J x).
+// Solves start from x = 0 as a rule; the product, FP64 bound, is then left
+// out: one pass over x finds out (65 x 65 x 49 nodes 45.8 us of product
+// against 4.5 us of pass and 5.8 us of y = sc b; 129 x 129 x 97 nodes 270
+// against 12 and 23 us).  Up to 8,192 nodes the product takes 10 us, no more
+// than the pass with its launch.
+p4d_status jvp_start(p4d_ctx* c, const double* x, double* y, int transpose, const double* b) {
+  const int64_t nn = c->g.nn;
+  if (nn <= 8192 || c->prm.transport_model != 0) return jvp_reduced(c, x, y, transpose, b, true);
+  P4D_TRY(cudaMemsetAsync(c->nzflag, 0, sizeof(unsigned), c->stream));
+  ::p4d::count_launch(), k_nonzero<<<std::min<unsigned>(nblocks(3 * nn, 4 * kBlock), 8 * 152), kBlock, 0, c->stream>>>(x, 3 * nn, c->nzflag);
+  JvpArgs a = make_args(c);
+  a.nz = c->nzflag;
+  const int bt = jvp_threads(nn);
+  if (!transpose) jvp_input(c, a, x, false);
+  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, true);
+  else ::p4d::count_launch(), k_jvp_macro<false, true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, true);
   P4D_TRY(cudaGetLastError());
   return P4D_OK;
 }
@@ -275,8 +344,8 @@ extern "C" p4d_status p4d_jvp_noalloc(p4d_handle h, const double* x, double* y, 
   JvpArgs a = make_args(h);
   a.tloc = tloc;   // each entry read by the particle rows is written first by the macro rows
   const int64_t nn = h->g.nn;
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
-  else ::p4d::count_launch(), k_jvp_macro<false, false><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
+  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false, false, true><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
+  else ::p4d::count_launch(), k_jvp_macro<false, false, false, true><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
   if (h->NE > 0) {
     const int64_t np = h->NE * h->nc;
     if (transpose) ::p4d::count_launch(), k_jvp_particle<true><<<nblocks(np), kBlock, 0, h->stream>>>(a, x, nullptr, y, false);

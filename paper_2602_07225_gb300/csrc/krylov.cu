@@ -899,6 +899,7 @@ p4d_status fg_cycle_launch(FgRun& r, bool gate = false) {
   const HLay& L = r.L;
   ++r.restarts;
   if (r.full) P4D_TRYS(jvp_full(c, r.x, c->V, r.trans, r.bk, true));
+  else if (r.restarts == 1) P4D_TRYS(jvp_start(c, r.x, c->V, r.trans, r.bk));
   else P4D_TRYS(jvp_reduced(c, r.x, c->V, r.trans, r.bk, true));
   R.mdot(c->V, 0, 0, c->V, r.len, true, misc + 2 * L.m + 2);
   Tail t;

@@ -241,6 +241,7 @@ struct p4d_ctx {
   double* tmp = nullptr;               // [ndof]
   double* bred = nullptr;              // [ndof] reduced right-hand side / scratch
   double* part = nullptr;              // block partial sums of a reduction
+  unsigned* nzflag = nullptr;          // whether a solve's initial guess has a nonzero entry
   unsigned* red_cnt = nullptr;         // blocks of the running reduction that have finished (0 between launches)
   double* hs = nullptr;                // device Hessenberg / Givens state
   double* hs_h = nullptr;              // pinned host mirror of small scalars
@@ -461,6 +462,8 @@ p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const
                     bool scaled, bool u_ready = false);
 p4d_status jvp_reduced(p4d_ctx* c, const double* x, double* y, int transpose, const double* b,
                        bool scaled, bool u_ready = false);
+
+p4d_status jvp_start(p4d_ctx* c, const double* x, double* y, int transpose, const double* b);
 
 // ---- particle elimination (particle.cu)
 p4d_status particle_solve64(p4d_ctx* c, const double* rc, double* yc, const double* tN, int transpose);
