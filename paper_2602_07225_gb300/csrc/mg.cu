@@ -690,22 +690,34 @@ __global__ void k_dense0(Grid g, const double* __restrict__ Jst, const double* _
 }
 
 // Coarsest-level inverse, n <= kLuMax: LU with partial pivoting of each
-// hierarchy's matrix in one block (perm[i] = the original row now at row i),
-// then the columns of the inverse, one warp each, by forward and backward
-// substitution.  FP64 throughout.  Up to kLuSmem rows the matrix stays in
-// shared memory (rows padded by one entry); larger ones in global memory.  A
-// pivot step is a pivot search by one warp and the update of the rows below,
-// four block barriers.  A warp's FP64 instruction occupies an SM's FP64 unit
-// for 20 clocks whatever its active lanes, so the trailing block is updated
-// as m^2 elements over full warps, one multiplication per multiplier, and
-// the substitutions divide through precomputed reciprocals.  A warp per row,
-// with the multiplier formed by every lane, and a division per row and
-// column took 145 + 75 us at 63 rows and 380 + 151 us at 120; this takes 111
-// + 50 and 353 + 107.
+// hierarchy's matrix by a cluster of kLuBlocks blocks (perm[i] = the original
+// row now at row i; the factors leave column by column), then the columns of
+// the inverse, one warp each, by forward and backward substitution.  FP64
+// throughout.
+//
+// Factorization: panels of kLuPanel columns, panel b in the shared memory of
+// block b mod kLuBlocks, a row per thread.  Rows stay where they are; their
+// positions move.  The owner factors a panel in registers (a step: pivot
+// search over the warps, one division, the updates left in the panel) and
+// sends the multipliers and pivots to all blocks, one cluster barrier per
+// panel.  The owner of the next panel updates that one first and factors it
+// while the others update the rest, so that the chain is the n pivot steps.
+// An FP64 instruction of a warp occupies its scheduler's FP64 unit for 64
+// clocks whatever its lanes: the rows are spread over the warps, and each
+// warp forms the reciprocal itself (352 clocks).  Every entry sees the same
+// operations in the same order as in the plain row-by-row elimination (a zero
+// multiplier is skipped).  One block per hierarchy, all of the trailing block
+// by it, took 111 us at 63 rows and 353 us at 120; the panel in one warp 104
+// and 267, clusters of 8 with a second block barrier per step 102 and 219;
+// this takes 94 and 214.
 constexpr int kLuMax = 256;
-constexpr int kLuSmem = 160;
-constexpr int kLuThreads = 512;
-inline size_t lu_smem(int n) { return n <= kLuSmem ? sizeof(double) * n * (n + 1) : 0; }
+constexpr int kLuBlocks = 4;
+constexpr int kLuPanel = 4;
+inline int lu_panels(int n) { return (n + kLuPanel - 1) / kLuPanel; }
+inline int lu_threads(int n) { return (n + 31) / 32 * 32; }
+inline size_t lu_smem(int n) {   // own columns, and three panels of multipliers
+  return sizeof(double) * n * (size_t)kLuPanel * ((lu_panels(n) + kLuBlocks - 1) / kLuBlocks + 3);
+}
 
 // Row n of the dense scaled coarsest operator, from difference form.
 struct DenseRows {
@@ -718,35 +730,52 @@ struct DenseRows {
 __device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
+__device__ __forceinline__ unsigned cluster_addr(const void* p, int rank) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  unsigned ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  return ra;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
+
 template <typename TV>
-__global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, Ptr4<const double> F, Ptr4<const TV> V,
-                                                          const double* __restrict__ mats, double* __restrict__ lu,
-                                                          int* __restrict__ perm) {
+__global__ void __cluster_dims__(kLuBlocks, 1, 1) __launch_bounds__(kLuMax)
+    k_lu_factor(int n, DenseRows dr, Ptr4<const double> F, Ptr4<const TV> V, const double* __restrict__ mats,
+                double* __restrict__ lu, int* __restrict__ perm) {
+  constexpr int NB = kLuPanel, C = kLuBlocks;
   extern __shared__ double lu_s[];
-  const int h = blockIdx.x;
-  double* G = lu + (size_t)h * n * n;
-  const bool sm = n <= kLuSmem;
-  double* A = sm ? lu_s : G;
-  const int ld = sm ? n + 1 : n;
-  int* P = perm + (size_t)h * n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __shared__ int piv;
-  __shared__ double inv_d;
-  if (mats) {
-    const double* A0 = mats + (size_t)h * n * n;
-    for (int r = warp; r < n; r += nw)
-      for (int cc = lane; cc < n; cc += 32) A[(size_t)r * ld + cc] = A0[(size_t)r * n + cc];
-  } else {
-    for (int r = warp; r < n; r += nw)
-      for (int cc = lane; cc < n; cc += 32) A[(size_t)r * ld + cc] = 0.0;
-    __syncthreads();
-    const double sc = pk(dr.sc, h);
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+  __shared__ int2 pivs[3][NB];               // (row, its position before) of a panel's pivots
+  __shared__ double U[kLuMax / C][NB];       // the pivot rows' entries in the own columns
+  // candidates of the warps for a pivot, two steps in turn: key, (row,
+  // position), the row's entries in the panel
+  __shared__ long long ckey[2][kLuMax / 32];
+  __shared__ int2 crow[2][kLuMax / 32];
+  __shared__ double cval[2][kLuMax / 32][NB];
+  const int h = blockIdx.x / C, rank = blockIdx.x % C;
+  const int r = threadIdx.x, lane = r & 31, warp = r >> 5, nw = blockDim.x >> 5;
+  const bool row = r < n;
+  const int np = (n + NB - 1) / NB;
+  const int nloc = rank < np ? (np - 1 - rank) / C + 1 : 0;   // own panels
+  double* A = lu_s;                                           // [own column][row]
+  double* L = lu_s + (size_t)n * NB * ((np + C - 1) / C);     // [3][NB][row]
+  if (row) {
+    for (int l = 0; l < nloc * NB; ++l) {
+      const int c = (l / NB * C + rank) * NB + l % NB;
+      A[l * n + r] = mats && c < n ? mats[((size_t)h * n + r) * n + c] : 0.0;
+    }
+    if (!mats) {
+      const double sc = pk(dr.sc, h);
       int i, j, k;
       node_ijk(dr.d, r, i, j, k);
       double a[27];
 #pragma unroll
       for (int o = 0; o < 27; ++o) a[o] = pk(F.p, h)[o * dr.d.n + r] + (double)pk(V.p, h)[o * dr.d.n + r];
+      auto put = [&](int c, double v) {
+        const int b = c / NB;
+        if (b % C == rank) A[(b / C * NB + c % NB) * n + r] = v;
+      };
       double diag = 0.0;
 #pragma unroll
       for (int o = 0; o < 27; ++o) {
@@ -754,72 +783,172 @@ __global__ void __launch_bounds__(kLuThreads) k_lu_factor(int n, DenseRows dr, P
         diag -= a[o];
         const int ii = i + o % 3 - 1, jj = j + (o / 3) % 3 - 1, kk = k + o / 9 - 1;
         if (ii < 0 || jj < 0 || kk < 0 || ii >= dr.d.nnx || jj >= dr.d.nny || kk >= dr.d.nnz) continue;
-        A[(size_t)r * ld + ii + dr.d.nnx * (jj + dr.d.nny * kk)] = sc * a[o];
+        put(ii + dr.d.nnx * (jj + dr.d.nny * kk), sc * a[o]);
       }
-      A[(size_t)r * ld + r] = sc * diag;
+      put(r, sc * diag);
     }
   }
-  for (int r = threadIdx.x; r < n; r += blockDim.x) P[r] = r;
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (warp == 0) {
+  int pos = r;
+
+  // Factors panel b (this block's, up to date) and sends it to all blocks.
+  auto factor = [&](int b) {
+    double* P = A + (size_t)(b / C * NB) * n;
+    int at = row ? pos : -1;
+    double v[NB];
+#pragma unroll
+    for (int m = 0; m < NB; ++m) v[m] = row ? P[m * n + r] : 0.0;
+#pragma unroll
+    for (int m = 0; m < NB; ++m) {
+      const int k = b * NB + m;
+      if (k >= n) continue;   // uniform
       // magnitudes compared as integers (the bits of non-negative doubles are
-      // ordered; a NaN is never chosen), the first of equal ones
-      long long best = -1;
-      int idx = k;
-      for (int r = k + lane; r < n; r += 32) {
-        long long v = __double_as_longlong(A[(size_t)r * ld + k]) & 0x7fffffffffffffffll;
-        if (v > 0x7ff0000000000000ll) v = -1;
-        if (v > best) { best = v; idx = r; }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ob > best || (ob == best && oi < idx)) { best = ob; idx = oi; }
-      }
-      if (lane == 0) {
-        piv = idx;
-        const double d = A[(size_t)idx * ld + k];
-        inv_d = d != 0.0 ? 1.0 / d : 0.0;
-      }
-    }
-    __syncthreads();
-    const int p = piv;
-    if (p != k) {   // uniform
-      for (int cc = threadIdx.x; cc < n; cc += blockDim.x) {
-        const double t = A[(size_t)k * ld + cc];
-        A[(size_t)k * ld + cc] = A[(size_t)p * ld + cc];
-        A[(size_t)p * ld + cc] = t;
-      }
-      if (threadIdx.x == 0) {
-        const int t = P[k];
-        P[k] = P[p];
-        P[p] = t;
+      // ordered; a NaN is never chosen), the row that comes first of equal ones
+      long long key = __double_as_longlong(v[m]) & 0x7fffffffffffffffll;
+      if (key > 0x7ff0000000000000ll) key = -1;
+      const bool cand = at >= k;
+      const int hi = cand ? (int)(key >> 32) : -2;
+      const int mh = __reduce_max_sync(0xffffffffu, hi);
+      const unsigned lo = cand && hi == mh ? (unsigned)key : 0u;
+      const unsigned ml = __reduce_max_sync(0xffffffffu, lo);
+      const bool top = cand && hi == mh && lo == ml;
+      const int mp = (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)at : 0xffffu);
+      if (mh == -2 ? lane == 0 : top && at == mp) {
+        ckey[m & 1][warp] = mh == -2 ? -2 : key;
+        crow[m & 1][warp] = make_int2(r, mp);
+#pragma unroll
+        for (int q = m; q < NB; ++q) cval[m & 1][warp][q] = v[q];
       }
       __syncthreads();
+      long long best = ckey[m & 1][0];
+      int2 bw = crow[m & 1][0];
+      int wb = 0;
+#pragma unroll 1
+      for (int w = 1; w < nw; ++w) {
+        const long long kw = ckey[m & 1][w];
+        const int2 cw = crow[m & 1][w];
+        if (kw > best || (kw == best && cw.y < bw.y)) { best = kw; bw = cw; wb = w; }
+      }
+      const double* u = cval[m & 1][wb];
+      const double d = u[m];
+      const double id = nonzero(d) ? 1.0 / d : 0.0;
+      if (r < C)
+        asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(cluster_addr(&pivs[b % 3][m], r)), "r"(bw.x),
+                     "r"(bw.y) : "memory");
+      if (at == bw.y) at = k;
+      else if (at == k) at = bw.y;
+      if (at > k) {
+        v[m] *= id;
+        if (nonzero(v[m])) {
+#pragma unroll
+          for (int q = m + 1; q < NB; ++q) v[q] = fma(-v[m], u[q], v[q]);
+        }
+      }
+      __syncwarp();
     }
-    // multipliers, one row per thread
-    const double id = inv_d;
-    const int m = n - k - 1;
-    for (int r = threadIdx.x; r < m; r += blockDim.x) A[(size_t)(k + 1 + r) * ld + k] *= id;
-    __syncthreads();
-    // the trailing block, its m x m elements spread evenly over the lanes
-    const float rm = 1.0f / (float)max(1, m);
-    const double* rowk = A + (size_t)k * ld + k + 1;
-    for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
-      int r = (int)((float)q * rm);   // q / m up to one, corrected (q < 2^16)
-      int cc = q - r * m;
-      if (cc < 0) { --r; cc += m; }
-      else if (cc >= m) { ++r; cc -= m; }
-      double* row = A + (size_t)(k + 1 + r) * ld;
-      const double l = row[k];
-      if (l != 0.0) row[k + 1 + cc] -= l * rowk[cc];
+    if (row) {
+#pragma unroll
+      for (int m = 0; m < NB; ++m) {
+        P[m * n + r] = v[m];
+        // a multiplier where the row's position is below the column's pivot
+        const double l = at > b * NB + m ? v[m] : 0.0;
+        double* dst = L + ((size_t)(b % 3) * NB + m) * n + r;
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+          asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(dst, q)), "d"(l) : "memory");
+      }
+    }
+  };
+
+  cluster_arrive();   // every block has started and written its columns
+  cluster_wait();
+  if (rank == 0) factor(0);
+  cluster_arrive();
+#pragma unroll 1
+  for (int b = 0; b < np; ++b) {
+    cluster_wait();
+    const double* Lb = L + (size_t)(b % 3) * NB * n;
+    double l[NB];
+    bool piv = false;
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      l[t] = row ? Lb[t * n + r] : 0.0;
+      if (b * NB + t >= n) continue;
+      const int2 p = pivs[b % 3][t];
+      if (r == p.x) {
+        pos = b * NB + t;
+        piv = true;
+      } else if (pos == b * NB + t) {
+        pos = p.y;
+      }
+    }
+    if (b + 1 == np) break;
+    // own columns after panel b; the first panel of them may be the next one
+    const int c0 = NB * (b < rank ? 0 : (b - rank) / C + 1), c1 = nloc * NB;
+    // the pivot rows' entries, a column per lane of the first warp
+    if (r < 32) {
+      for (int c = c0 + lane; c < c1; c += 32) {
+        double u[NB];
+#pragma unroll
+        for (int t = 0; t < NB; ++t) u[t] = A[c * n + pivs[b % 3][t].x];
+#pragma unroll
+        for (int t = 0; t < NB; ++t) {
+          const int p = pivs[b % 3][t].x;
+#pragma unroll
+          for (int q = 0; q < t; ++q) {
+            const double m = Lb[q * n + p];
+            if (nonzero(m)) u[t] = fma(-m, u[q], u[t]);
+          }
+          A[c * n + p] = u[t];
+          U[c][t] = u[t];
+        }
+      }
     }
     __syncthreads();
+    // every other row by its thread
+    bool on[NB], any[NB];
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      on[t] = !piv && nonzero(l[t]);
+      any[t] = __any_sync(0xffffffffu, on[t]);
+    }
+    auto update = [&](int e0, int e1) {
+#pragma unroll 4
+      for (int c = e0; c < e1; ++c) {
+        if (!row) break;
+        double w = A[c * n + r];
+#pragma unroll
+        for (int t = 0; t < NB; ++t)
+          if (any[t]) {
+            const double x = fma(-l[t], U[c][t], w);
+            w = on[t] ? x : w;
+          }
+        if (!piv) A[c * n + r] = w;
+      }
+    };
+    const bool mine = (b + 1) % C == rank;
+    if (mine) {
+      update(c0, c0 + NB);
+      factor(b + 1);
+      // (buffers of three panels: this block's work on panel b below is done
+      // when it arrives for panel b + 2)
+      cluster_arrive();
+      update(c0 + NB, c1);
+      // the pivot rows' entries of the next step are read and U is written
+      // by the first warp
+      __syncthreads();
+    } else {
+      update(c0, c1);
+      cluster_arrive();
+    }
   }
-  if (sm)
-    for (int r = warp; r < n; r += nw)
-      for (int cc = lane; cc < n; cc += 32) G[(size_t)r * n + cc] = A[(size_t)r * ld + cc];
+  double* G = lu + (size_t)h * n * n;
+  if (row) {
+    for (int l = 0; l < nloc * NB; ++l) {
+      const int c = (l / NB * C + rank) * NB + l % NB;
+      if (c < n) G[(size_t)c * n + pos] = A[l * n + r];
+    }
+    if (rank == 0) perm[(size_t)h * n + pos] = r;
+  }
 }
 
 // x / d from r = 1 / d (correctly rounded): one Newton correction of the
@@ -830,60 +959,102 @@ __device__ __forceinline__ double div_by(double x, double d, double r) {
   return finite_bits(q) && finite_bits(r) ? fma(fma(-q, d, x), r, q) : x / d;
 }
 
-// Columns of the inverse, a column per warp.
+// Columns of the inverse, a column per warp, its entries in registers (entry
+// lane + 32 t in x[t]).  A substitution step is a chain of a shuffle, (going
+// back) a quotient and an update; the factors' columns are loaded a batch
+// ahead, from the caches.  With the column in shared memory and the factors
+// staged there 50 us at 63 rows and 105 us at 120; now 32 and 68.
 constexpr int kLuCols = 4;
-template <bool SM>
+template <int NT>
 __global__ void __launch_bounds__(32 * kLuCols) k_lu_inverse(int n, const double* __restrict__ lu,
                                                              const int* __restrict__ perm, double* __restrict__ inv) {
-  extern __shared__ double lu_s[];
-  __shared__ double xs[kLuCols][kLuMax];
-  __shared__ double dg[kLuMax], rd[kLuMax];   // the diagonal and its reciprocals
+  constexpr int B = NT > 4 ? 2 : 4;           // factor columns of a batch
+  __shared__ double dg[32 * NT], rd[32 * NT];   // the diagonal and its reciprocals
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * kLuCols + warp;
-  const double* G = lu + (size_t)blockIdx.y * n * n;
-  const int ld = SM ? n + 1 : n;
-  if (SM)
-#pragma unroll 4
-    for (int r = warp; r < n; r += kLuCols)
-      for (int cc = lane; cc < n; cc += 32) lu_s[r * ld + cc] = G[(size_t)r * n + cc];
+  const double* G = lu + (size_t)blockIdx.y * n * n;   // [column][row]
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
     const double d = G[(size_t)r * n + r];
     dg[r] = d;
     rd[r] = d != 0.0 ? 1.0 / d : 0.0;
   }
-  const double* A = SM ? lu_s : G;
   __syncthreads();
   if (j >= n) return;   // per warp
   const int* P = perm + (size_t)blockIdx.y * n;
-  double* x = xs[warp];
   // x = P e_j, then L y = x (unit lower), then U x = y
+  double x[NT];
   int k0 = n;
-  for (int i = lane; i < n; i += 32) {
-    const bool one = P[i] == j;
-    x[i] = one ? 1.0 : 0.0;
+#pragma unroll
+  for (int t = 0; t < NT; ++t) {
+    const int i = lane + 32 * t;
+    const bool one = i < n && P[i] == j;
+    x[t] = one ? 1.0 : 0.0;
     if (one) k0 = i;
   }
-  for (int o = 16; o > 0; o >>= 1) k0 = min(k0, __shfl_xor_sync(0xffffffffu, k0, o));
-  __syncwarp();
-  for (int k = k0; k < n - 1; ++k) {   // x is zero above its unit entry
-    const double xk = x[k];
-    __syncwarp();
-    if (nonzero(xk))
+  k0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)k0);
+  double c[B][NT], cn[B][NT];
+  auto load = [&](int k, double (&d)[B][NT]) {   // factor columns k .. k + B - 1
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const int i = lane + 32 * t;
+        d[q][t] = k + q >= 0 && k + q < n && i < n ? __ldg(G + (size_t)(k + q) * n + i) : 0.0;
+      }
+  };
+  auto next = [&] {
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+#pragma unroll
+      for (int t = 0; t < NT; ++t) c[q][t] = cn[q][t];
+  };
+  const int kb = k0 / B * B;   // x is zero above its unit entry
+  load(kb, cn);
+#pragma unroll
+  for (int tb = 0; tb < NT; ++tb) {
 #pragma unroll 1
-      for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[i * ld + k] * xk;
-    __syncwarp();
+    for (int k = max(kb, 32 * tb); k < min(n, 32 * tb + 32); k += B) {
+      next();
+      load(k + B, cn);
+#pragma unroll
+      for (int q = 0; q < B; ++q) {
+        const double xk = __shfl_sync(0xffffffffu, x[tb], (k + q) & 31);
+        if (nonzero(xk)) {   // uniform
+          const double v = fma(-c[q][tb], xk, x[tb]);
+          if (lane > ((k + q) & 31)) x[tb] = v;
+#pragma unroll
+          for (int t = tb + 1; t < NT; ++t) x[t] = fma(-c[q][t], xk, x[t]);
+        }
+      }
+    }
   }
-  for (int k = n - 1; k >= 0; --k) {
-    const double d = dg[k], xk = nonzero(d) ? div_by(x[k], d, rd[k]) : 0.0;
-    __syncwarp();
-    if (lane == 0) x[k] = xk;
-    if (nonzero(xk))
+  load((n - 1) / B * B, cn);
+#pragma unroll
+  for (int tb = NT - 1; tb >= 0; --tb) {
 #pragma unroll 1
-      for (int i = lane; i < k; i += 32) x[i] -= A[i * ld + k] * xk;
-    __syncwarp();
+    for (int k = (min(n, 32 * tb + 32) - 1) / B * B; k >= 32 * tb; k -= B) {
+      next();
+      load(k - B, cn);
+#pragma unroll
+      for (int q = B - 1; q >= 0; --q) {
+        if (k + q >= n) continue;
+        const double d = dg[k + q];
+        double xk = __shfl_sync(0xffffffffu, x[tb], (k + q) & 31);
+        xk = nonzero(d) ? div_by(xk, d, rd[k + q]) : 0.0;
+        if (lane == ((k + q) & 31)) x[tb] = xk;
+        if (nonzero(xk)) {   // uniform
+          const double v = fma(-c[q][tb], xk, x[tb]);
+          if (lane < ((k + q) & 31)) x[tb] = v;
+#pragma unroll
+          for (int t = 0; t < tb; ++t) x[t] = fma(-c[q][t], xk, x[t]);
+        }
+      }
+    }
   }
   double* Inv = inv + (size_t)blockIdx.y * n * n;
-  for (int i = lane; i < n; i += 32) Inv[(size_t)i * n + j] = x[i];
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+    if (lane + 32 * t < n) Inv[(size_t)(lane + 32 * t) * n + j] = x[t];
 }
 
 __global__ void k_gauss_jordan(int n, double* mats, double* work) {
@@ -2008,9 +2179,8 @@ p4d_status mg_plan(p4d_ctx* c) {
   }
   c->nlev = L;
   // process-wide attributes: the largest sizes the kernels use
-  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
-  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
-  P4D_TRY(cudaFuncSetAttribute(k_lu_inverse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuSmem)));
+  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuMax)));
+  P4D_TRY(cudaFuncSetAttribute(k_lu_factor<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_smem(kLuMax)));
   if (c->lev[L - 1].n > 4096) return P4D_ERR_INVALID_ARG;   // coarsest level too large for a dense inverse
   P4D_TRYS(tail_plan(c));
   double* lam = nullptr;
@@ -2237,13 +2407,9 @@ p4d_status mg_update_levels(p4d_ctx* c, const double* svar, const double* sch) {
   if (n <= kLuMax) {
     const double* dense = c->nlev == 1 ? mats : nullptr;
     const dim3 gi((n + kLuCols - 1) / kLuCols, kNH);
-    if (n <= kLuSmem) {
-      ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, lu_smem(n), c->stream>>>(n, dr, F, V, dense, work, C.perm);
-      ::p4d::count_launch(), k_lu_inverse<true><<<gi, 32 * kLuCols, lu_smem(n), c->stream>>>(n, work, C.perm, mats);
-    } else {
-      ::p4d::count_launch(), k_lu_factor<TV><<<kNH, kLuThreads, 0, c->stream>>>(n, dr, F, V, dense, work, C.perm);
-      ::p4d::count_launch(), k_lu_inverse<false><<<gi, 32 * kLuCols, 0, c->stream>>>(n, work, C.perm, mats);
-    }
+    auto k = n <= 64 ? k_lu_inverse<2> : n <= 128 ? k_lu_inverse<4> : k_lu_inverse<8>;
+    ::p4d::count_launch(), k_lu_factor<TV><<<kNH * kLuBlocks, lu_threads(n), lu_smem(n), c->stream>>>(n, dr, F, V, dense, work, C.perm);
+    ::p4d::count_launch(), k<<<gi, 32 * kLuCols, 0, c->stream>>>(n, work, C.perm, mats);
   } else {
     if (c->nlev > 1)
       ::p4d::count_launch(), k_dense<TV><<<dim3(nblocks(C.n), kNH), kBlock, 0, c->stream>>>(dims(C), F, V, sch[0], sch[1], sch[2], sch[3], mats);
