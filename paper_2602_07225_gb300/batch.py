@@ -34,7 +34,8 @@ CANDIDATES = ((1, 4.0), (2, 10.0), (3, 10.0), (3, 20.0), (4, 20.0))
 # Gauss-Seidel in every order of the fields (0 phi_s, 1 phi_e, 2 c_e)
 BJ = (0, (1, 0, 2))
 COMBOS = (BJ,) + tuple((1, o) for o in itertools.permutations((0, 1, 2)))
-# (coarse_max, mf_zchunk), the library defaults first.  No coarsest level
+# (coarse_max, mf_zchunk), the library's coarsening and its z depth for cells
+# above 60,000 nodes first (mf_zchunk = 0 picks 2 planes below).  No coarsest level
 # larger than the default's: timed on one cell a larger dense coarsest solve
 # looks free (the GPU is idle around it), but with all cells of a batch in
 # flight it doubled the time per Arnoldi step
