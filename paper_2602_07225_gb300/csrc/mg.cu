@@ -707,12 +707,13 @@ __global__ void k_dense0(Grid g, const double* __restrict__ Jst, const double* _
 // warp forms the reciprocal itself (352 clocks).  Every entry sees the same
 // operations in the same order as in the plain row-by-row elimination (a zero
 // multiplier is skipped).  One block per hierarchy, all of the trailing block
-// by it, took 111 us at 63 rows and 353 us at 120; the panel in one warp 104
-// and 267, clusters of 8 with a second block barrier per step 102 and 219;
-// this takes 94 and 214.
+// by it, took 111 us at 63 rows and 353 us at 120.  Columns per panel x blocks
+// (63 / 120 rows, us): 1 x 4 93 / 219, 1 x 8 84 / 182, 2 x 4 82 / 198, 2 x 8
+// 80 / 168, 4 x 4 90 / 210, 4 x 8 87 / 180, 8 x 4 109 / 241; 4 x 4 with the
+// panel in one warp 104 / 267.
 constexpr int kLuMax = 256;
-constexpr int kLuBlocks = 4;
-constexpr int kLuPanel = 4;
+constexpr int kLuBlocks = 8;
+constexpr int kLuPanel = 2;
 inline int lu_panels(int n) { return (n + kLuPanel - 1) / kLuPanel; }
 inline int lu_threads(int n) { return (n + 31) / 32 * 32; }
 inline size_t lu_smem(int n) {   // own columns, and three panels of multipliers
