@@ -1401,12 +1401,13 @@ __global__ void __launch_bounds__(32 * kCoarseWarps) k_coarse_solve(int n, const
 // steps and stores x into the shared memory of every block that owns a
 // neighbour row (the residual: of the blocks that own a parent row; the
 // final x: a child row), with one cluster barrier per step.  A level of at
-// most kTailThreads rows runs on the first block alone (block barriers); the
-// coarsest dense solve, FP64 and bound by the FP64 rate of an SM, is spread
-// over the cluster.  Only the x of level l0 goes back to global memory.  Per
-// row the arithmetic, its order and its contractions are those of k_cheb,
-// k_resid, k_restrict, k_prolong and k_coarse_solve: the results are
-// bit-identical to the level-by-level cycle's.
+// most kTailThreads rows runs on the first block alone (block barriers),
+// unless a coarser one takes more blocks (tail_blocks); the coarsest dense
+// solve, FP64 and bound by the FP64 rate of an SM, is spread over the
+// cluster.  Only the x of level l0 goes back to global memory.  Per row the
+// arithmetic, its order and its contractions are those of k_cheb, k_resid,
+// k_restrict, k_prolong and k_coarse_solve: the results are bit-identical to
+// the level-by-level cycle's.
 constexpr int kTailThreads = 512;
 constexpr int kTailMaxCluster = 16;
 // Rows per block before a level takes another block of the cluster: one per
@@ -1423,6 +1424,7 @@ struct TailLevel {
   Xfer1 X;                     // towards the next level
   int oA, oB, ob;              // shared offsets (elements): x buffers (at node 0, inside their guards), own b
   int lo[kNH], hi[kNH];        // row range of each hierarchy's mask
+  int nr[kNH];                 // blocks that own rows, not fewer than on a coarser level (tail_blocks)
   const void* st[kNH];
   const void* dinv[kNH];
   const uint8_t* mask[kNH];
@@ -1601,7 +1603,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const __grid_constant_
     v.X = L.X;
     v.lo = L.lo[h];
     v.rows = L.hi[h] - L.lo[h];
-    v.nr = max(1, min(a.cs, (v.rows + kTailRows<T> - 1) / kTailRows<T>));
+    v.nr = L.nr[h];
     v.chunk = (v.rows + v.nr - 1) / v.nr;
     v.oA = L.oA;
     v.oB = L.oB;
@@ -1944,6 +1946,26 @@ cudaLaunchConfig_t tail_config(int cs, int nhs, size_t smem, cudaStream_t stream
   return cfg;
 }
 
+// Blocks of the cluster that own rows, per level and hierarchy: as many as
+// the level's rows need, and at least as many as the next coarser level has.
+// A mask's row range is rounded to 256 rows and coarsening along z alone
+// halves no plane, so a coarser level can need more (a cathode at 9 x 7 nodes
+// per plane: rows 512 to 1007, on the next level 0 to 566).  A level that one
+// block owns runs without cluster barriers and without the other blocks: with
+// a shared level below it they would neither restrict into their rows nor
+// order their stores before the first block reads them.
+template <typename T>
+void tail_blocks(TailArgs& a) {
+  for (int h = 0; h < kNH; ++h) {
+    int least = 1;
+    for (int q = a.nl - 1; q >= 0; --q) {
+      TailLevel& L = a.lev[q];
+      const int need = (L.hi[h] - L.lo[h] + kTailRows<T> - 1) / kTailRows<T>;
+      least = L.nr[h] = std::max(least, std::min(a.cs, need));
+    }
+  }
+}
+
 // The levels l0 .. L - 1 in one launch (see k_tail).
 template <typename TS0, typename TS, typename T>
 p4d_status tail_launch(p4d_ctx* c, const int* hs, int nhs, int l0, const TailIO& io) {
@@ -1975,6 +1997,7 @@ p4d_status tail_launch(p4d_ctx* c, const int* hs, int nhs, int l0, const TailIO&
       B.mask[h] = A.mask[h];
     }
   }
+  tail_blocks<T>(a);
   cudaLaunchAttribute at[1];
   const cudaLaunchConfig_t cfg = tail_config(a.cs, nhs, sizeof(T) * a.len, c->stream, at);
   ::p4d::count_launch();
