@@ -398,7 +398,9 @@ __device__ void init_cycle(const Tail& t) {
   hs[L.misc + 2 * L.m + 5] = beta;
   hs[L.misc + 2 * L.m + 3] = beta;
   if (!t.gate) return;
-  // ||s.b_k|| and the tests the host makes before the first step
+  // ||s.b_k|| and the tests the host makes before the first step (fg_bnorm,
+  // fg_cycle_read): the same comparisons, so that a norm that is not a number
+  // (squares that overflow) runs the step that the host waits for
   const double* bn2 = hs + L.misc + 2 * L.m + 8;
   const double* bk2 = hs + L.misc + 2 * L.m + 16;
   double bn = 0.0;
@@ -407,7 +409,7 @@ __device__ void init_cycle(const Tail& t) {
     bn += wf * wf * bk2[f];
   }
   bn = sqrt(bn);
-  t.gate[0] = (bn > 0.0 && isfinite(beta) && beta > t.rtol * bn) ? 0.0 : 1.0;
+  t.gate[0] = bn == 0.0 || !isfinite(beta) || beta <= t.rtol * bn ? 1.0 : 0.0;
   t.gate[1] = t.gate[2] = t.gate[3] = 0.0;
   t.gate[4] = t.limit;
   t.gate[5] = bn;
