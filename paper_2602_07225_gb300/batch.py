@@ -34,22 +34,31 @@ CANDIDATES = ((1, 4.0), (2, 10.0), (3, 10.0), (3, 20.0), (4, 20.0))
 # Gauss-Seidel in every order of the fields (0 phi_s, 1 phi_e, 2 c_e)
 BJ = (0, (1, 0, 2))
 COMBOS = (BJ,) + tuple((1, o) for o in itertools.permutations((0, 1, 2)))
-# (coarse_max, mf_zchunk), the library's coarsening and its z depth for cells
-# above 60,000 nodes first (mf_zchunk = 0 picks 2 planes below).  No coarsest level
-# larger than the default's: timed on one cell a larger dense coarsest solve
-# looks free (the GPU is idle around it), but with all cells of a batch in
-# flight it doubled the time per Arnoldi step
+# (coarse_max, mf_zchunk), the library's coarsening with its z depths first:
+# mf_zchunk = 0 picks 8 planes above 60,000 nodes and 2 up to there, so both
+# are timed, and a depth that was chosen is set by its number, never by 0.  No
+# coarsest level larger than the default's: timed on one cell a larger dense
+# coarsest solve looks free (the GPU is idle around it), but with all cells of
+# a batch in flight it doubled the time per Arnoldi step.  SETUP_DEFAULT also
+# stands for the library's own options where no search ran
 SETUP_DEFAULT = (128, 8)
-SETUP_CANDIDATES = (SETUP_DEFAULT, (32, 8), (64, 8), (128, 4), (128, 16))
+SETUP_CANDIDATES = (SETUP_DEFAULT, (128, 2), (32, 8), (64, 8), (128, 4), (128, 16))
 
 
 class Autotuner:
+    """cache: (cheb_degree, cheb_ratio, combine, order) per shape, and as a
+    fifth entry (coarse_max, mf_zchunk) once these were searched.  Files with
+    six entries in a row are older: their search had no candidate at the small
+    cells' own depth, and shapes not searched carried the defaults; only the
+    first four are taken."""
+
     def __init__(self, path=None):
         self.path = path
         self.cache = {}
         if path and os.path.exists(path):
             with open(path) as fh:
-                self.cache = {tuple(json.loads(k)): tuple(v) for k, v in json.load(fh).items()}
+                self.cache = {tuple(json.loads(k)): tuple(v[:4]) if len(v) == 6 else tuple(v)
+                              for k, v in json.load(fh).items()}
 
     @staticmethod
     def key(solver, case):
@@ -104,19 +113,22 @@ class Autotuner:
         """(cheb_degree, cheb_ratio, combine, order, coarse_max, mf_zchunk);
         without build the setup options stay at the library defaults."""
         k = self.key(solver, case)
-        if k not in self.cache or (build is not None and len(self.cache[k]) < 6):
-            got = self.cache[k][:4] if k in self.cache else self.tune(solver, state, b)
+        if k not in self.cache or (build is not None and self.setup(k) is None):
+            got = self.cache[k] if k in self.cache else self.tune(solver, state, b)
             deg, ratio, combine, order = got
-            setup = SETUP_DEFAULT
             if build is not None:
-                setup = self.tune_setup(build, dict(cheb_degree=deg, cheb_ratio=ratio, combine=combine,
-                                                    order=tuple(order)))
-            self.cache[k] = tuple(got) + tuple(setup)
+                got = tuple(got) + (self.tune_setup(build, dict(cheb_degree=deg, cheb_ratio=ratio, combine=combine,
+                                                                order=tuple(order))),)
+            self.cache[k] = tuple(got)
             if self.path:
                 with open(self.path, "w") as fh:
                     json.dump({json.dumps(list(kk)): list(v) for kk, v in self.cache.items()}, fh)
+        return tuple(self.cache[k][:4]) + (self.setup(k) or SETUP_DEFAULT)
+
+    def setup(self, k):
+        """(coarse_max, mf_zchunk) found for the shape; None: not searched."""
         v = self.cache[k]
-        return tuple(v) + (tuple(SETUP_DEFAULT) if len(v) < 6 else ())
+        return tuple(v[4]) if len(v) > 4 else None
 
 
 class BatchSolver:
@@ -150,7 +162,10 @@ class BatchSolver:
                         self.tuned[k] = self.tuner.get(s, c, self.states[i], b, build=build)
                 deg, ratio, combine, order, cm, zc = self.tuned[k]
                 want = dict(coarse_max=cm, mf_zchunk=zc)
-                if (int(s.params.coarse_max), int(s.params.mf_zchunk) or SETUP_DEFAULT[1]) != (cm, zc):
+                # a searched depth is built as such; without a search the
+                # library's own (0) stands
+                own = 0 if self.tuner.setup(k) else SETUP_DEFAULT[1]
+                if (int(s.params.coarse_max), int(s.params.mf_zchunk) or own) != (cm, zc):
                     s.close()
                     s, self.states[i] = self._make(c, {**opts, **want})
                     self.solvers[i] = s
