@@ -1270,19 +1270,19 @@ __global__ void __launch_bounds__(256) k_resid(LevelDims dd, LvlPtrs<TS, T> P, H
 }
 
 
-// Full-weighting restriction (P^T r)_C over the fine nodes of the mask.
-// The phi_e / c_e masks are all ones (no mask load); elsewhere a masked-out
-// residual is selected away (never multiplied: it may hold stale values).
 // Node planes of the listed hierarchies that hold rows of their masks.
 struct PRange {
   int lo[kNH];
   int cnt[kNH];
 };
 
-// Restriction by planes: the block's coarse plane K (and with it the z
-// support) is uniform, one integer division per node is left; absent
-// support nodes of an axis get weight 0 on a node of the plane (acc + 0 r =
-// acc; the support is summed in increasing node order).
+// Full-weighting restriction (P^T r)_C over the fine nodes of the mask.
+// The phi_e / c_e masks are all ones (no mask load); elsewhere a masked-out
+// residual is selected away (never multiplied: it may hold stale values).
+// By planes: a block's coarse plane K (and with it the z support) is uniform,
+// one integer division per node is left; absent support nodes of an axis get
+// weight 0 on a node of the plane (acc + 0 r = acc; the support is summed in
+// increasing node order).
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(LevelDims fd, LevelDims cd, Xfer1 X, Ptr4<const T> fr,
                                                   Ptr4<const uint8_t> fm, Ptr4<T> cb, HList hl, PRange pr) {
@@ -1837,18 +1837,6 @@ template <> const float* cheb_tab<float>(const p4d_ctx* c) { return c->cheb_dev3
 // grid width (the widest range).  The transfer kernels take one row per
 // thread in blocks of kBlock and share these ranges.
 static_assert(kNpt == 1, "block ranges are shared by the one-row-per-thread transfer kernels");
-// Threads per block of the transfers: a multiple of 64 that wastes little of
-// the plane's last block.
-int plane_threads(const MGLevel& L) {
-  const int sxy = L.nnx * L.nny;
-  int best = 256, waste = 1 << 30;
-  for (int t = 256; t >= 128; t -= 64) {
-    const int w = (int)nblocks(sxy, t) * t - sxy;
-    if (w < waste) { waste = w; best = t; }
-  }
-  return best;
-}
-
 PRange prange(const MGLevel& A, const int* hs, int nhs, unsigned* gy) {
   PRange r{};
   int w = 1;
@@ -1861,6 +1849,30 @@ PRange prange(const MGLevel& A, const int* hs, int nhs, unsigned* gy) {
   for (int t = 0; t < nhs; ++t) w = std::max(w, r.cnt[hs[t]]);
   *gy = (unsigned)w;
   return r;
+}
+
+// Launches of the transfers over the planes of L: f(grid, block, planes).
+// Blocks of a multiple of 64 threads that wastes little of the plane's last
+// block; planes beyond a grid's y extent go in further launches.
+template <typename F>
+void for_planes(const MGLevel& L, const int* hs, int nhs, F&& f) {
+  unsigned planes = 1;
+  PRange pr = prange(L, hs, nhs, &planes);
+  const int sxy = L.nnx * L.nny;
+  dim3 block(256);
+  int waste = 1 << 30;
+  for (int t = 256; t >= 128; t -= 64) {
+    const int w = (int)nblocks(sxy, t) * t - sxy;
+    if (w < waste) { waste = w; block.x = t; }
+  }
+  const unsigned most = 65535;
+  for (unsigned y = 0; y < planes; y += most) {
+    f(dim3(nblocks(sxy, block.x), std::min(planes - y, most), nhs), block, pr);
+    for (int h = 0; h < kNH; ++h) {
+      pr.lo[h] += most;
+      pr.cnt[h] -= most;
+    }
+  }
 }
 
 BRange brange(const MGLevel& A, const int* hs, int nhs, unsigned* gx) {
@@ -2030,10 +2042,9 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs, const TailIO& io = TailI
     Ptr4<const uint8_t> fm;
     Ptr4<T> cb;
     for (int h = 0; h < kNH; ++h) { fr.p[h] = (const T*)A.r[h]; fm.p[h] = A.mask[h]; cb.p[h] = (T*)B.b[h]; }
-    unsigned gy = 1;
-    const PRange pr = prange(B, hs, nhs, &gy);
-    const int bt = plane_threads(B);
-    ::p4d::count_launch(), k_restrict<T><<<dim3(nblocks(B.nnx * B.nny, bt), gy, nhs), bt, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fr, fm, cb, hl, pr);
+    for_planes(B, hs, nhs, [&](dim3 g, dim3 b, const PRange& pr) {
+      ::p4d::count_launch(), k_restrict<T><<<g, b, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), fr, fm, cb, hl, pr);
+    });
   }
   if (c->tail_l0 >= 0) {
     P4D_TRYS((tail_launch<TS0, TS, T>(c, hs, nhs, LT, io)));
@@ -2055,10 +2066,9 @@ p4d_status vcycle_t(p4d_ctx* c, const int* hs, int nhs, const TailIO& io = TailI
     unsigned gx = 1;
     const BRange br = brange(A, hs, nhs, &gx);
     const dim3 grid(gx, nhs);
-    unsigned gy = 1;
-    const PRange pr = prange(A, hs, nhs, &gy);
-    const int bt = plane_threads(A);
-    ::p4d::count_launch(), k_prolong<T><<<dim3(nblocks(A.nnx * A.nny, bt), gy, nhs), bt, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), cxp, fm, fx, hl, pr);
+    for_planes(A, hs, nhs, [&](dim3 g, dim3 b, const PRange& pr) {
+      ::p4d::count_launch(), k_prolong<T><<<g, b, 0, c->stream>>>(dims(A), dims(B), xfer1(A, B), cxp, fm, fx, hl, pr);
+    });
     for (int s = 0; s < deg; ++s) {
       if (l == 0) prof_mark(c, 3);
       if (l == 0) P4D_TRYS((level0_stencil_step<TS0, T>(c, A, hs, nhs, hl, br, grid, 0, s)));
