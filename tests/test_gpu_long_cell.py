@@ -1,5 +1,5 @@
 """Cells of many thin node planes (the transfers between levels go plane by
-plane): more planes than a grid's y extent (65,535)."""
+plane): more planes than a grid's y extent (65,535), planes that share a block."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +22,10 @@ def _built():
 # elements (nx, ny, layers), thickness
 MESHES = {
     "66001 x 4": (1, 1, (30000, 6000, 30000), (0.4, 0.08, 0.4)),
+    "2651 x 25": (4, 4, (1300, 50, 1300), (16e-3, 6e-4, 16e-3)),  # ten planes per block, the last ones fewer
+    "1051 x 100": (9, 9, (500, 50, 500), (4e-3, 4e-4, 4e-3)),     # two
+    "142 x 126": (13, 8, (60, 21, 60), (100e-6, 25e-6, 100e-6)),
+    "142 x 128": (31, 3, (60, 21, 60), (100e-6, 25e-6, 100e-6)),  # blocks of one plane
 }
 
 
