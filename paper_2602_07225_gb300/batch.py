@@ -35,8 +35,9 @@ CANDIDATES = ((1, 4.0), (2, 10.0), (3, 10.0), (3, 20.0), (4, 20.0))
 BJ = (0, (1, 0, 2))
 COMBOS = (BJ,) + tuple((1, o) for o in itertools.permutations((0, 1, 2)))
 # (coarse_max, mf_zchunk), the library's coarsening with its z depths first:
-# mf_zchunk = 0 picks 8 planes above 60,000 nodes and 2 up to there, so both
-# are timed, and a depth that was chosen is set by its number, never by 0.  No
+# mf_zchunk = 0 picks 8 planes above 60,000 nodes and 2 up to there (long thin
+# cells 8), so both are timed, and a depth that was chosen is set by its
+# number, never by 0.  No
 # coarsest level larger than the default's: timed on one cell a larger dense
 # coarsest solve looks free (the GPU is idle around it), but with all cells of
 # a batch in flight it doubled the time per Arnoldi step.  SETUP_DEFAULT also

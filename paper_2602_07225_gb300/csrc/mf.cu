@@ -61,8 +61,15 @@ static_assert((kTX + 1) * (kTY + 1) <= kMfThreads, "one element per thread");
 // run at once, want it short, large ones the fewer repeated element planes
 // of a deep tile.  FGMRES solves at 2 / 8 planes: 25 x 25 x 25 nodes 1.67 /
 // 1.87 ms, 37 x 37 x 34 2.40 / 2.50 ms, 49 x 49 x 44 3.45 / 3.40 ms, 129 x
-// 129 x 97 18.9 / 17.2 ms (same results at every depth).
-inline int default_zchunk(int64_t nn) { return nn <= 60000 ? 2 : 8; }
+// 129 x 97 18.9 / 17.2 ms (same results at every depth).  Long thin cells
+// have many blocks of few nodes: more than 20 per SM at 2 planes (five run at
+// once) go deep too.  One application at 2 / 8 planes: 16 x 16 x 227 nodes
+// (1,368 blocks) 151 / 159 us, 5 x 5 x 2,301 (3,453) 198 / 180, 2 x 2 x 14,001
+// (21,003) 566 / 396.
+inline int default_zchunk(int64_t nn, int ntiles, int nnz) {
+  const int64_t blocks = (int64_t)3 * ntiles * ((nnz + 1) / 2);
+  return nn <= 60000 && blocks <= 20 * 152 ? 2 : 8;
+}
 
 template <typename T>
 struct MfField {
@@ -531,7 +538,7 @@ p4d_status mf_setup(p4d_ctx* c) {
   c->mf_ntx = (nnx + kTX - 1) / kTX;
   c->mf_nty = (nny + kTY - 1) / kTY;
   const int mw = nnx - (c->mf_ntx - 1) * kTX, mh = nny - (c->mf_nty - 1) * kTY;
-  const int zc = c->prm.mf_zchunk > 0 ? c->prm.mf_zchunk : default_zchunk(c->g.nn);
+  const int zc = c->prm.mf_zchunk > 0 ? c->prm.mf_zchunk : default_zchunk(c->g.nn, c->mf_ntx * c->mf_nty, nnz);
   // planes holding phi_s unknowns
   std::vector<uint8_t> lab(c->g.nn);
   P4D_TRY(cudaMemcpy(lab.data(), c->label, c->g.nn, cudaMemcpyDeviceToHost));

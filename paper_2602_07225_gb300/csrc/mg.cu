@@ -1859,7 +1859,7 @@ PRange prange(const MGLevel& A, const int* hs, int nhs, unsigned* gy) {
 // block; planes of fewer than 128 nodes share a block while every SM keeps
 // four of them; planes beyond a grid's y extent go in further launches.  One
 // application with a block of at least 128 threads per plane / now: 44,001
-// planes of 4 nodes FP64 2.13 / 1.05 ms, FP32 1.29 / 0.99; 9,001 of 25 nodes
+// planes of 4 nodes FP64 2.13 / 1.04 ms, FP32 1.29 / 0.99; 9,001 of 25 nodes
 // 0.92 / 0.76, 0.42 / 0.37; 1,101 of 64 the same.  (Ten planes of 110 nodes in
 // five blocks cost an FP64 application 2.5 us.)
 template <typename F>

@@ -46,3 +46,18 @@ def test_preconditioner_matches_oracle_algorithm(name, precision):
     # changes of the operator move them up to 80 times as much
     for sl in d.field_slices()[1:3]:
         assert np.linalg.norm(z[sl] - z_ref[sl]) < {0: 1e-11, 1: 1e-5}[precision] * np.linalg.norm(z_ref[sl])
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(1, 1, 4000), (4, 4, 2300), (15, 15, 226)])
+def test_tile_depth_of_thin_cells_leaves_the_results(nx, ny, nz):
+    """The depth picked for mf_zchunk = 0 (8 planes, 8 and 2 here) and both set by number."""
+    from paper_2602_07225_gb300 import P4DSolver
+    n = 4 * nz // 9
+    case = make_box_case(nx, ny, (n, nz - 2 * n, n), 60e-6, (3e-6 * n, 3e-6 * (nz - 2 * n), 3e-6 * n), 3, 5)
+    z = []
+    for zc in (0, 2, 8):
+        s = P4DSolver(case, precision=1, mf_zchunk=zc)
+        s.jacobian_update(s.state_tensors(case["state"]))
+        r = torch.tensor(np.random.default_rng(2).standard_normal(s.ndof), device="cuda")
+        z.append(s.precond(r))
+    assert bool(torch.isfinite(z[0]).all()) and torch.equal(z[0], z[1]) and torch.equal(z[0], z[2])
