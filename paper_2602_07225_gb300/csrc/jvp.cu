@@ -48,21 +48,62 @@ __global__ void k_jvp_combine(int64_t nn, const double* __restrict__ x, const do
 
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
+// Node n's rows of the plain product with every neighbour tested (CHECK below).
+template <bool TRANS>
+__device__ __noinline__ void tested_rows(const JvpArgs& a, const double* x, double* y, int n) {
+  const int64_t nn = a.g.nn;
+  const int N = (int)nn;
+  const double *xs = x, *xe = x + nn, *xc = x + 2 * nn;
+  const bool act = a.label[n] & kLabActive;
+  const int q = n / a.g.nnx, i = n - q * a.g.nnx, k = q / a.g.nny, j = q - k * a.g.nny;
+  double ys = 0.0, ye = 0.0, yc = 0.0;
+#pragma unroll 1
+  for (int o = 0; o < 27; ++o) {
+    const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+    if ((unsigned)(i + dx) >= (unsigned)a.g.nnx || (unsigned)(j + dy) >= (unsigned)a.g.nny ||
+        (unsigned)(k + dz) >= (unsigned)a.g.nnz)
+      continue;
+    const int m = n + dx + a.g.nnx * (dy + a.g.nny * dz);
+    const double* J = a.Jst + o * N + n;
+    if (act) ys += J[0] * xs[m];
+    ye += J[27 * nn] * (TRANS ? xe[m] : (a.u ? a.u[m] : fma(a.gdc[m], xc[m], xe[m])));
+    yc += J[2 * 27 * nn] * xc[m];
+  }
+  if (TRANS) yc += a.gdc[n] * ye;
+  if (!act) ys = xs[n];
+  const int32_t e = a.eidx[n];
+  if (e >= 0) {
+    const double t = a.tloc[e];   // left by the kernel
+    if (act) ys += (TRANS ? a.ge[e] : a.Aj[e]) * t;
+    ye -= (TRANS ? a.ge[e] : a.Aj[e]) * t;
+    if (TRANS) yc += a.gc[e] * t;
+    else yc -= a.tau * a.Aj[e] * t;
+  }
+  y[n] = ys;
+  y[nn + n] = ye;
+  y[2 * nn + n] = yc;
+}
+
 // Macro rows.  reduced: Schur operator on [phi_s | phi_e | c_e] only.
 // Large cells are bound by the FP64 rate, small ones by the latency of the
 // loads: every neighbour is loaded without a test (the stencils hold exact
 // zeros in the slots of neighbours outside the grid, the index is clamped to
 // the vector), one stencil line of three offsets at a time.
 // CHECK: an entry that is not finite must not reach a row that it does not
-// couple to (0 x Inf is NaN): a row that ends non-finite is summed again with
-// the tests.  The Krylov solves, whose vectors are finite or end the solve,
-// go without (reduced product 10.1 instead of 12.3 us on 2,025 nodes, 271
-// instead of 293 us on 129 x 129 x 97).
+// couple to (0 x Inf is NaN): a row of the plain product (b null, not scaled)
+// that ends non-finite is summed again with the tests.  After the store and
+// not inlined: inlined it held 96 registers a thread, and a product of
+// 152,439 nodes took 58.0 us, 242,406 88.3, 1,614,177 470; at 64 registers
+// (CHECK: blocks of 128 threads that an SM is to hold) 53.9, 80.8 and 449.
+// Called before the coupling or the store, small products wait for it (42,439
+// nodes 28.8 us instead of 26.8).  The Krylov solves, whose vectors are finite
+// or end the solve, go without.
 // GATED: see jvp_start.
-template <bool TRANS, bool REDUCED, bool GATED = false, bool CHECK = false>
-__global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __restrict__ x,
-                                                   const double* __restrict__ b, double* __restrict__ y,
-                                                   bool scaled) {
+template <bool TRANS, bool REDUCED, bool GATED = false, int CHECK = 0>
+__global__ void __launch_bounds__(128, CHECK) k_jvp_macro(const __grid_constant__ JvpArgs a,
+                                                          const double* __restrict__ x, const double* __restrict__ b,
+                                                          double* __restrict__ y, bool scaled) {
+  static_assert(!CHECK || (!REDUCED && !GATED), "tested_rows is the plain product");
   const int64_t nn = a.g.nn;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;   // 27 nn < 2^31 (checked at setup)
   const int N = (int)nn;
@@ -141,25 +182,10 @@ __global__ void __launch_bounds__(128) k_jvp_macro(JvpArgs a, const double* __re
     }
   };
   couple();
-  if (CHECK && !(finite_bits(ys) && finite_bits(ye) && finite_bits(yc))) {
-    const int q = n / a.g.nnx, i = n - q * a.g.nnx, k = q / a.g.nny, j = q - k * a.g.nny;
-    ys = ye = yc = 0.0;
-#pragma unroll 1
-    for (int o = 0; o < 27; ++o) {
-      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
-      if ((unsigned)(i + dx) >= (unsigned)a.g.nnx || (unsigned)(j + dy) >= (unsigned)a.g.nny ||
-          (unsigned)(k + dz) >= (unsigned)a.g.nnz)
-        continue;
-      const int m = n + dx + a.g.nnx * (dy + a.g.nny * dz);
-      if (act) ys += Ks[o * N + n] * xs[m];
-      ye += Kk[o * N + n] * (comb ? fma(a.gdc[m], xc[m], ue[m]) : ue[m]);
-      yc += Cc[o * N + n] * xc[m];
-    }
-    couple();
-  }
   y[n] = outscale(a, scaled, 0, n) * ys;
   y[nn + n] = outscale(a, scaled, 1, nn + n) * ye;
   y[2 * nn + n] = outscale(a, scaled, 2, 2 * nn + n) * yc;
+  if (CHECK && !(finite_bits(ys) && finite_bits(ye) && finite_bits(yc))) tested_rows<TRANS>(a, x, y, n);
 }
 
 // Particle rows of the full operator (after k_jvp_macro wrote tloc).
@@ -227,13 +253,18 @@ static int jvp_threads(int64_t nn) {
   return t;
 }
 
+// Macro rows of the plain product.
+static auto jvp_checked(int transpose) {
+  return transpose ? k_jvp_macro<true, false, false, 8> : k_jvp_macro<false, false, false, 8>;
+}
+
 p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled, bool u_ready) {
   JvpArgs a = make_args(c);
   const int64_t nn = c->g.nn;
   const int bt = jvp_threads(nn);
   if (!transpose) jvp_input(c, a, x, u_ready);
-  auto k = scaled ? (transpose ? k_jvp_macro<true, false> : k_jvp_macro<false, false>)
-                  : (transpose ? k_jvp_macro<true, false, false, true> : k_jvp_macro<false, false, false, true>);
+  auto k = transpose ? k_jvp_macro<true, false> : k_jvp_macro<false, false>;
+  if (!scaled && !b) k = jvp_checked(transpose);
   ::p4d::count_launch(), k<<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
   if (c->NE > 0) {
     const int64_t np = c->NE * c->nc;
@@ -344,8 +375,8 @@ extern "C" p4d_status p4d_jvp_noalloc(p4d_handle h, const double* x, double* y, 
   JvpArgs a = make_args(h);
   a.tloc = tloc;   // each entry read by the particle rows is written first by the macro rows
   const int64_t nn = h->g.nn;
-  if (transpose) ::p4d::count_launch(), k_jvp_macro<true, false, false, true><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
-  else ::p4d::count_launch(), k_jvp_macro<false, false, false, true><<<nblocks(nn, jvp_threads(nn)), jvp_threads(nn), 0, h->stream>>>(a, x, nullptr, y, false);
+  const int bt = jvp_threads(nn);
+  ::p4d::count_launch(), jvp_checked(transpose)<<<nblocks(nn, bt), bt, 0, h->stream>>>(a, x, nullptr, y, false);
   if (h->NE > 0) {
     const int64_t np = h->NE * h->nc;
     if (transpose) ::p4d::count_launch(), k_jvp_particle<true><<<nblocks(np), kBlock, 0, h->stream>>>(a, x, nullptr, y, false);
