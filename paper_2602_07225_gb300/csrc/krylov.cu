@@ -699,7 +699,9 @@ __global__ void k_surface_coupling(int64_t NE, double tau, const int32_t* __rest
 
 // Vectors up to the size of a cell whose whole V-cycle is one launch (8,192
 // nodes, three fields) are partitioned finer: their kernels are latency
-// bound.  Above it the sums keep one partition at every size.
+// bound.  Above it the dots and norms of the Arnoldi process keep one partition
+// at every size; the right-hand side's field norms do above 4 kSmallLen
+// entries (norm_blocks).
 constexpr int64_t kSmallLen = 3 * 8192;
 
 struct Reducer {
@@ -761,7 +763,10 @@ struct Reducer {
 };
 
 // Blocks of a sum over len entries: four per thread on the smallest vectors
-// (608 blocks took 13 us for 24 k entries, mostly in the last sum).
+// (608 blocks took 13 us for 24 k entries, mostly in the last sum).  Up to 4
+// kSmallLen entries (32,768 nodes of three fields, about 14,000 nodes with
+// their particles) the field norms, and with them the Krylov weights, depend
+// on this partition in their last bits.
 inline int norm_blocks(int64_t len) {
   return len <= 4 * kSmallLen ? (int)std::max<int64_t>(1, len / (4 * kRedThreads)) : kRedBlocks;
 }

@@ -1128,8 +1128,7 @@ struct LvlPtrs {
 // updates.  The kernels are bound by memory latency unless enough loads are
 // in flight; on cube128 level 0 one row per thread with plane-batched loads
 // was fastest (two rows per thread with per-offset loads came close, four or
-// more were slower from register pressure).  The block ranges of the masks
-// are shared with the one-row-per-thread transfer kernels.
+// more were slower from register pressure).
 constexpr int kNpt = 1;
 
 // ax[q] = (A x)_{n[q]} in difference form, for the rows with on[q]:
@@ -1836,10 +1835,9 @@ template <typename T> const T* cheb_tab(const p4d_ctx* c);
 template <> const double* cheb_tab<double>(const p4d_ctx* c) { return c->cheb_dev; }
 template <> const float* cheb_tab<float>(const p4d_ctx* c) { return c->cheb_dev32; }
 
-// Block ranges of a level for the listed hierarchies, and the launch's
-// grid width (the widest range).  The transfer kernels take one row per
-// thread in blocks of kBlock and share these ranges.
-static_assert(kNpt == 1, "block ranges are shared by the one-row-per-thread transfer kernels");
+// Node planes that hold a level's block ranges for the listed hierarchies (the
+// transfers go by planes), and the widest range.
+static_assert(kNpt == 1, "a block of the ranges is kBlock rows");
 PRange prange(const MGLevel& A, const int* hs, int nhs, unsigned* gy) {
   PRange r{};
   int w = 1;
@@ -1888,6 +1886,8 @@ void for_planes(const MGLevel& L, const int* hs, int nhs, F&& f) {
   }
 }
 
+// Block ranges of a level for the listed hierarchies, and the launch's grid
+// width (the widest range).
 BRange brange(const MGLevel& A, const int* hs, int nhs, unsigned* gx) {
   BRange r{};
   int w = 1;
