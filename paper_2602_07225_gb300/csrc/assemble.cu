@@ -551,8 +551,7 @@ p4d_status residual(p4d_ctx* c, const p4d_state* st, double* r) {
     ::p4d::count_launch(), k_kinetics_only<<<nblocks(NE), kBlock, 0, c->stream>>>(NE, nc, kn, c->enode, c->label, c->etype, st->phis,
                                                             st->phie, st->ce, st->cs, c->rin, c->flags);
   const double* trows = transport_residual_rows(c, st, c->lnce_r);
-  int bt = 128;   // as the Jacobian product's rows (jvp.cu)
-  while (bt > 32 && nn < (int64_t)2 * 152 * bt) bt /= 2;
+  const int bt = row_threads(nn);
   ::p4d::count_launch(), k_residual_macro<<<nblocks(nn, bt), bt, 0, c->stream>>>(c->g, kn, c->Jst, c->label, c->eidx, c->Aj, c->gpw,
                                                              st->phis, c->ue_r, st->ce, c->dce_r, c->rin, c->sfix, trows, r);
   if (NE > 0)

@@ -46,8 +46,6 @@ __global__ void k_jvp_combine(int64_t nn, const double* __restrict__ x, const do
   u[n] = fma(gdc[n], x[2 * nn + n], x[nn + n]);
 }
 
-__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
-
 // Node n's rows of the plain product with every neighbour tested (CHECK below).
 template <bool TRANS>
 __device__ __noinline__ void tested_rows(const JvpArgs& a, const double* x, double* y, int n) {
@@ -243,16 +241,6 @@ static void jvp_input(p4d_ctx* c, JvpArgs& a, const double* x, bool u_ready) {
   a.u = c->ujvp;
 }
 
-// Threads per block of the macro rows: 128, fewer while that leaves SMs
-// without a block (the rows of a block share an SM's FP64 units; the reduced
-// product of 2,025 nodes took 17 us with 128 and its own combination pass,
-// 11 us with 32, launch gaps included).
-static int jvp_threads(int64_t nn) {
-  int t = 128;
-  while (t > 32 && nn < (int64_t)2 * 152 * t) t /= 2;
-  return t;
-}
-
 // Macro rows of the plain product.
 static auto jvp_checked(int transpose) {
   return transpose ? k_jvp_macro<true, false, false, 8> : k_jvp_macro<false, false, false, 8>;
@@ -261,7 +249,7 @@ static auto jvp_checked(int transpose) {
 p4d_status jvp_full(p4d_ctx* c, const double* x, double* y, int transpose, const double* b, bool scaled, bool u_ready) {
   JvpArgs a = make_args(c);
   const int64_t nn = c->g.nn;
-  const int bt = jvp_threads(nn);
+  const int bt = row_threads(nn);
   if (!transpose) jvp_input(c, a, x, u_ready);
   auto k = transpose ? k_jvp_macro<true, false> : k_jvp_macro<false, false>;
   if (!scaled && !b) k = jvp_checked(transpose);
@@ -301,7 +289,7 @@ p4d_status jvp_start(p4d_ctx* c, const double* x, double* y, int transpose, cons
   ::p4d::count_launch(), k_nonzero<<<std::min<unsigned>(nblocks(3 * nn, 4 * kBlock), 8 * 152), kBlock, 0, c->stream>>>(x, 3 * nn, c->nzflag);
   JvpArgs a = make_args(c);
   a.nz = c->nzflag;
-  const int bt = jvp_threads(nn);
+  const int bt = row_threads(nn);
   if (!transpose) jvp_input(c, a, x, false);
   if (transpose) ::p4d::count_launch(), k_jvp_macro<true, true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, true);
   else ::p4d::count_launch(), k_jvp_macro<false, true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, true);
@@ -313,7 +301,7 @@ p4d_status jvp_reduced(p4d_ctx* c, const double* x, double* y, int transpose, co
                        bool u_ready) {
   JvpArgs a = make_args(c);
   const int64_t nn = c->g.nn;
-  const int bt = jvp_threads(nn);
+  const int bt = row_threads(nn);
   if (!transpose) jvp_input(c, a, x, u_ready);
   if (transpose) ::p4d::count_launch(), k_jvp_macro<true, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
   else ::p4d::count_launch(), k_jvp_macro<false, true><<<nblocks(nn, bt), bt, 0, c->stream>>>(a, x, b, y, scaled);
@@ -375,7 +363,7 @@ extern "C" p4d_status p4d_jvp_noalloc(p4d_handle h, const double* x, double* y, 
   JvpArgs a = make_args(h);
   a.tloc = tloc;   // each entry read by the particle rows is written first by the macro rows
   const int64_t nn = h->g.nn;
-  const int bt = jvp_threads(nn);
+  const int bt = row_threads(nn);
   ::p4d::count_launch(), jvp_checked(transpose)<<<nblocks(nn, bt), bt, 0, h->stream>>>(a, x, nullptr, y, false);
   if (h->NE > 0) {
     const int64_t np = h->NE * h->nc;

@@ -729,7 +729,6 @@ struct DenseRows {
 // Tests of doubles on their bits: a floating-point comparison is an FP64
 // instruction (20 clocks of an SM's FP64 unit per warp).
 __device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
-__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 __device__ __forceinline__ unsigned cluster_addr(const void* p, int rank) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(p);
